@@ -104,8 +104,9 @@ dptq_status dptq_pack_weights_rh(const void* W_fp16, int N, int K, int had_block
  *   bits 0-3 and code 2j+1 in bits 4-7, each 4-bit two's complement;
  *   bits == 8: int8 [M][K].
  * scales (device, written): float [M], s_a per token.
- * One fused kernel: 128-bit loads, Walsh-Hadamard butterflies on exact 64-bit fixed
- * point, one correctly rounded conversion to fp32, row absmax, rounding, packing. */
+ * One fused kernel: 128-bit loads, exact Walsh-Hadamard sums (fp32 pairs, 64-bit
+ * integers for rows whose range needs them), one correctly rounded fp32 per sum, row
+ * absmax, rounding, packing. */
 dptq_status dptq_rotate_quant_act(const void* x_fp16, int M, int K, int had_block, int bits,
                                   void* codes, float* scales, void* stream);
 

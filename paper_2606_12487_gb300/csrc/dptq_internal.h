@@ -189,9 +189,8 @@ bool l2_prefetch_allowed();
 int pre_stages_setting();
 bool decode_whole_tiles();   // DPTQ_DECODE_WHOLE_TILES=0: decode grids never shrink to one CTA per tile
 bool a8_tile128();   // DPTQ_A8_TILE128=1: A8 prefill on 128-token tiles (weights widened into shared memory)
-// The GEMM operand rows are rotated and quantized by the whole-row kernel (sums kept in
-// registers) unless DPTQ_ROWS_KERNEL=0 (the per-row kernel with an fp32 row in shared
-// memory).
+// Activation rows are rotated by the tensor-core kernel unless DPTQ_ROWS_KERNEL=0 (the
+// per-row kernel in 64-bit integers).
 bool rows_kernel_allowed();
 
 // The fixed scratch of dptq_qlinear_static on device `dev`: read its device error word

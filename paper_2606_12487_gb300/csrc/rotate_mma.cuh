@@ -1,0 +1,571 @@
+// rotate_mma.cuh -- the exact block-Hadamard rotation of rotate_row.cuh on the tensor
+// cores and the packed fp32 pipe: the same sums, scales and codes, bit for bit.
+//
+// Numbers.  Every value x of a Hadamard block of 2^l elements is split into x = hi + lo with
+// hi a multiple of 2^u and |lo| <= 2^(u - 1), u = 1 - l + k; both halves are binary16 numbers.
+// A sum of such halves with signs is exact in fp32 while it stays below 2^24 of its unit:
+//   hi: the block's sum of |x| is below 2^(24 + u) = 2^(25 - l + k)      (k is chosen so);
+//   lo: 2^l 2^(u - 1) = 2^k is at most 2^24 units of 2^(k - 24), and every x is a multiple
+//       of 2^(k - 24): always true for k = 0 (binary16 is a multiple of 2^-24), tested
+//       for k > 0.
+// So each Hadamard sum is an exact fp32 pair, and fl(hi + lo), one addition, is the
+// correctly rounded fp32 of the sum.  Rows that fail the test (a sum of |x| of 2^(25 - l) or
+// more next to values below 2^(k - 14), infinities, NaN) are rotated in 64-bit integers
+// (rotate_slow_row).
+//
+// Work split.  A warp takes a unit of 1024 consecutive elements, 32 a thread; 1, 2 or 4 warps
+// share a block (G).  Element i of a unit, bits i9..i0:
+//   * loads: lane (q = lane % 4, g = lane / 4) reads 8 consecutive halves (i2..i0) at
+//     i4 i3 = q, i5 = g0, i9 i8 = g2 g1, four times (i7 i6);
+//   * butterflies of bits 0, 1, 3, 4: one m16n8k16 MMA per half (hi, lo) and 128 elements
+//     (a 16-point transform is the 16 x 16 matrix H; the fp16 registers are its B operand
+//     as loaded), products and fp32 sums exact;
+//   * bits 2, 6, 7 across the 8 MMAs' accumulators, packed fp32 pairs; bit 5 inside a pair;
+//   * one exchange through shared memory (16 bytes = two sums' pairs, swizzled: no bank
+//     conflicts either way) after which a thread holds bits 8 .. 11 of the block and 8, 4 or
+//     2 consecutive elements (G = 1, 2, 4);
+//   * bits 8 .. 11 on (hi, lo) pairs, one packed addition per element and level.
+// Bits of l and above are left out (the MMA's matrix is the identity on them), so smaller
+// blocks take the same code.
+#pragma once
+#include <cstdint>
+#include <cuda_runtime.h>
+#include <cuda_fp16.h>
+
+#include "dptq_device.cuh"
+#include "dptq_internal.h"
+#include "rotate_row.cuh"
+
+namespace dptq {
+
+constexpr int kUnit = 1024;            // elements of one warp
+constexpr int kUnitBytes = kUnit * 8;  // its (hi, lo) pairs in the exchange
+
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ void f2_bfly(uint64_t& a, uint64_t& b) {
+  const uint64_t s = f2_add(a, b);
+  b = f2_sub(a, b);
+  a = s;
+}
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+__device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+__device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+
+// A operand of the 16-point transform for this lane: entry (row, k) is the product over
+// the bit pairs of H_2 (bits below l) or I_2 (the others).  Row bits (g0, g1, g2, reg) and k
+// bits stand for element bits 1, 3, 4, 0 and 0, 3, 4, 1.
+__device__ __forceinline__ void mma_hadamard_a(int l, int lane, uint32_t (&a)[4]) {
+  const uint32_t act = (l > 0 ? 1u : 0u) | (l > 1 ? 2u : 0u) | (l > 3 ? 4u : 0u) | (l > 4 ? 8u : 0u);
+  const uint32_t g = lane >> 2, q = lane & 3;
+  auto entry = [&](uint32_t rho, uint32_t k) -> uint32_t {   // both as bits (0, 1, 3, 4) of the element
+    if ((rho ^ k) & ~act) return 0u;
+    return (__popc(rho & k & act) & 1) ? 0xBC00u : 0x3C00u;   // -1, 1
+  };
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    // register r: row g + 8 (r & 1), k = 2 q + 8 (r >> 1) and the next
+    const uint32_t rho = (uint32_t)(r & 1) | ((g & 1) << 1) | ((g >> 1) << 2);
+    const uint32_t kk = ((uint32_t)(r >> 1) << 1) | (q << 2);
+    a[r] = entry(rho, kk) | (entry(rho, kk | 1u) << 16);
+  }
+}
+
+// 16-byte granule of the exchange that holds elements i and i + 1 (i even) of a unit.
+// Writers of a quarter warp differ in bits 1, 8, 9, readers in bits 3, 4, 5 (G = 1),
+// 2, 3, 4 (G = 2) or 1, 2, 3 (G = 4): the low three bits of the granule differ in each.
+// xch_granule(i ^ j) = xch_granule(i) ^ xch_granule(j), and its bits 3 and up are those of i / 2.
+__host__ __device__ __forceinline__ constexpr int xch_granule(int i) {
+  return (i >> 1) ^ ((i >> 4) & 1) ^ ((((i >> 8) ^ (i >> 5)) & 1) << 1) ^ (((i >> 9) & 1) << 2);
+}
+
+// The units of a row: whole blocks first, then the tail block in units of its own.
+struct UnitMap {
+  int nmain;   // units of whole blocks (a multiple of G)
+  int units;   // with the tail's
+};
+__host__ __device__ __forceinline__ UnitMap unit_map(int K, int tail, int G) {
+  const int main_len = K - tail;
+  const int nm = (main_len + kUnit * G - 1) / (kUnit * G) * G;
+  return UnitMap{nm, nm + (tail ? G : 0)};
+}
+
+// Correctly rounded fp32 of S / sqrt(2^l), S = hi + lo exactly (the value fixed_to_rotated
+// gives for the same sum).
+__device__ __forceinline__ float pair_to_rotated(float hi, float lo, int l, float c_hi, float c_lo) {
+  const float sc = __int_as_float((127 - (l >> 1)) << 23);
+  const float f = __fadd_rn(hi, lo);
+  if ((l & 1) == 0) return __fmul_rn(f, sc);
+  const float bv = __fsub_rn(f, hi);   // two-sum: rem = S - f exactly
+  const float rem = __fadd_rn(__fsub_rn(hi, __fsub_rn(f, bv)), __fsub_rn(lo, bv));
+  const float p = __fmul_rn(f, c_hi);
+  const float err = __fmaf_rn(f, c_hi, -p);
+  const float t = __fmaf_rn(f, c_lo, __fmaf_rn(rem, c_hi, err));
+  return __fmul_rn(__fadd_rn(p, t), sc);
+}
+
+// ---------------------------------------------------------------- rotation of one unit
+// The 16 halves-pairs of this lane (w[4 j + m]: elements 64 j + 2 m, 2 m + 1 of its run).
+__device__ __forceinline__ int unit_lane_offset(int lane) {
+  return (lane & 3) * 8 + ((lane >> 2) & 1) * 32 + (lane >> 3) * 256;
+}
+__device__ __forceinline__ void unit_load(const __half* row, int e0, int end, int lane, uint32_t (&w)[16]) {
+  const int o = e0 + unit_lane_offset(lane);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (o + 64 * j < end) v = __ldg(reinterpret_cast<const uint4*>(row + o + 64 * j));
+    w[4 * j] = v.x;
+    w[4 * j + 1] = v.y;
+    w[4 * j + 2] = v.z;
+    w[4 * j + 3] = v.w;
+  }
+}
+__device__ __forceinline__ void unit_signs(const int8_t* signs, int e0, int end, int lane, uint32_t (&w)[16]) {
+  const int o = e0 + unit_lane_offset(lane);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (o + 64 * j < end) {
+      const uint2 s = __ldg(reinterpret_cast<const uint2*>(signs + o + 64 * j));
+      w[4 * j] ^= __byte_perm(s.x, 0u, 0x1404) & 0x80008000u;   // bytes 0, 1 to the sign bits
+      w[4 * j + 1] ^= __byte_perm(s.x, 0u, 0x3424) & 0x80008000u;
+      w[4 * j + 2] ^= __byte_perm(s.y, 0u, 0x1404) & 0x80008000u;
+      w[4 * j + 3] ^= __byte_perm(s.y, 0u, 0x3424) & 0x80008000u;
+    }
+  }
+}
+
+// An upper bound of the unit's sum of |x| in units of 1/4, at least 2^22 when the sum is
+// not known to be below 2^20 (also for infinities and NaN).  Eight binary16 additions in a
+// row lose at most 7 2^-11 of their sum; the factor 1 + 2^-7 covers that and the fp32 steps.
+constexpr uint32_t kL1Slow = 1u << 22;
+__device__ __forceinline__ uint32_t unit_l1(const uint32_t (&w)[16]) {
+  __half2 s0 = __habs2(as_half2(w[0])), s1 = __habs2(as_half2(w[8]));
+#pragma unroll
+  for (int i = 1; i < 8; ++i) {
+    s0 = __hadd2_rn(s0, __habs2(as_half2(w[i])));
+    s1 = __hadd2_rn(s1, __habs2(as_half2(w[8 + i])));
+  }
+  const float2 a = __half22float2(s0), b = __half22float2(s1);
+  const float s = (a.x + a.y) + (b.x + b.y);
+  uint32_t v = kL1Slow;
+  if (s < 500000.f) v = (uint32_t)(int)(s * 4.04f) + 2u;   // 4 (1 + 2^-7) < 4.04
+  return __reduce_add_sync(0xffffffffu, v);
+}
+// k of the block from the sum of its units' bounds.
+__device__ __forceinline__ int split_k(uint32_t l1q, int l) {
+  const int lg = 32 - __clz(l1q - 1);   // ceil(log2): l1q >= 2
+  const int k = lg - (27 - l);
+  return k > 0 ? k : 0;
+}
+// Whether every value is a multiple of 2^(k - 24) (k >= 1).
+__device__ __forceinline__ bool unit_on_grid(const uint32_t (&w)[16], int k) {
+  const __half2 c = __half2half2(__ushort_as_half((unsigned short)((k - 14 + 15) << 10)));   // 2^(k - 14)
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const __half2 m = __hmin2(__habs2(as_half2(w[i])), c);
+    ok = ok && as_u32(__hsub2_rn(__hadd2_rn(m, c), c)) == as_u32(m);
+  }
+  return ok;
+}
+
+// Split, MMAs and the butterflies of bits 0 .. 7, then the unit's pairs into the exchange
+// (`xu`: the unit's 8192 bytes).  FULL: l >= 8, every level applies; a level under a
+// condition costs a register move for each of its additions.
+template <bool FULL>
+__device__ __forceinline__ void unit_phase1(const uint32_t (&w)[16], const uint32_t (&am)[4], int l, int k, int lane,
+                                            uint8_t* xu) {
+  // C = T = 2^(10 + u): |x| + C for |x| <= T rounds to a multiple of 2^u; larger values
+  // are multiples of 2^u already.
+  const __half2 c = __half2half2(__ushort_as_half((unsigned short)((11 - l + k + 15) << 10)));
+  uint64_t h[8][2], o[8][2];   // [instance 2 j + b2][bit 0]: pairs over bit 5
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int b2 = 0; b2 < 2; ++b2) {
+      uint32_t hi[2], lo[2];
+#pragma unroll
+      for (int b1 = 0; b1 < 2; ++b1) {
+        const uint32_t x = w[4 * j + 2 * b2 + b1];
+        const __half2 m = __hmin2(__habs2(as_half2(x)), c);
+        const __half2 r = __hsub2_rn(__hadd2_rn(m, c), c);
+        lo[b1] = as_u32(__hsub2_rn(m, r)) ^ (x & 0x80008000u);
+        hi[b1] = as_u32(__hsub2_rn(as_half2(x), as_half2(lo[b1])));
+      }
+      float dh[4], dl[4];
+      mma_16816(dh, am, hi[0], hi[1]);
+      mma_16816(dl, am, lo[0], lo[1]);
+      const int n = 2 * j + b2;
+      h[n][0] = f2_pack(dh[0], dh[1]);
+      h[n][1] = f2_pack(dh[2], dh[3]);
+      o[n][0] = f2_pack(dl[0], dl[1]);
+      o[n][1] = f2_pack(dl[2], dl[3]);
+    }
+  }
+#pragma unroll
+  for (int bit = 0; bit < 3; ++bit) {   // instance bits: element bits 2, 6, 7
+    if (FULL || l > (bit == 0 ? 2 : 5 + bit)) {
+#pragma unroll
+      for (int n = 0; n < 8; ++n)
+        if (!(n & (1 << bit))) {
+#pragma unroll
+          for (int b0 = 0; b0 < 2; ++b0) {
+            f2_bfly(h[n][b0], h[n + (1 << bit)][b0]);
+            f2_bfly(o[n][b0], o[n + (1 << bit)][b0]);
+          }
+        }
+    }
+  }
+  // bit 5 and the stores: element bits 1 = g0, 3 = g1, 4 = g2, 8 = q0, 9 = q1
+  const int g = lane >> 2, q = lane & 3;
+  const int gb = xch_granule(((g & 1) << 1) | ((g >> 1) << 3) | (q << 8));
+#pragma unroll
+  for (int n = 0; n < 8; ++n) {
+    float h00, h01, h10, h11, o00, o01, o10, o11;   // [bit 0][bit 5]
+    f2_unpack(h[n][0], h00, h01);
+    f2_unpack(h[n][1], h10, h11);
+    f2_unpack(o[n][0], o00, o01);
+    f2_unpack(o[n][1], o10, o11);
+    float4 v0, v1;   // bit 5 = 0, 1: (hi, lo) of bit 0 = 0, then of bit 0 = 1
+    if (FULL || l > 5) {
+      v0 = make_float4(h00 + h01, o00 + o01, h10 + h11, o10 + o11);
+      v1 = make_float4(h00 - h01, o00 - o01, h10 - h11, o10 - o11);
+    } else {
+      v0 = make_float4(h00, o00, h10, o10);
+      v1 = make_float4(h01, o01, h11, o11);
+    }
+    const int i = ((n & 1) << 2) | ((n >> 1) << 6);
+    // (gb ^ low) + high: gb and the constant share no bit of 8 and up
+    const int g0 = xch_granule(i), g1 = xch_granule(i | 32);
+    *reinterpret_cast<float4*>(xu + 16 * (gb ^ (g0 & 7)) + 16 * (g0 & ~7)) = v0;
+    *reinterpret_cast<float4*>(xu + 16 * (gb ^ (g1 & 7)) + 16 * (g1 & ~7)) = v1;
+  }
+}
+
+// Where a thread's 32 values sit after the exchange: 32 / R runs of R consecutive elements,
+// run c at 256 c + low of the group's 1024 G elements.
+template <int G>
+struct RunLayout {
+  static constexpr int R = G == 1 ? 8 : G == 2 ? 4 : 2;
+  static constexpr int C = 32 / R;
+  static __device__ __forceinline__ int low(int t) { return t * R; }   // t: thread of the group
+};
+
+// The exchange's reads and the butterflies of bits 8 .. 11.  v[c R + e]: (hi, lo) of element
+// 256 c + low + e of the group.  FULL: every level applies (l = 8 + log2 of the runs).
+template <int G, bool FULL>
+__device__ __forceinline__ void unit_phase2(const uint8_t* xg, int t, int l, uint64_t (&v)[32]) {
+  using RL = RunLayout<G>;
+  const int gb = xch_granule(RL::low(t));
+#pragma unroll
+  for (int c = 0; c < RL::C; ++c) {
+#pragma unroll
+    for (int e = 0; e < RL::R; e += 2) {
+      const int gc = xch_granule(256 * (c & 3) + e);
+      const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(xg + 16 * (gb ^ (gc & 7)) + (c >> 2) * kUnitBytes +
+                                                                16 * (gc & ~7));
+      v[c * RL::R + e] = p.x;
+      v[c * RL::R + e + 1] = p.y;
+    }
+  }
+#pragma unroll
+  for (int bit = 0; (1 << bit) < RL::C; ++bit) {
+    if (FULL || l > 8 + bit) {
+#pragma unroll
+      for (int x = 0; x < 32; ++x)
+        if (!(x & (RL::R << bit))) f2_bfly(v[x], v[x + (RL::R << bit)]);
+    }
+  }
+}
+
+// Largest |fl(S)| of the warp's values, as fp32 bits; `mine`: the lane's.
+__device__ __forceinline__ uint32_t warp_sum_max(const uint64_t (&v)[32], uint32_t& mine) {
+  float m0 = 0.f, m1 = 0.f;
+#pragma unroll
+  for (int e = 0; e < 32; e += 2) {
+    float h, o, h2, o2;
+    f2_unpack(v[e], h, o);
+    f2_unpack(v[e + 1], h2, o2);
+    m0 = fmaxf(m0, fabsf(__fadd_rn(h, o)));
+    m1 = fmaxf(m1, fabsf(__fadd_rn(h2, o2)));
+  }
+  mine = __float_as_uint(fmaxf(m0, m1));
+  return __reduce_max_sync(0xffffffffu, mine);
+}
+
+// Largest |y| over the values whose |fl(S)| is `wm` (odd l: 1 / sqrt 2 and the sum's own
+// remainder decide y's last bit), in lanes that hold one; 0 in the others.
+__device__ __forceinline__ float largest_rotated(const uint64_t (&v)[32], uint32_t wm, bool has, int l, float c_hi,
+                                                 float c_lo) {
+  float ym = 0.f;
+  int left = has ? 1 : 0;
+#pragma unroll 1
+  for (int it = 0; it < left; ++it) {   // the it-th such value of the lane
+    float ch = 0.f, cl = 0.f;
+    int c = 0;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      float h, o;
+      f2_unpack(v[e], h, o);
+      if ((__float_as_uint(__fadd_rn(h, o)) & 0x7FFFFFFFu) == wm) {
+        if (c == it) {
+          ch = h;
+          cl = o;
+        }
+        ++c;
+      }
+    }
+    left = c;
+    ym = fmaxf(ym, fabsf(pair_to_rotated(ch, cl, l, c_hi, c_lo)));
+  }
+  return ym;
+}
+
+// Codes of the thread's values as floats (whole numbers, no -0).  t = f r with f the fp32 of
+// the sum and r = fl(factor / s) carries at most a few units of 2^-24 against the IEEE
+// quotient of the correctly rounded y: |difference| <= |t| 2^-20.  Outside that distance from a
+// half-integer both round to the same code; inside it (rare, margin 2^-17 at |t| <= 8 and
+// 2^-13 at |t| <= 128) the quotient itself decides.  |t| never exceeds qmax (1 + 2^-22), so no
+// code needs a clamp.
+constexpr float kRoundBias = 12582912.0f;   // 1.5 * 2^23: x + bias rounds x to a whole number
+__device__ __forceinline__ void pair_codes(const uint64_t (&v)[32], int e0, int l, float s, float r, float margin,
+                                           float c_hi, float c_lo, float (&q)[8]) {
+  const uint64_t nr = f2_pack(-r, -r), bias = f2_pack(kRoundBias, kRoundBias);
+  float dm = 0.f;
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    float h0, o0, h1, o1;
+    f2_unpack(v[e0 + e], h0, o0);
+    f2_unpack(v[e0 + e + 1], h1, o1);
+    const uint64_t f = f2_pack(__fadd_rn(h0, o0), __fadd_rn(h1, o1));
+    const uint64_t qq = f2_sub(bias, f2_fma(f, nr, bias));   // rint(f r), +0 for zero
+    float d0, d1;
+    f2_unpack(f2_fma(f, nr, qq), d0, d1);                    // rint(f r) - f r
+    dm = fmaxf(dm, fmaxf(fabsf(d0), fabsf(d1)));
+    f2_unpack(qq, q[e], q[e + 1]);
+  }
+  if (__any_sync(0xffffffffu, dm > 0.5f - margin)) {
+    uint32_t near = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float h, o;
+      f2_unpack(v[e0 + e], h, o);
+      if (fabsf(__fmaf_rn(__fadd_rn(h, o), -r, q[e])) > 0.5f - margin) near |= 1u << e;
+    }
+#pragma unroll 1
+    while (near) {   // one value at a time, so that the division appears once
+      const uint32_t bit = near & (0u - near);
+      near ^= bit;
+      float ch = 0.f, cl = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        float h, o;
+        f2_unpack(v[e0 + e], h, o);
+        if (bit == (1u << e)) {
+          ch = h;
+          cl = o;
+        }
+      }
+      const float c = __fadd_rn(rintf(__fdiv_rn(pair_to_rotated(ch, cl, l, c_hi, c_lo), s)), 0.f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (bit == (1u << e)) q[e] = c;
+    }
+    __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------- writers
+// Destination of one row in mode MODE.
+struct RowOut {
+  uint8_t* p;          // row base (kRQPublic, kRQY) or the operand planes (kRQAct)
+  size_t plane;        // kRQAct, 8 bits: bytes to the second plane
+  size_t kb_stride;    // kRQAct: rows_out * 128
+  int row, bits;
+  // Address of element k, and from it to element k + 256.
+  template <int MODE>
+  __device__ __forceinline__ uint8_t* at(int k) const {
+    if constexpr (MODE == kRQAct)
+      return p + (size_t)(k >> 7) * kb_stride + (size_t)row * 128 + ((((k >> 4) & 7) ^ (row & 7)) << 4) + (k & 15);
+    else
+      return p + (MODE == kRQY ? 4 * k : bits == 4 ? k >> 1 : k);
+  }
+  template <int MODE>
+  __device__ __forceinline__ size_t step256() const {
+    return MODE == kRQAct ? 2 * kb_stride : MODE == kRQY ? 1024 : bits == 4 ? 128 : 256;
+  }
+};
+
+// R (2, 4 or 8) consecutive codes from element k on (k a multiple of R, whole numbers); `p`
+// the address of element k.
+template <int MODE, int R>
+__device__ __forceinline__ void store_codes_at(const RowOut& d, uint8_t* p, const float* q);
+template <int MODE, int R>
+__device__ __forceinline__ void store_codes(const RowOut& d, int k, const float* q) {
+  store_codes_at<MODE, R>(d, d.at<MODE>(k), q);
+}
+template <int MODE, int R>
+__device__ __forceinline__ void store_codes_at(const RowOut& d, uint8_t* p, const float* q) {
+  if constexpr (MODE == kRQAct) {
+    auto put = [&](uint8_t* at, const float* c) {
+      if constexpr (R == 2) *reinterpret_cast<uint16_t*>(at) = (uint16_t)e4m3x2(c[0], c[1]);
+      if constexpr (R == 4) *reinterpret_cast<uint32_t*>(at) = e4m3x2(c[0], c[1]) | (e4m3x2(c[2], c[3]) << 16);
+      if constexpr (R == 8)
+        *reinterpret_cast<uint2*>(at) = make_uint2(e4m3x2(c[0], c[1]) | (e4m3x2(c[2], c[3]) << 16),
+                                                   e4m3x2(c[4], c[5]) | (e4m3x2(c[6], c[7]) << 16));
+    };
+    if (d.bits == 4) {
+      put(p, q);
+    } else {
+      // c = hi + lo, hi = sign * 16 (|c| >> 4): |c| - 7.5 rounds to 16 (|c| >> 4) at a
+      // spacing of 16 (adding 1.5 * 2^27).
+      float hi[R], lo[R];
+#pragma unroll
+      for (int e = 0; e < R; ++e) {
+        const float h = __fsub_rn(__fadd_rn(__fadd_rn(fabsf(q[e]), -7.5f), 201326592.f), 201326592.f);
+        hi[e] = h == 0.f ? 0.f : copysignf(h, q[e]);
+        lo[e] = __fsub_rn(q[e], hi[e]);
+      }
+      put(p, hi);
+      put(p + d.plane, lo);
+    }
+  } else if constexpr (MODE == kRQPublic) {
+    uint32_t b[R];   // two's complement in the low bits of q + 1.5 * 2^23
+#pragma unroll
+    for (int e = 0; e < R; ++e) b[e] = __float_as_uint(__fadd_rn(q[e], kRoundBias));
+    if (d.bits == 4) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int e = 0; e < R; ++e) w |= (b[e] & 0xFu) << (4 * e);
+      if constexpr (R == 2) *p = (uint8_t)w;
+      if constexpr (R == 4) *reinterpret_cast<uint16_t*>(p) = (uint16_t)w;
+      if constexpr (R == 8) *reinterpret_cast<uint32_t*>(p) = w;
+    } else {
+      auto word = [&](int e) { return __byte_perm(__byte_perm(b[e], b[e + 1], 0x0040), __byte_perm(b[e + 2], b[e + 3], 0x0040), 0x5410); };
+      if constexpr (R == 2) *reinterpret_cast<uint16_t*>(p) = (uint16_t)__byte_perm(b[0], b[1], 0x0040);
+      if constexpr (R == 4) *reinterpret_cast<uint32_t*>(p) = word(0);
+      if constexpr (R == 8) {   // rows start 4-byte aligned at least
+        reinterpret_cast<uint32_t*>(p)[0] = word(0);
+        reinterpret_cast<uint32_t*>(p)[1] = word(4);
+      }
+    }
+  } else {   // kRQY: q holds the rotated values
+#pragma unroll
+    for (int e = 0; e < R; ++e) reinterpret_cast<float*>(p)[e] = q[e];
+  }
+}
+
+// ---------------------------------------------------------------- rows outside the pair form
+// Block-sized chunks of the CTA's share [k0, k1) of a row in 64-bit fixed point, by all its
+// threads: `ch` elements at a time through `sx` (ch + ch / 16 values), two butterfly levels per
+// pass.  visit(k, S0, S1, l) sees elements k and k + 1 of every chunk.  Small code on purpose:
+// it runs for few rows and must not cost the others registers.
+template <class Visit>
+__device__ __forceinline__ void slow_sums(const RQArgs& a, int row, int k0, int k1, int ch, long long* sx, Visit visit) {
+  const int tid = threadIdx.x, NT = blockDim.x;
+  const int tail_start = a.nfull << a.log2B;
+#pragma unroll 1
+  for (int c0 = k0; c0 < k1;) {
+    const int end = c0 < tail_start ? min(k1, tail_start) : k1;
+    const int l = c0 < tail_start ? a.log2B : a.log2T;
+    const int len = min(ch, end - c0);
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < ch; i += NT) {
+      long long f = 0;
+      if (i < len) {
+        f = half_to_fixed(__half_as_ushort(a.x[(size_t)row * a.K + c0 + i]));
+        if (a.signs != nullptr && a.signs[c0 + i] < 0) f = -f;
+      }
+      sx[pad_idx(i)] = f;
+    }
+#pragma unroll 1
+    for (int b = 0; b < l; b += 2) {
+      __syncthreads();
+      const bool two = b + 1 < l;
+#pragma unroll 1
+      for (int t = tid; t < ch >> (two ? 2 : 1); t += NT) {
+        const int i0 = ((t >> b) << (b + (two ? 2 : 1))) | (t & ((1 << b) - 1));
+        long long* p0 = sx + pad_idx(i0);
+        long long* p1 = sx + pad_idx(i0 + (1 << b));
+        const long long s = *p0 + *p1, d = *p0 - *p1;
+        if (!two) {
+          *p0 = s;
+          *p1 = d;
+        } else {
+          long long* p2 = sx + pad_idx(i0 + (2 << b));
+          long long* p3 = sx + pad_idx(i0 + (3 << b));
+          const long long s2 = *p2 + *p3, d2 = *p2 - *p3;
+          *p0 = s + s2;
+          *p1 = d + d2;
+          *p2 = s - s2;
+          *p3 = d - d2;
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = 2 * tid; i < len; i += 2 * NT) visit(c0 + i, sx[pad_idx(i)], sx[pad_idx(i + 1)], l);
+    c0 += len;
+  }
+}
+
+// The CTA's share of a row in 64-bit fixed point, twice: the row maximum (`rowmax`: this
+// thread's maximum in, the row's out), then the codes.
+template <int MODE, class RowMax>
+__device__ __forceinline__ void rotate_slow_row(const RQArgs& a, int row, int k0, int k1, int ch, uint8_t* smem,
+                                                const RowOut& dst, RowMax rowmax) {
+  long long* sx = reinterpret_cast<long long*>(smem);
+  float m = 0.f, amax = 0.f, s = 0.f;
+  const float qmaxf = (float)((1 << (a.bits - 1)) - 1), qminf = -(float)(1 << (a.bits - 1));
+#pragma unroll 1
+  for (int pass = MODE == kRQY ? 1 : 0; pass < 2; ++pass) {
+    slow_sums(a, row, k0, k1, ch, sx, [&](int k, long long S0, long long S1, int l) {
+      const float y0 = fixed_to_rotated(S0, l, a.c_hi, a.c_lo), y1 = fixed_to_rotated(S1, l, a.c_hi, a.c_lo);
+      if (pass == 0) {
+        m = fmaxf(m, fmaxf(fabsf(y0), fabsf(y1)));
+        return;
+      }
+      float q[2] = {y0, y1};
+      if (MODE != kRQY) {
+        q[0] = amax > 0.f ? __fadd_rn(fminf(fmaxf(rintf(__fdiv_rn(y0, s)), qminf), qmaxf), 0.f) : 0.f;
+        q[1] = amax > 0.f ? __fadd_rn(fminf(fmaxf(rintf(__fdiv_rn(y1, s)), qminf), qmaxf), 0.f) : 0.f;
+      }
+      store_codes<MODE, 2>(dst, k, q);
+    });
+    if (pass == 0) {
+      amax = rowmax(m);
+      s = __fdiv_rn(amax, qmaxf);
+    }
+  }
+}
+
+}  // namespace dptq

@@ -1,13 +1,16 @@
 // rotate_quant.cu -- standalone launches of the fused online block-Hadamard rotation +
-// symmetric per-row quantization whose per-row body lives in rotate_row.cuh
-// (Section 2, Eq. 4 then Eq. 2; Section 4.2): one CTA of 256 threads per row, in the
-// four writer modes, and the converter of public codes into the GEMM's E4M3 planes.
+// symmetric per-row quantization (Section 2, Eq. 4 then Eq. 2; Section 4.2): the
+// tensor-core kernel for activations (rotate_mma.cuh), the per-row kernel in 64-bit integers
+// (rotate_row.cuh; weights, Paley tails), and the converter of public codes into the
+// GEMM's E4M3 planes.
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 
 #include "dptq_device.cuh"
 #include "dptq_internal.h"
+#include "rotate_mma.cuh"
 #include "rotate_row.cuh"
 
 namespace dptq {
@@ -24,180 +27,279 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
   rotate_quant_row<MODE>(a, blockIdx.x, rq_smem, red, threadIdx.x, [] { __syncthreads(); });
 }
 
-// ---------------------------------------------------------------- whole-row kernel (GEMM operand)
-// Codes of 16 exact Hadamard sums (units of 2^-24) of one thread, without converting each
-// sum exactly.  For a value of block-size class log2n, y = S 2^-24 / sqrt(2^log2n) and the
-// oracle's code is rint(fl(y_f32 / s)), y_f32 the correctly rounded y.  Here
-// t = fl(fl(S) r) with r = fl(fl(2^-(24 + j) [/sqrt 2]) / s-ish): every factor carries at most
-// a few units of 2^-24, so |t - fl(y_f32 / s)| <= |y / s| 8 2^-24 <= |t| 2^-21 (1 + 2^-21).
-// Both round to the same integer unless t lies within m = |t| 2^-20 + 2^-30 of a
-// half-integer; only there (a warp-uniform rare branch) is y_f32 formed exactly and the
-// IEEE quotient taken.  The results are clamped to [qmin, qmax] and -0 becomes +0.
-__device__ __forceinline__ float s_to_float_approx(long long S) {
-  // S = hi 2^24 + lo with 0 <= lo < 2^24 (exact in fp32); one rounding of hi, one of the fma.
-  const int hi = (int)(S >> 24);
-  const int lo = (int)(S & 0xFFFFFFLL);
-  return __fmaf_rn((float)hi, 16777216.f, (float)lo);
-}
-
-template <int NCH>
-__global__ void __launch_bounds__(kRQThreads * NCH, NCH == 1 ? 3 : 1) rotate_quant_rows_kernel(const RQArgs a) {
-  // Group g (threads 256 g .. 256 g + 255) rotates chunk g of the row (4096 elements, whole
-  // Hadamard blocks), keeps its 16 exact sums per thread in registers through the row
-  // absmax, quantizes them directly and writes the GEMM operand planes.
-  extern __shared__ __align__(16) unsigned char rqr_smem[];
-  __shared__ float redf[kRQThreads * NCH / 32];
+// ---------------------------------------------------------------- tensor-core kernel
+// Persistent: each CTA (or cluster of CTAs, for rows of more than 16 units) takes rows
+// blockIdx.x / csize, + gridDim.x / csize, ...  A warp holds its unit's pairs in registers from
+// the exchange to the codes; the next row's loads are issued before the exchange.
+//
+// Bound by the issue of its own arithmetic (36 warp instructions per 32 elements, half of
+// the slots used: 14 to 16 warps of 128 registers an SM wait for one another once per row),
+// not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
+// 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 60.1 us; K = 4096,
+// B = 2048: 33.0 -> 20.1 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 628 us; M = 64,
+// same row: 33.8 -> 7.3 us.
+template <int MODE, int G>
+__global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
+  extern __shared__ __align__(16) uint8_t rm_smem[];
+  __shared__ uint32_t red[2][16];    // [row parity][warp]: fp32 bits of the largest |y|, or kSlow
+  __shared__ uint32_t xmax[2][8];    // the same of the cluster's CTAs
+  __shared__ uint32_t l1s[16];
+  __shared__ uint32_t lead[2];       // [row parity]: largest |y| so far, nearly (odd log2 blocks)
+  constexpr uint32_t kSlow = 0xFFFFFFFFu;
+  constexpr int kBatch = 1024;       // rows between looks at the left-over ones (32 words)
+  __shared__ uint32_t slow_rows[kBatch / 32];
   pdl_launch_dependents();
   pdl_wait();
-  const int g = threadIdx.x / kRQThreads;
-  const int tid = threadIdx.x - g * kRQThreads;
-  const int row = blockIdx.x;
-  const int K = a.K;
-  const int K_pad = a.KB * 128;
-  const int bits = a.bits;
-  const int c0 = g * kChunk;
-  const int len = c0 < K ? min(kChunk, K - c0) : 0;
-  long long* sx = reinterpret_cast<long long*>(rqr_smem + (size_t)g * kChunkPadded * 8);
-  uint8_t* stg = reinterpret_cast<uint8_t*>(sx);   // staged codes once the butterflies are done
-  uint8_t* act = static_cast<uint8_t*>(a.out);
-  const size_t plane_stride = (size_t)a.KB * a.rows_out * 128;
-  auto gsync = [g] { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(kRQThreads) : "memory"); };
-  auto store4 = [&](int k, uint32_t w0, uint32_t w1) {   // codes k .. k + 3 (k % 4 == 0)
-    const int kb = k >> 7, j = (k >> 4) & 7;
-    const size_t off = ((size_t)kb * a.rows_out + row) * 128 + ((j ^ (row & 7)) << 4) + (k & 15);
-    *reinterpret_cast<uint32_t*>(act + off) = w0;
-    if (bits == 8) *reinterpret_cast<uint32_t*>(act + plane_stride + off) = w1;
-  };
-  if (row >= a.rows_in) {   // padding row: zero codes and scale
-    for (int w = threadIdx.x; w < K_pad / 4; w += kRQThreads * NCH) store4(4 * w, 0u, 0u);
-    if (threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = 0.f;
-    return;
-  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int W = blockDim.x >> 5;
+  const int rank = csize > 1 ? (int)(blockIdx.x % csize) : 0;   // one-dimensional clusters
+  const int ncl = (int)gridDim.x / csize;
+  const int K = a.K, K_pad = a.KB * 128;
   const int tail_start = a.nfull << a.log2B;
-  long long f[16];
-  int L = 0;
-  long long mB = 0, mT = 0;
-  if (len > 0) {
-    const uint4* src = reinterpret_cast<const uint4*>(a.x + (size_t)row * K);
-    uint4 u[2];
-    rq_load16(src, c0, len, tid, u);
-    rq_fix16(a, u, c0, len, tid, f);
-    L = rq_bfly(a, c0, len, tail_start, f, sx, tid, gsync);
-    if (len == kChunk && c0 + len <= tail_start) {
-      long long m[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const long long p = f[e] < 0 ? -f[e] : f[e], q = f[e + 8] < 0 ? -f[e + 8] : f[e + 8];
-        m[e] = p > q ? p : q;
-      }
-#pragma unroll
-      for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-        for (int e = 0; e < w; ++e) m[e] = m[e] > m[e + w] ? m[e] : m[e + w];
-      mB = m[0];
-    } else {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int i = rq_pos(L, tid, e);
-        const long long v = f[e] < 0 ? -f[e] : f[e];
-        if (i < len) {
-          if (c0 + i < tail_start)
-            mB = v > mB ? v : mB;
-          else
-            mT = v > mT ? v : mT;
-        }
-      }
+  const UnitMap um = unit_map(K, a.tail, G);
+  const int wg = warp % G, tg = wg * 32 + lane;   // warp and thread within the group
+  const int Ug = rank * W + warp - wg;            // the group's first unit (whole groups are in or out)
+  const bool main_unit = Ug < um.nmain;
+  const int eg = main_unit ? Ug * kUnit : Ug < um.units ? tail_start + (Ug - um.nmain) * kUnit : K_pad;
+  const int e0 = eg + wg * kUnit;
+  const int load_end = main_unit ? tail_start : K;
+  const int store_end = main_unit && a.tail ? tail_start : MODE == kRQAct ? K_pad : K;
+  const int l = main_unit ? a.log2B : a.log2T;
+  constexpr int full_l = G == 1 ? 10 : G == 2 ? 11 : 12;
+  uint8_t* const xu = rm_smem + warp * kUnitBytes;
+  uint8_t* const xg = xu - wg * kUnitBytes;
+  auto group_sync = [&] {
+    if constexpr (G == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / G), "n"(32 * G) : "memory");
+  };
+  // Maximum over the cluster's CTAs of `v` (the same in every thread of the CTA).
+  int xpar = 0;
+  auto cluster_max = [&](uint32_t v) -> uint32_t {
+    if (csize == 1) return v;
+    if ((int)threadIdx.x < csize) {
+      const uint32_t at = smem_u32(&xmax[xpar][rank]);
+      asm volatile(
+          "{\n\t.reg .b32 r;\n\tmapa.shared::cluster.u32 r, %0, %1;\n\tst.shared::cluster.u32 [r], %2;\n\t}\n" ::"r"(at),
+          "r"(threadIdx.x), "r"(v)
+          : "memory");
     }
-  }
-  // Row absmax: the fp32 of the largest |S| of each block size (odd, monotone conversion),
-  // a warp redux on the bit patterns, then one step across the CTA's warps.
-  const float yB = mB ? fixed_to_rotated(mB, a.log2B, a.c_hi, a.c_lo) : 0.f;
-  const float yT = mT ? fixed_to_rotated(mT, a.log2T, a.c_hi, a.c_lo) : 0.f;
-  const uint32_t wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(yB, yT)));
-  if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = __uint_as_float(wmax);
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    uint32_t m = v;
+    for (int i = 0; i < csize; ++i) m = max(m, xmax[xpar][i]);
+    xpar ^= 1;
+    return m;
+  };
+  uint32_t am[4];
+  mma_hadamard_a(l, lane, am);
+  const int bits = a.bits;
+  const float qmaxf = (float)((1 << (bits - 1)) - 1);
+  const float margin = bits == 4 ? 0x1p-17f : 0x1p-13f;
+  RowOut dst;
+  dst.plane = (size_t)a.KB * a.rows_out * 128;
+  dst.kb_stride = (size_t)a.rows_out * 128;
+  dst.bits = bits;
+
+  const float p2 = __int_as_float((127 - (l >> 1)) << 23);   // 2^-(l / 2)
+  if (threadIdx.x < 2) lead[threadIdx.x] = 0u;
+  if (threadIdx.x < kBatch / 32) slow_rows[threadIdx.x] = 0u;
   __syncthreads();
-  float amax = redf[0];
-#pragma unroll
-  for (int w = 1; w < kRQThreads * NCH / 32; ++w) amax = fmaxf(amax, redf[w]);
-  const int qmax = (1 << (bits - 1)) - 1;
-  const float qmaxf = (float)qmax, qminf = (float)(-(1 << (bits - 1)));
-  const float s = __fdiv_rn(amax, qmaxf);
-  const bool nz = amax > 0.f;
-  const float rs = nz ? __frcp_rn(s) : 0.f;
-  if (threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = nz ? s : 0.f;
-  if (len > 0) {
-    // Per block size: y = S 2^-(24 + j) [x 1/sqrt 2 for odd log2]; r = that factor / s.
-    auto rfac = [&](int log2n) {
-      const float p2 = __int_as_float((127 - 24 - (log2n >> 1)) << 23);
-      return __fmul_rn((log2n & 1) ? __fmul_rn(p2, a.c_hi) : p2, rs);
-    };
-    const float rB = rfac(a.log2B), rT = rfac(a.log2T);
-    const bool uni = len == kChunk && c0 + len <= tail_start;
-#pragma unroll
-    for (int e4 = 0; e4 < 16; e4 += 4) {
-      float t[4], q[4];
-      uint32_t nearm = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int e = e4 + j;
-        const float r = (uni || c0 + rq_pos(L, tid, e) < tail_start) ? rB : rT;
-        t[j] = __fmul_rn(s_to_float_approx(f[e]), r);
-        q[j] = rintf(t[j]);
-        const float m = __fmaf_rn(fabsf(t[j]), 0x1p-20f, 0x1p-30f);
-        nearm |= (fabsf(__fsub_rn(t[j], q[j])) > 0.5f - m) ? (1u << j) : 0u;
-      }
-      if (__any_sync(0xffffffffu, nearm != 0u)) {
+
+  auto row_out = [&](int r) {
+    dst.row = r;
+    dst.p = static_cast<uint8_t*>(a.out);
+    if (MODE == kRQPublic) dst.p += (size_t)r * (bits == 4 ? K / 2 : K);
+    if (MODE == kRQY) dst.p += (size_t)r * K * 4;
+  };
+
+  // Batches of up to kBatch rows: all of them by the pairs, then the ones left over.
+  int par = 0;
 #pragma unroll 1
-        for (int j = 0; j < 4; ++j) {
-          if ((nearm >> j) & 1u) {
-            const int e = e4 + j;
-            long long v = f[0];
+  for (int row0 = (int)blockIdx.x / csize; row0 < a.rows_out; row0 += kBatch * ncl) {
+  bool any_slow = false;
+  uint32_t w[16];
+  if (row0 < a.rows_in) unit_load(a.x + (size_t)row0 * K, e0, load_end, lane, w);
+#pragma unroll 1
+  for (int it = 0; it < kBatch; ++it, par ^= 1) {
+    const int row = row0 + it * ncl;
+    if (row >= a.rows_out) break;
+    row_out(row);
+    if (row >= a.rows_in) {   // padding row (operand planes): zero codes and scale
+      if (MODE == kRQAct) {
+        const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int k = 4 * (rank * (int)blockDim.x + (int)threadIdx.x); k < K_pad; k += 4 * csize * (int)blockDim.x)
+          store_codes<kRQAct, 4>(dst, k, zero);
+        if (rank == 0 && threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = 0.f;
+      }
+      continue;
+    }
+    if (a.signs != nullptr) unit_signs(a.signs, e0, load_end, lane, w);
+    uint32_t l1 = unit_l1(w);
+    if constexpr (G > 1) {
+      if (lane == 0) l1s[warp] = l1;
+      group_sync();
+      l1 = 0;
 #pragma unroll
-            for (int ee = 1; ee < 16; ++ee)
-              if (ee == e) v = f[ee];
-            const int lg = (uni || c0 + rq_pos(L, tid, e) < tail_start) ? a.log2B : a.log2T;
-            const float qq = rintf(__fdiv_rn(fixed_to_rotated(v, lg, a.c_hi, a.c_lo), s));
-            if (j == 0) q[0] = qq;
-            if (j == 1) q[1] = qq;
-            if (j == 2) q[2] = qq;
-            if (j == 3) q[3] = qq;
-          }
+      for (int i = 0; i < G; ++i) l1 += l1s[warp - wg + i];
+    }
+    bool slow = l1 >= kL1Slow;
+    const int k = slow ? 0 : split_k(l1, l);
+    if (k > 0) slow = !__all_sync(0xffffffffu, unit_on_grid(w, k));
+    if (l >= 8)
+      unit_phase1<true>(w, am, l, k, lane, xu);
+    else
+      unit_phase1<false>(w, am, l, k, lane, xu);
+    if (it + 1 < kBatch && row + ncl < a.rows_in) unit_load(a.x + (size_t)(row + ncl) * K, e0, load_end, lane, w);
+    group_sync();
+    uint64_t v[32];
+    if (l == full_l)
+      unit_phase2<G, true>(xg, tg, l, v);
+    else
+      unit_phase2<G, false>(xg, tg, l, v);
+    uint32_t m = 0u;
+    if constexpr (MODE != kRQY) {
+      uint32_t mine;
+      const uint32_t wm = warp_sum_max(v, mine);
+      m = __float_as_uint(__fmul_rn(__uint_as_float(wm), p2));
+      if (l & 1) {
+        // 2^-j fl(S) / sqrt 2, rounded twice, is within 2 units of y: only warps that are not
+        // clearly below another form their largest y exactly.
+        m = __float_as_uint(__fmul_rn(__uint_as_float(m), a.c_hi));
+        uint32_t seen = 0u;
+        if (lane == 0) seen = atomicMax(&lead[par], m);
+        seen = __shfl_sync(0xffffffffu, seen, 0);
+        m = seen > m + 8u ? 0u
+                          : __reduce_max_sync(0xffffffffu, __float_as_uint(largest_rotated(
+                                                               v, wm, mine == wm, l, a.c_hi, a.c_lo)));
+      }
+    }
+    if (slow) m = kSlow;
+    if (lane == 0) red[par][warp] = m;
+    if (threadIdx.x == 0) lead[par ^ 1] = 0u;
+    __syncthreads();
+    m = __reduce_max_sync(0xffffffffu, lane < W ? red[par][lane] : 0u);
+    m = cluster_max(m);
+    if (m == kSlow) {   // left for the loop below
+      if (threadIdx.x == 0) slow_rows[it >> 5] |= 1u << (it & 31);
+      any_slow = true;
+      continue;
+    }
+    const float amax = __uint_as_float(m);
+    const float s = __fdiv_rn(amax, qmaxf);
+    const float rs = amax > 0.f ? __frcp_rn(s) : 0.f;
+    if (MODE != kRQY && rank == 0 && threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = s;
+    const float r = __fmul_rn((l & 1) ? __fmul_rn(p2, a.c_hi) : p2, rs);
+    using RL = RunLayout<G>;
+    const int kb = eg + RL::low(tg);
+    uint8_t* at = dst.at<MODE>(kb);
+    const size_t step = dst.step256<MODE>();
+#pragma unroll
+    for (int e = 0; e < 32; e += 8) {
+      float q[8];
+      if constexpr (MODE == kRQY) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float h, o;
+          f2_unpack(v[e + i], h, o);
+          q[i] = pair_to_rotated(h, o, l, a.c_hi, a.c_lo);
         }
+      } else {
+        pair_codes(v, e, l, s, r, margin, a.c_hi, a.c_lo, q);
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = rq_pos(L, tid, e4 + j);
-        const float c = nz ? __fadd_rn(fminf(fmaxf(q[j], qminf), qmaxf), 0.0f) : 0.f;
-        if (i < len) {
-          if (bits == 4) {
-            stg[i] = (uint8_t)(e4m3x2(c, 0.f) & 0xFFu);
-          } else {
-            const float mm = fabsf(c);
-            const float h = __fmul_rn(floorf(__fmul_rn(mm, 0.0625f)), 16.f);
-            stg[i] = (uint8_t)(e4m3x2(__fadd_rn(copysignf(h, c), 0.0f), 0.f) & 0xFFu);
-            stg[kChunk + i] = (uint8_t)(e4m3x2(__fadd_rn(copysignf(__fsub_rn(mm, h), c), 0.0f), 0.f) & 0xFFu);
-          }
-        }
+      for (int c = 0; c < 8 / RL::R; ++c) {
+        const int kk = kb + 256 * (e / RL::R + c);
+        if (kk < store_end) store_codes_at<MODE, RL::R>(dst, at, q + c * RL::R);
+        at += step;
       }
     }
   }
-  gsync();   // the group's codes are staged (sx is free: the max step synchronized the CTA)
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int i = 4 * (j * kRQThreads + tid);
-    if (i < len)
-      store4(c0 + i, *reinterpret_cast<const uint32_t*>(stg + i), *reinterpret_cast<const uint32_t*>(stg + kChunk + i));
+  if (!any_slow) continue;
+  const int u0 = rank * W, u1 = u0 + W;
+  auto first = [&](int u) { return u < um.nmain ? u * kUnit : u == um.nmain ? tail_start : K; };
+#pragma unroll 1
+  for (int it = 0; it < kBatch; ++it) {
+    const int row = row0 + it * ncl;
+    if (row >= a.rows_out) break;
+    __syncthreads();
+    if (!((slow_rows[it >> 5] >> (it & 31)) & 1u)) continue;
+    row_out(row);
+    rotate_slow_row<MODE>(a, row, min(first(u0), K), min(first(u1), K), kUnit * G, rm_smem, dst, [&](float mine) {
+      const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mine));
+      __syncthreads();
+      if (lane == 0) red[0][warp] = wm;
+      __syncthreads();
+      const float rm = __uint_as_float(cluster_max(__reduce_max_sync(0xffffffffu, lane < W ? red[0][lane] : 0u)));
+      if (MODE != kRQY && rank == 0 && threadIdx.x == 0 && a.scales != nullptr)
+        a.scales[row] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
+      return rm;
+    });
+    if (MODE == kRQAct && rank == csize - 1) {
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int kz = K + 4 * (int)threadIdx.x; kz < K_pad; kz += 4 * (int)blockDim.x) store_codes<kRQAct, 4>(dst, kz, zero);
+    }
   }
-  if (g == NCH - 1)   // k in [K, K_pad): zero codes
-    for (int k = K + 4 * tid; k < K_pad; k += 4 * kRQThreads) store4(k, 0u, 0u);
+  __syncthreads();
+  if (threadIdx.x < kBatch / 32) slow_rows[threadIdx.x] = 0u;
+  __syncthreads();
+  }
 }
 
-// Whole-row kernel for the GEMM operand when the row fits in registers (K <= 16384, one
-// group of 256 threads per 4096-element chunk); -1 when it does not apply.
-int rows_kernel_chunks(const RQArgs& a) {
-  if (a.B > kChunk || a.K > 4 * kChunk || a.tail_p > 1) return -1;
-  const int nch = (a.K + kChunk - 1) / kChunk;
-  return nch;
+// Warps that share a Hadamard block of the row.
+int rotate_group(const RQArgs& a) {
+  const int b = a.nfull > 0 ? a.B : a.tail;
+  return b <= kUnit ? 1 : b / kUnit;
+}
+
+cudaError_t device_sms(int* sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+template <int MODE, int G>
+cudaError_t launch_rotate_mma_g(const RQArgs& a, cudaStream_t s, bool pdl) {
+  const int units = unit_map(a.K, a.tail, G).units;
+  const int csize = ceil_div(units, 16);
+  const int W = round_up(ceil_div(units, csize), G);
+  // The exchange, and (rows rotated in 64-bit integers) a padded block of 1024 G values.
+  const int smem = std::max(W * kUnitBytes, G * (kUnit + kUnit / 16) * 8);
+  int sms = 0;
+  cudaError_t e = device_sms(&sms);
+  if (e == cudaSuccess) e = ensure_max_dyn_smem(rotate_mma_kernel<MODE, G>);
+  if (e != cudaSuccess) return e;
+  const int per_sm = std::max(1, 16 / W);   // 128 registers a thread: 16 warps an SM
+  const int clusters = std::max(1, std::min(a.rows_out, sms * per_sm / csize));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * csize));
+  cfg.blockDim = dim3((unsigned)(32 * W));
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (pdl && pdl_allowed()) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (csize > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)csize;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = (unsigned)n;
+  return cudaLaunchKernelEx(&cfg, rotate_mma_kernel<MODE, G>, a, csize);
+}
+
+template <int MODE>
+cudaError_t launch_rotate_mma(const RQArgs& a, cudaStream_t s, bool pdl) {
+  switch (rotate_group(a)) {
+    case 1: return launch_rotate_mma_g<MODE, 1>(a, s, pdl);
+    case 2: return launch_rotate_mma_g<MODE, 2>(a, s, pdl);
+    default: return launch_rotate_mma_g<MODE, 4>(a, s, pdl);
+  }
 }
 
 size_t rotate_quant_smem(int K, int chunk) {
@@ -207,62 +309,37 @@ size_t rotate_quant_smem(int K, int chunk) {
 }
 
 cudaError_t launch_rotate_quant(RQMode mode, const RQArgs& a, cudaStream_t s, bool pdl) {
-  const size_t smem = rotate_quant_smem(a.K, a.chunk);
+  // Activations take the tensor-core kernel; a Paley tail and the weight packer (16
+  // consecutive codes a thread) the per-row kernel.
+  if (a.tail_p == 1 && rows_kernel_allowed()) {
+    switch (mode) {
+      case kRQPublic: return launch_rotate_mma<kRQPublic>(a, s, pdl);
+      case kRQAct: return launch_rotate_mma<kRQAct>(a, s, pdl);
+      case kRQY: return launch_rotate_mma<kRQY>(a, s, pdl);
+      case kRQWeights: break;
+    }
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.rows_out);
   cfg.blockDim = dim3(kRQThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = rotate_quant_smem(a.K, a.chunk);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (pdl && pdl_allowed()) ? 1 : 0;
-  cudaError_t e = cudaSuccess;
+  auto launch = [&](void (*kernel)(const RQArgs)) {
+    const cudaError_t e = ensure_max_dyn_smem(kernel);
+    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, kernel, a);
+  };
   switch (mode) {
-    case kRQPublic:
-      e = ensure_max_dyn_smem(rotate_quant_kernel<kRQPublic>);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_kernel<kRQPublic>, a);
-      break;
-    case kRQAct: {
-      const int nch = rows_kernel_chunks(a);
-      if (nch >= 1 && rows_kernel_allowed()) {
-        cfg.blockDim = dim3(kRQThreads * nch);
-        cfg.dynamicSmemBytes = (size_t)nch * kChunkPadded * 8;
-        switch (nch) {
-          case 1:
-            e = ensure_max_dyn_smem(rotate_quant_rows_kernel<1>);
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_rows_kernel<1>, a);
-            break;
-          case 2:
-            e = ensure_max_dyn_smem(rotate_quant_rows_kernel<2>);
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_rows_kernel<2>, a);
-            break;
-          case 3:
-            e = ensure_max_dyn_smem(rotate_quant_rows_kernel<3>);
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_rows_kernel<3>, a);
-            break;
-          default:
-            e = ensure_max_dyn_smem(rotate_quant_rows_kernel<4>);
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_rows_kernel<4>, a);
-            break;
-        }
-        break;
-      }
-      e = ensure_max_dyn_smem(rotate_quant_kernel<kRQAct>);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_kernel<kRQAct>, a);
-      break;
-    }
-    case kRQY:
-      e = ensure_max_dyn_smem(rotate_quant_kernel<kRQY>);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_kernel<kRQY>, a);
-      break;
-    case kRQWeights:
-      e = ensure_max_dyn_smem(rotate_quant_kernel<kRQWeights>);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, rotate_quant_kernel<kRQWeights>, a);
-      break;
+    case kRQPublic: return launch(rotate_quant_kernel<kRQPublic>);
+    case kRQAct: return launch(rotate_quant_kernel<kRQAct>);
+    case kRQY: return launch(rotate_quant_kernel<kRQY>);
+    case kRQWeights: return launch(rotate_quant_kernel<kRQWeights>);
   }
-  return e;
+  return cudaErrorInvalidValue;
 }
 
 // ------------------------------------------------------------------ public codes -> E4M3 planes

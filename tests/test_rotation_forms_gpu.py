@@ -1,0 +1,97 @@
+"""The tensor-core rotation at the edges of its forms: units of 1024 elements, blocks over
+1, 2 and 4 warps, tails in units of their own, rows over a cluster of CTAs, and rows whose
+values leave the fp32-pair form and are rotated in 64-bit integers."""
+import numpy as np
+import pytest
+
+import parity
+from paper_2606_12487_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def dp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_12487_gb300 import dptq
+    dptq.load()
+    return dptq
+
+
+# one short unit; exactly one unit; a tail after it; a unit that holds whole blocks and
+# part of the next; two- and four-warp blocks with and without tails; 17, 20 and 28 units
+# (two CTAs a row)
+FORMS = [(32, 32), (160, 32), (1024, 1024), (1056, 1024), (2080, 64), (3072, 2048), (4096, 4096), (6144, 4096),
+         (5888, 512), (17408, 1024), (20480, 2048), (28672, 4096)]
+
+
+def rows_of_every_kind(K):
+    rng = np.random.default_rng(K)
+    n = rng.standard_normal((7, K)).astype(np.float32)
+    n[1] *= 1e-4                                   # near binary16's smallest values
+    n[2] = 40.0 * rng.integers(-100, 101, K)       # large sums on a coarse grid: pairs with k > 0
+    n[3, :3] = 60000.0                             # large sums and fine values: 64-bit integers
+    n[4] = 65504.0                                 # the largest sum
+    n[5] = 0.0
+    n[6, K // 2:] = 0.0                            # zero units
+    return inputs.to_f16(n)
+
+
+@pytest.mark.parametrize("K,B", FORMS)
+def test_forms_match_the_oracle(dp, orc, K, B):
+    x = rows_of_every_kind(K)
+    M = x.shape[0]
+    signs = np.where(np.random.default_rng(5).random(K) < 0.5, -1, 1).astype(np.int8)
+    xd, sd = torch.from_numpy(x).to(DEV), torch.from_numpy(signs).to(DEV)
+    exact = (B.bit_length() - 1) % 2 == 0 and K % B == 0   # even log2: no irrational factor
+    for sg in (None, signs):
+        y_ref = orc.rotate(x, B, sg)
+        y = torch.empty((M, K), dtype=torch.float32, device=DEV)
+        if sg is None:
+            dp.dptq_rotate_act(xd, B, y)
+        else:
+            dp.dptq_rotate_act_rh(xd, B, sd, y)
+        parity.check_rotation(y.cpu().numpy(), y_ref)
+        if exact:
+            assert np.array_equal(y.cpu().numpy(), y_ref)
+        for bits in (4, 8):
+            c_ref, s_ref = orc.rotate_quant_act(x, B, bits, sg)
+            codes = torch.empty((M, K // 2) if bits == 4 else (M, K),
+                                dtype=torch.uint8 if bits == 4 else torch.int8, device=DEV)
+            sc = torch.empty((M,), dtype=torch.float32, device=DEV)
+            if sg is None:
+                dp.dptq_rotate_quant_act(xd, B, bits, codes, sc)
+            else:
+                dp.dptq_rotate_quant_act_rh(xd, B, bits, sd, codes, sc)
+            c = codes.cpu().numpy()
+            c = orc.unpack_nibbles(c, K) if bits == 4 else c
+            parity.check_scales(sc.cpu().numpy(), s_ref)
+            n = parity.check_codes(c, c_ref, y_ref, s_ref, bits)
+            if exact:
+                assert n == 0 and np.array_equal(sc.cpu().numpy(), s_ref)
+    dp.dptq_last_device_error()
+
+
+@pytest.mark.parametrize("K,B", [(160, 32), (1056, 1024), (4096, 4096), (14336, 2048), (17408, 1024)])
+@pytest.mark.parametrize("bits", [4, 8])
+def test_operand_planes_hold_the_public_codes(dp, K, B, bits):
+    """The rotate-quantize launch of a layer (more rows than CTAs, padded token tiles) feeds
+    the GEMM the codes and scales that the public call returns."""
+    base = rows_of_every_kind(K)
+    M = 700
+    x = torch.from_numpy(base).to(DEV).repeat(M // 7, 1)
+    x[7:] *= torch.linspace(0.1, 1.0, M - 7, device=DEV)[:, None].half()
+    layer = dp.dptq_pack_weights(torch.from_numpy(inputs.weights(64, K)).to(DEV), B)
+    got = torch.empty((M, 64), dtype=torch.float16, device=DEV)
+    dp.dptq_qlinear(layer, x, bits, got)
+    codes = torch.empty((M, K // 2) if bits == 4 else (M, K), dtype=torch.uint8 if bits == 4 else torch.int8, device=DEV)
+    sc = torch.empty((M,), dtype=torch.float32, device=DEV)
+    dp.dptq_rotate_quant_act(x, B, bits, codes, sc)
+    ref = torch.empty((M, 64), dtype=torch.float16, device=DEV)
+    dp.dptq_qgemm_codes(layer, codes, sc, bits, ref)
+    assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+    dp.dptq_last_device_error()
+    layer.close()
