@@ -187,8 +187,8 @@ bool capturing(cudaStream_t s) {
 }
 
 constexpr int kMaxNT = 256;
-// Rows of up to 16384 elements take the fused launch (each of a row's four parts rotates
-// at most 4096 of them).
+// Rows of up to 16384 elements take the fused launch (at most two CTAs of 8 warps a row,
+// 1024 elements a warp).
 constexpr int kFusedMaxKPad = 16384;
 // Counter words: split-tile arrivals and grid counters, then the row-maximum slots, one
 // 128-byte line per row (only the parts of one row poll a line).
@@ -305,10 +305,7 @@ dptq_status run_gemm(dptq_handle h, const GemmPlan& plan0, const uint8_t* act, c
   g.gsync = sc->gsync;
   g.err = sc->err;
   g.wait_cycles = wait_cycles_setting();
-  if (plan.fused) {
-    g.rq_shortfall = take_rows_shortfall();
-    g.pre_stages = pre_stages_setting();
-  }
+  if (plan.fused) g.rq_shortfall = take_rows_shortfall();
   DPTQ_CUDA(launch_gemm(plan, s, true), "qgemm launch");
   return DPTQ_OK;
 }
@@ -379,18 +376,6 @@ bool a8_tile128() {
     return v && v[0] == '1';
   }();
   return on;
-}
-
-// Weight stages a fused launch requests before its token rows are ready (DPTQ_PRE_STAGES,
-// a tuning knob; default 4: of 2, 3, 4 and 6 the fastest LLaMA-2-7B decode stack at
-// M = 32).
-int pre_stages_setting() {
-  static const int v = [] {
-    const char* e = std::getenv("DPTQ_PRE_STAGES");
-    const int n = e ? std::atoi(e) : 4;
-    return n < 1 ? 1 : n;
-  }();
-  return v;
 }
 
 long long wait_cycles_setting() {
@@ -643,15 +628,18 @@ dptq_status dptq_qlinear(dptq_handle h, const void* x_fp16, int M, int bits, voi
   if (!x_fp16 || !out_fp16) return fail(DPTQ_ERR_INVALID_ARG, "null pointer");
   // Small M: one launch that rotates and quantizes the rows and runs the GEMM.
   GemmPlan fp;
+  int cpr = 0, wpc = 0;
   if (fused_allowed() && h->K_pad <= kFusedMaxKPad && pow2_tail(h->K, h->had_block) &&
-      plan_gemm(M, h->N, h->K_pad, bits, sc->num_sms, fp, kRQPartSmemBytes) && fp.M_pad == plan.M_pad &&
-      fp.M_pad <= 64 && fused_rotation_variant(h->K, h->had_block, h->K % h->had_block, fp.args.rq_np) >= 0) {
+      plan_gemm(M, h->N, h->K_pad, bits, sc->num_sms, fp, true) && fp.M_pad == plan.M_pad && fp.M_pad <= 64 &&
+      fused_rotation_split(h->K, h->had_block, h->K % h->had_block, cpr, wpc)) {
     int nfull, tail, log2B;
     if ((st = check_shape(h->K, h->had_block, nfull, tail, log2B)) != DPTQ_OK) return st;
     fp.args.rq = make_rq(x_fp16, M, fp.M_pad, h->K, h->KB, h->had_block, nfull, tail, log2B, bits, sc->sa, sc->act);
     fp.args.rq.signs = h->signs;
-    fp.args.rq.np = fp.args.rq_np;
     fp.args.rq.pmax = sc->pmax;
+    fp.args.rq_cpr = cpr;
+    fp.args.rq_wpc = wpc;
+    fp.args.rq_items = M * cpr;
     return run_gemm(h, fp, sc->act, sc->sa, out_fp16, nullptr, sc, s);
   }
   if ((st = quantize_into_scratch(h, x_fp16, M, bits, plan, sc, s)) != DPTQ_OK) return st;
@@ -756,7 +744,7 @@ dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused
   if (bits != 4 && bits != 8) return fail(DPTQ_ERR_INVALID_ARG, "bits must be 4 or 8");
   if (info == nullptr || info_len < DPTQ_PLAN_INFO_LEN) return fail(DPTQ_ERR_INVALID_ARG, "info too short");
   GemmPlan plan{};
-  if (!plan_gemm(M, N, round_up(K, kKBlock), bits, num_sms, plan, fused ? kRQPartSmemBytes : 0))
+  if (!plan_gemm(M, N, round_up(K, kKBlock), bits, num_sms, plan, fused != 0))
     return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
   const GemmArgs& g = plan.args;
   const long long sk = g.sk_iters;

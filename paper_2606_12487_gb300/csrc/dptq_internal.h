@@ -61,20 +61,15 @@ struct RQArgs {
   int tail_j;
   float t_hi, t_lo;
   int bits;          // 4 or 8
-  // Fused decode launch: parts per row and the row-maximum slots, kRowMaxStride words
-  // per row of which the first np are used (1 + the bits of each part's largest |y|;
-  // 0 = not yet written; zero between launches).
-  int np;
+  // Fused decode launch: the row-maximum slots of rows shared by two CTAs, kRowMaxStride
+  // words per row (1 + the bits of each CTA's largest |y| in words 0 and 1, of rows in 64-bit
+  // integers in words 4 and 5; 0 = not yet written; zero between launches).
   uint32_t* pmax;
   float* scales;     // [rows_out] (rows >= rows_in get 0); may be null in kRQY
   void* out;         // mode-dependent destination
 };
 
 cudaError_t launch_rotate_quant(RQMode mode, const RQArgs& a, cudaStream_t s, bool pdl);
-// Shared memory of one row part in the fused decode launch: the padded int64 transpose
-// chunk (4096 + 256 values), two planes of staged codes (4096 bytes each) and 16 warp
-// maxima.
-constexpr int kRQPartSmemBytes = (4096 + 256) * 8 + 2 * 4096 + 16 * 8;
 size_t rotate_quant_smem(int K, int chunk);
 // Shared-memory budget of one CTA (227 KB opt-in).
 constexpr size_t kSmemPerBlock = 232448;
@@ -134,18 +129,15 @@ struct GemmArgs {
   uint32_t tmem_cols;
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
   long long l2_prefetch;  // weight bytes past the first ring stages each CTA requests into L2 up front (0: none)
-  // Fused launch: weight stages the producer requests before the token rows are ready
-  // (set from pre_stages_setting());
-  // the rest of the ring and the L2 prefetch wait for the rows (while the rows are
-  // rotated, the parts' exchanges of their maxima cross the memory system, and a full
-  // ring fill in flight delays them by microseconds).
-  int pre_stages;
   // Fused decode launches only: the rotation + quantization of the M_pad token rows
-  // (written to `act` / `sa` by the converter warps of CTAs 0, 1, ...) and the two grid
-  // counters [rows ready, CTAs done] that order it before the GEMM (zero between launches).
+  // (written to `act` / `sa` by the converter warps of CTAs 0, 1, ...: CTA row * rq_cpr +
+  // part) and the two grid counters [rows ready, CTAs done] that order it before the GEMM
+  // (zero between launches).
   RQArgs rq;
-  int rq_np;           // parts per token row (1, 2 or 4): work item = row * rq_np + part
-  int rq_items;        // M_pad * rq_np: the value the rows-ready counter reaches
+  int rq_np;           // CTAs the grid holds per token row (2 or 4)
+  int rq_cpr;          // CTAs that share a row's rotation (1 or 2)
+  int rq_wpc;          // units of 1024 elements (warps) of a row in each of them, at most 8
+  int rq_items;        // M * rq_cpr: the value the rows-ready counter reaches
   int rq_shortfall;    // test hook: extra items the activation producer waits for (0)
   uint32_t* gsync;
   long long wait_cycles;   // bound of every pipeline wait (SM cycles) before the kernel gives up
@@ -164,12 +156,15 @@ struct GemmPlan {
 
 // Fills everything in `plan.args` that depends only on shapes; the caller sets the
 // pointers.  Returns false if the shape cannot be run.
-// `rot_smem` > 0 plans the fused decode kernel: that many extra bytes of shared memory
-// for the rotation of one row, two k-blocks per stage; false if it does not fit.
-bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, int rot_smem = 0);
-// Row split of the fused launch for K, B, the (power-of-two) tail and np parts per row:
-// kPartBlocks, kPartSlice4 or kPartSlice8 (rotate_row.cuh), or -1 when none applies.
-int fused_rotation_variant(int K, int B, int tail, int np);
+// `fused` plans the decode kernel that rotates and quantizes the rows itself: two k-blocks
+// per stage; false if it does not fit.
+bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused = false);
+// Warps that share a Hadamard block of a row in the tensor-core rotation (1, 2 or 4; K, B and
+// a power-of-two tail).
+int rotate_group(int K, int B, int tail);
+// How a fused launch splits a row: CTAs per row and units in each.  False for rows of more
+// than 16 units.
+bool fused_rotation_split(int K, int B, int tail, int& cpr, int& wpc);
 cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl);
 
 // Programmatic dependent launch is on unless the environment sets DPTQ_PDL=0 (kernels
@@ -186,7 +181,6 @@ long long wait_cycles_setting();
 int take_rows_shortfall();
 // Decode GEMM launches prefetch their weight share into L2 unless DPTQ_L2PF=0.
 bool l2_prefetch_allowed();
-int pre_stages_setting();
 bool decode_whole_tiles();   // DPTQ_DECODE_WHOLE_TILES=0: decode grids never shrink to one CTA per tile
 bool a8_tile128();   // DPTQ_A8_TILE128=1: A8 prefill on 128-token tiles (weights widened into shared memory)
 // Activation rows are rotated by the tensor-core kernel unless DPTQ_ROWS_KERNEL=0 (the

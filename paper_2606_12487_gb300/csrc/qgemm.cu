@@ -41,6 +41,7 @@
 
 #include "dptq_device.cuh"
 #include "dptq_internal.h"
+#include "rotate_mma.cuh"
 #include "rotate_row.cuh"
 
 namespace dptq {
@@ -169,18 +170,17 @@ struct Smem {
   __device__ __forceinline__ uint8_t* end(int S) const { return slot(S); }
 };
 
-// RQV != 0 (decode, two-block stages) makes the launch FUSED: it first rotates and
-// quantizes the token rows itself.  Each row is split into rq_np parts, each part
-// rotating only its own outputs (RQV = kPartBlocks: whole blocks per part;
-// kPartSlice4 / kPartSlice8: slices of one block, 4 or 8 values per thread); the parts
-// of a row exchange their maxima through global slots, and the converter warps publish
-// the rows on a grid counter.  Every producer streams its first weight stages meanwhile
-// and requests activation tiles once all rows are in; the epilogue reads the token
-// scales after the same point, and the last CTA to get there resets the counters and
-// the slots.
-template <int NT, int KPS, int RQV>
+// RG != 0 (decode, two-block stages) makes the launch FUSED: it first rotates and quantizes
+// the token rows itself (RG = 1, 2 or 4 warps per Hadamard block, rotate_mma.cuh).  CTA
+// row * rq_cpr + part takes a row, or half of one of more than 8 units, with its 8 converter
+// warps, in the shared memory of the copy ring, which this CTA fills only afterwards; its
+// weight share is requested into L2 meanwhile.  The other CTAs fill their rings from the
+// start.  The rows are published on a grid counter; every activation producer waits for all
+// of them; the epilogue reads the token scales after the same point, and the last CTA to get
+// there resets the counters and the slots.
+template <int NT, int KPS, int RG>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a) {
-  constexpr bool FUSED = RQV != 0;
+  constexpr bool FUSED = RG != 0;
   // Two-block stages (token tiles of up to 64, weight streaming) and 192-token tiles
   // widen the weights straight into tensor memory and feed the MMA's A operand from
   // there; other one-block stages widen into shared memory.
@@ -204,12 +204,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   uint64_t* drain = tempty + 2;
   uint64_t* esync = drain + 1;   // epilogue-group barrier (4 warps), bounded waits
   uint64_t* aready = esync + 1;  // fused: all token rows are quantized (producer -> epilogue)
-  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(aready + 1);
+  uint64_t* rdone = aready + 1;  // fused: this CTA's row is quantized, the ring's memory is free
+  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(rdone + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_sh + 1);
   volatile int* flags = reinterpret_cast<volatile int*>(tmem_base_sh + 2);   // epilogue: 2 units x 2
   float* sa_sh = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);   // token scales (NT <= 64)
   __half* xpose = reinterpret_cast<__half*>(reinterpret_cast<uint8_t*>(bars) + 1024);  // 4 x [4 tokens][32 ch]
-  unsigned char* rot_smem = reinterpret_cast<unsigned char*>(bars) + kBarrierBytes;    // fused: one row's scratch
+  uint32_t* rot_sh = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + 768);   // fused: 32 words
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -233,6 +234,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     mbar_init(drain, 1);
     mbar_init(esync, kNumEpiWarps);
     mbar_init(aready, 1);
+    mbar_init(rdone, 1);
+    if (FUSED) rot_sh[16] = 0u;
     *abort_flag = 0;
     for (int i = 0; i < 4; ++i) flags[i] = 0;
     fence_mbar_init();
@@ -277,12 +280,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     // previous kernel finishes).  Units are visited in processing order; each unit's
     // weight range is contiguous (tile-major, k-blocks consecutive) and, with one token
     // tile, belongs to this CTA.
-    auto prefetch_share = [&]() {
+    auto prefetch_share = [&](long long skip) {   // skip: bytes fetched by the ring directly
       if (!(wprod && leader && a.l2_prefetch > 0)) return;
       UnitIter pit;
       pit.init(a);
       Unit pu;
-      long long skip = (long long)S * w_bytes;   // fetched by the ring directly
       long long budget = a.l2_prefetch;
       while (budget > 0 && pit.next(pu)) {
         const int tile_n = pu.tile / a.m_tiles;
@@ -304,7 +306,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     // The activation producer starts once the previous kernel has finished and, in a fused
     // launch, every token row has been quantized.
     bool ok = true;
-    if (!wprod) {
+    const bool rotates = FUSED && (int)blockIdx.x < a.rq_items;
+    if (rotates) {   // the ring's memory holds the row until it is quantized
+      prefetch_share(0);
+      __syncwarp();
+      ok = mbar_wait_warp(rdone, 0, abort_flag, a.err, kDevTimeoutGrid, a.wait_cycles);
+    }
+    if (!wprod && ok) {
       pdl_wait();
       if constexpr (FUSED) {
         const long long t0 = clock64();
@@ -350,11 +358,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         const int s = rg.s;
         const bool tg = kTraceStages > 10 && wprod && leader && g >= 8 && g < 11;   // clocked stages (trace builds)
         (void)tg;
-        if (FUSED && wprod && g == a.pre_stages &&
-            !mbar_wait_warp(aready, 0, abort_flag, a.err, kDevTimeoutGrid, a.wait_cycles)) {
-          ok = false;   // the rows never became ready
-          break;
-        }
         if (tg) DPTQ_TRACE_CLOCK(tr, 224 + 3 * (g - 8));
         if (!mbar_wait_warp(&empty[s], rg.ph ^ 1u, abort_flag, a.err, kDevTimeoutEmpty, a.wait_cycles)) {
           ok = false;
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
             if (DPTQ_CHECK(nt < a.n_wtiles && (it + 1) * KPS <= a.KB, a.err, 1))
               bulk_g2s(sm.wpack(s), wsrc, w_bytes, &full[s], pol_w);
             if (g < kTraceStages) DPTQ_TRACE_POINT(tr, 24 + g);
-            if (g == S - 1) prefetch_share();
+            if (g == S - 1 && !rotates) prefetch_share((long long)S * w_bytes);
           } else {
             mbar_arrive_expect_tx(&afull[s], a_tx);
             // debug builds: the stage's token tile lies inside the operand planes (site 2)
@@ -503,38 +506,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     // ------------------------------------------------------------ converters
     const int ctid = threadIdx.x - kConvWarp0 * 32;   // 0..255
     if constexpr (FUSED) {
-      // Rotate + quantize this CTA's (row, part) items into the activation planes and
-      // scales, then publish them.  The 8 converter warps meet at named barrier 1.
+      // Rotate + quantize this CTA's row (or its part of it) into the activation planes and
+      // scales, then publish it.  The 8 converter warps meet at named barrier 1.
       pdl_wait();   // the rows come from the previous kernel
-      if (ctid == 0) {
-        DPTQ_TRACE_POINT(tr, 125);
-        DPTQ_TRACE_CLOCK(tr, 160);
-      }
-      const auto csync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kConvThreads) : "memory"); };
-      // Rows go out in rounds of G / np rows, CTA c taking part c % np of rows
-      // c / np, c / np + G / np, ...: the parts of a row, which wait for one another's
-      // maxima, always run in the same round.
-      const int np = a.rq.np;
-      const int rpr = (int)gridDim.x / np;
-      int nitems = 0;
-      if ((int)blockIdx.x < rpr * np) {
-        const int part = (int)blockIdx.x % np;
-        for (int row = (int)blockIdx.x / np; row < a.rq.rows_out; row += rpr) {
-          if (nitems) csync();   // the previous row's readers are done with the scratch
-          if constexpr (RQV == kPartBlocks)
-            rotate_quant_part_blocks(a.rq, row, part, rot_smem, ctid, csync, a.wait_cycles, a.err);
-          else
-            rotate_quant_part_slice<RQV>(a.rq, row, part, rot_smem, ctid, csync, a.wait_cycles, a.err);
-          ++nitems;
+      if (ctid == 0) DPTQ_TRACE_POINT(tr, 125);
+      if ((int)blockIdx.x < a.rq_items) {
+        const auto csync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kConvThreads) : "memory"); };
+        fused_rotate_row<RG>(a.rq, (int)blockIdx.x / a.rq_cpr, (int)blockIdx.x % a.rq_cpr, a.rq_cpr, a.rq_wpc, smem,
+                             rot_sh, warp - kConvWarp0, lane, csync, a.wait_cycles, a.err);
+        if (ctid == 0) DPTQ_TRACE_POINT(tr, 126);
+        fence_proxy_async_smem();   // the ring's copies overwrite what was read and written here
+        csync();                    // every converter thread's code and scale stores precede the release
+        if (ctid == 0) {
+          release_add_gpu(a.gsync, 1u);
+          mbar_arrive(rdone);
         }
-      }
-      if (ctid == 0) {
-        DPTQ_TRACE_POINT(tr, 126);
-        DPTQ_TRACE_CLOCK(tr, 161);
-      }
-      if (nitems) {
-        csync();   // every converter thread's code and scale stores precede the release
-        if (ctid == 0) release_add_gpu(a.gsync, (uint32_t)nitems);
       }
       if (ctid == 0) DPTQ_TRACE_POINT(tr, 127);
     }
@@ -691,8 +677,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         if (prev == gridDim.x - 1) {   // every part has also read its row's maxima
           a.gsync[0] = 0u;
           a.gsync[1] = 0u;
-          for (int r = 0; r < a.rq.rows_out; ++r)
-            *reinterpret_cast<uint4*>(a.rq.pmax + kRowMaxStride * r) = make_uint4(0u, 0u, 0u, 0u);
+          if (a.rq_cpr > 1)
+            for (int r = 0; r < a.rq.rows_in; ++r) {
+              uint4* line = reinterpret_cast<uint4*>(a.rq.pmax + kRowMaxStride * r);
+              line[0] = line[1] = make_uint4(0u, 0u, 0u, 0u);
+            }
         }
       }
     }
@@ -1008,7 +997,7 @@ static int smem_for(int nt, int kps, int stages, int planes, int conv_slots) {
   return 1024 + conv_slots * kps * kConvBytes + stages * kps * (planes * nt * 128 + kWTileBytes) + kBarrierBytes;
 }
 
-bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, int rot_smem) {
+bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused) {
   GemmArgs& a = plan.args;
   const int KB = K_pad / kKBlock;
   const int planes = bits == 8 ? 2 : 1;
@@ -1049,14 +1038,14 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, i
   else   // room for two accumulators next to the slots
     while (conv_slots > 2 && 2 * nt * segs + conv_slots * kps * 32 > 512) --conv_slots;
   const int smem_conv = a_tmem ? 0 : conv_slots;
-  // A fused launch needs two-block stages (weights widened into TMEM) and room for one
-  // row's rotation scratch next to at least 3 stages.
-  const bool fused = rot_smem > 0;
-  if (fused && kps != 2) return false;
-  auto smem_total = [&](int st) { return smem_for(nt, kps, st, planes, smem_conv) + (fused ? rot_smem : 0); };
+  // A fused launch needs two-block stages (weights widened into TMEM) and a ring that holds
+  // the eight units of a row's rotation.
+  if (fused && (kps != 2 || nt > 64)) return false;
+  auto smem_total = [&](int st) { return smem_for(nt, kps, st, planes, smem_conv); };
   int stages = kMaxStages;
   while (stages > 2 && smem_total(stages) > kSmemLimit) --stages;
-  if (smem_total(stages) > kSmemLimit || (fused && stages < 3)) return false;
+  if (smem_total(stages) > kSmemLimit) return false;
+  if (fused && stages * kps * (planes * nt * 128 + kWTileBytes) < 8 * kUnitBytes) return false;
   // The converters learn that a widened slot is free from the `empty` barrier of the
   // stage that last read it, CS stages back; with CS <= stages that barrier cannot
   // complete a further phase before they look.
@@ -1082,9 +1071,8 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, i
     // extra round trip at the end of the launch; measured on GB300 that outweighs a
     // longer stream per CTA.  So: whole tiles, one per CTA, when they fit on the SMs and a
     // tile is at most twice a CTA's fair share of the stages; otherwise stream-K with at
-    // most four CTAs per tile.  A fused launch keeps whole tiles only while they leave a
-    // CTA for each of four parts of every token row: with fewer, its rows would be split
-    // in two (slower rotation, measured: LLaMA-2-7B q|k|v at M = 32 is faster on all SMs).
+    // most four CTAs per tile.  A fused launch keeps whole tiles only while they leave four
+    // CTAs for every token row.
     const bool rows_fit = !fused || (long long)M_pad * 4 <= tiles;
     if (decode_whole_tiles() && rows_fit && tiles <= num_sms && (long long)KI * num_sms <= 2 * iters)
       G = (int)tiles;
@@ -1127,11 +1115,10 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, i
   a.l2_prefetch = (nt <= 64 && m_tiles == 1 && l2_prefetch_allowed()) ? 512LL * 1024 : 0;
   a.rq = RQArgs{};
   a.gsync = nullptr;
-  // Fused: every token row is split into 4 parts (each rotates and quantizes its share
-  // of the row) when each part gets a CTA of its own; else into 2 parts with a CTA each,
-  // for rows of at most 8192 elements (at most 4096 per part); else into 4 parts in two
-  // rounds of rows.  A launch whose grid is smaller than that leaves the rows to the
-  // separate rotate-quantize launch (no fused plan).
+  // Fused: the grid holds four CTAs per token row (padding included), or two; a launch whose
+  // grid is smaller leaves the rows to the separate rotate-quantize launch (no fused plan).
+  // A row's rotation takes one of them, or two (rows of more than 8 units), so that most
+  // CTAs only stream weights meanwhile and no CTA takes a second row.
   int np = 1;
   if (fused) {
     if ((long long)M_pad * 4 <= G)
@@ -1144,32 +1131,25 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, i
       return false;
   }
   a.rq_np = np;
-  a.rq_items = fused ? M_pad * np : 0;
+  a.rq_cpr = 0;
+  a.rq_wpc = 0;
+  a.rq_items = 0;
   a.rq_shortfall = 0;
-  a.pre_stages = 2;
   a.wait_cycles = kWaitTimeoutCycles;
   return true;
 }
 
-// How the fused launch splits a row over its np parts (two or four): slices of one
-// block when the row has fewer blocks than parts (K a multiple of B, n = np B / K >= 2
-// parts per block, slices of 1024 or 2048 elements), else whole blocks (every part at
-// most 4096 elements: K <= 4096 np).  -1: neither applies.
-int fused_rotation_variant(int K, int B, int tail, int np) {
-  if (np != 2 && np != 4) return -1;
-  if (tail == 0 && K % B == 0 && (np * B) % K == 0) {
-    const int n = np * B / K;
-    if (n >= 2 && B / n == 1024) return kPartSlice4;
-    if (n >= 2 && B / n == 2048) return kPartSlice8;
-  }
-  const int gr = B > 128 ? B : 128;
-  const int ng = (K + gr - 1) / gr;
-  return (ng + np - 1) / np * gr <= 4096 ? kPartBlocks : -1;
+bool fused_rotation_split(int K, int B, int tail, int& cpr, int& wpc) {
+  const int G = rotate_group(K, B, tail);
+  const int units = unit_map(K, tail, G).units;
+  cpr = ceil_div(units, kNumConvWarps);
+  wpc = round_up(ceil_div(units, cpr), G);
+  return cpr <= 2 && wpc <= kNumConvWarps;
 }
 
-template <int NT, int KPS, int RQV = 0>
+template <int NT, int KPS, int RG = 0>
 static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
-  cudaError_t e = ensure_max_dyn_smem(qgemm_kernel<NT, KPS, RQV>);
+  cudaError_t e = ensure_max_dyn_smem(qgemm_kernel<NT, KPS, RG>);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)plan.grid);
@@ -1181,18 +1161,19 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (pdl && pdl_allowed()) ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RQV>, plan.args);
+  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RG>, plan.args);
 }
 
 cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
   if (plan.fused) {
-    const int v = fused_rotation_variant(plan.args.rq.K, plan.args.rq.B, plan.args.rq.tail, plan.args.rq_np);
-    if (v < 0 || plan.args.rq.np != plan.args.rq_np) return cudaErrorInvalidValue;
-#define DPTQ_FUSED_NT(nt)                                                      \
-  case nt:                                                                     \
-    return v == kPartSlice4   ? launch_nt<nt, 2, kPartSlice4>(plan, s, pdl)    \
-           : v == kPartSlice8 ? launch_nt<nt, 2, kPartSlice8>(plan, s, pdl)    \
-                              : launch_nt<nt, 2, kPartBlocks>(plan, s, pdl);
+    const GemmArgs& g = plan.args;
+    if (g.rq_cpr < 1 || g.rq_items > plan.grid) return cudaErrorInvalidValue;
+    const int rg = rotate_group(g.rq.K, g.rq.B, g.rq.tail);
+#define DPTQ_FUSED_NT(nt)                                       \
+  case nt:                                                      \
+    return rg == 1   ? launch_nt<nt, 2, 1>(plan, s, pdl)        \
+           : rg == 2 ? launch_nt<nt, 2, 2>(plan, s, pdl)        \
+                     : launch_nt<nt, 2, 4>(plan, s, pdl);
     switch (plan.nt) {
       DPTQ_FUSED_NT(16)
       DPTQ_FUSED_NT(32)

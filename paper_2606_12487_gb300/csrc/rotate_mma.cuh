@@ -40,6 +40,7 @@ namespace dptq {
 
 constexpr int kUnit = 1024;            // elements of one warp
 constexpr int kUnitBytes = kUnit * 8;  // its (hi, lo) pairs in the exchange
+constexpr uint32_t kRowSlow = 0x7FFFFFFFu;   // in place of a maximum: the row leaves the pair form
 
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
   uint64_t r;
@@ -484,20 +485,20 @@ __device__ __forceinline__ void store_codes_at(const RowOut& d, uint8_t* p, cons
 }
 
 // ---------------------------------------------------------------- rows outside the pair form
-// Block-sized chunks of the CTA's share [k0, k1) of a row in 64-bit fixed point, by all its
-// threads: `ch` elements at a time through `sx` (ch + ch / 16 values), two butterfly levels per
-// pass.  visit(k, S0, S1, l) sees elements k and k + 1 of every chunk.  Small code on purpose:
-// it runs for few rows and must not cost the others registers.
-template <class Visit>
-__device__ __forceinline__ void slow_sums(const RQArgs& a, int row, int k0, int k1, int ch, long long* sx, Visit visit) {
-  const int tid = threadIdx.x, NT = blockDim.x;
+// Block-sized chunks of [k0, k1) of a row in 64-bit fixed point, by NT threads that meet at
+// sync(): `ch` elements at a time through `sx` (ch values), two butterfly levels per pass.
+// visit(k, S0, S1, l) sees elements k and k + 1 of every chunk.  Small code on purpose: it
+// runs for few rows and must not cost the others registers.
+template <class Sync, class Visit>
+__device__ __forceinline__ void slow_sums(const RQArgs& a, int row, int k0, int k1, int ch, long long* sx, int tid, int NT,
+                                          Sync sync, Visit visit) {
   const int tail_start = a.nfull << a.log2B;
 #pragma unroll 1
   for (int c0 = k0; c0 < k1;) {
     const int end = c0 < tail_start ? min(k1, tail_start) : k1;
     const int l = c0 < tail_start ? a.log2B : a.log2T;
     const int len = min(ch, end - c0);
-    __syncthreads();
+    sync();
 #pragma unroll 1
     for (int i = tid; i < ch; i += NT) {
       long long f = 0;
@@ -505,50 +506,47 @@ __device__ __forceinline__ void slow_sums(const RQArgs& a, int row, int k0, int 
         f = half_to_fixed(__half_as_ushort(a.x[(size_t)row * a.K + c0 + i]));
         if (a.signs != nullptr && a.signs[c0 + i] < 0) f = -f;
       }
-      sx[pad_idx(i)] = f;
+      sx[i] = f;
     }
 #pragma unroll 1
     for (int b = 0; b < l; b += 2) {
-      __syncthreads();
+      sync();
       const bool two = b + 1 < l;
 #pragma unroll 1
       for (int t = tid; t < ch >> (two ? 2 : 1); t += NT) {
-        const int i0 = ((t >> b) << (b + (two ? 2 : 1))) | (t & ((1 << b) - 1));
-        long long* p0 = sx + pad_idx(i0);
-        long long* p1 = sx + pad_idx(i0 + (1 << b));
-        const long long s = *p0 + *p1, d = *p0 - *p1;
+        long long* p = sx + (((t >> b) << (b + (two ? 2 : 1))) | (t & ((1 << b) - 1)));
+        const int d = 1 << b;
+        const long long s = p[0] + p[d], e = p[0] - p[d];
         if (!two) {
-          *p0 = s;
-          *p1 = d;
+          p[0] = s;
+          p[d] = e;
         } else {
-          long long* p2 = sx + pad_idx(i0 + (2 << b));
-          long long* p3 = sx + pad_idx(i0 + (3 << b));
-          const long long s2 = *p2 + *p3, d2 = *p2 - *p3;
-          *p0 = s + s2;
-          *p1 = d + d2;
-          *p2 = s - s2;
-          *p3 = d - d2;
+          const long long s2 = p[2 * d] + p[3 * d], e2 = p[2 * d] - p[3 * d];
+          p[0] = s + s2;
+          p[d] = e + e2;
+          p[2 * d] = s - s2;
+          p[3 * d] = e - e2;
         }
       }
     }
-    __syncthreads();
+    sync();
 #pragma unroll 1
-    for (int i = 2 * tid; i < len; i += 2 * NT) visit(c0 + i, sx[pad_idx(i)], sx[pad_idx(i + 1)], l);
+    for (int i = 2 * tid; i < len; i += 2 * NT) visit(c0 + i, sx[i], sx[i + 1], l);
     c0 += len;
   }
 }
 
-// The CTA's share of a row in 64-bit fixed point, twice: the row maximum (`rowmax`: this
+// A share [k0, k1) of a row in 64-bit fixed point, twice: the row maximum (`rowmax`: this
 // thread's maximum in, the row's out), then the codes.
-template <int MODE, class RowMax>
-__device__ __forceinline__ void rotate_slow_row(const RQArgs& a, int row, int k0, int k1, int ch, uint8_t* smem,
-                                                const RowOut& dst, RowMax rowmax) {
+template <int MODE, class Sync, class RowMax>
+__device__ __forceinline__ void rotate_slow_row(const RQArgs& a, int row, int k0, int k1, int ch, uint8_t* smem, int tid,
+                                                int NT, Sync sync, const RowOut& dst, RowMax rowmax) {
   long long* sx = reinterpret_cast<long long*>(smem);
   float m = 0.f, amax = 0.f, s = 0.f;
   const float qmaxf = (float)((1 << (a.bits - 1)) - 1), qminf = -(float)(1 << (a.bits - 1));
 #pragma unroll 1
   for (int pass = MODE == kRQY ? 1 : 0; pass < 2; ++pass) {
-    slow_sums(a, row, k0, k1, ch, sx, [&](int k, long long S0, long long S1, int l) {
+    slow_sums(a, row, k0, k1, ch, sx, tid, NT, sync, [&](int k, long long S0, long long S1, int l) {
       const float y0 = fixed_to_rotated(S0, l, a.c_hi, a.c_lo), y1 = fixed_to_rotated(S1, l, a.c_hi, a.c_lo);
       if (pass == 0) {
         m = fmaxf(m, fmaxf(fabsf(y0), fabsf(y1)));
@@ -566,6 +564,218 @@ __device__ __forceinline__ void rotate_slow_row(const RQArgs& a, int row, int k0
       s = __fdiv_rn(amax, qmaxf);
     }
   }
+}
+
+// ---------------------------------------------------------------- one unit, all steps
+// The steps that the standalone kernel and the fused decode launch share.  Geometry of a
+// warp's unit within its row:
+template <int G>
+struct UnitGeom {
+  int e0, eg;            // first element of the unit, of its group
+  int load_end, store_end;
+  int l;                 // log2 of the unit's block
+  int wg, tg;            // warp and thread within the group
+  bool in;               // the unit exists (the same for a whole group)
+  // `u`: the warp's unit in the row (groups start at multiples of G)
+  __device__ __forceinline__ UnitGeom(const RQArgs& a, int u, int lane, int row_end) {
+    const UnitMap um = unit_map(a.K, a.tail, G);
+    const int tail_start = a.nfull << a.log2B;
+    wg = u % G;
+    tg = wg * 32 + lane;
+    const int ug = u - wg;
+    const bool main_unit = ug < um.nmain;
+    in = ug < um.units;
+    eg = main_unit ? ug * kUnit : in ? tail_start + (ug - um.nmain) * kUnit : row_end;
+    e0 = eg + wg * kUnit;
+    load_end = main_unit ? tail_start : a.K;
+    store_end = main_unit && a.tail ? tail_start : row_end;
+    l = main_unit ? a.log2B : a.log2T;
+  }
+  // First element of unit u (K past the last).
+  static __device__ __forceinline__ int first(const RQArgs& a, int u) {
+    const UnitMap um = unit_map(a.K, a.tail, G);
+    return u < um.nmain ? min(u * kUnit, a.K) : u == um.nmain ? a.nfull << a.log2B : a.K;
+  }
+};
+
+// From the loaded halves to the thread's exact sums; false when the unit's block leaves the
+// pair form (v is then meaningless).  l1s: a word per warp of the group; group_sync: its
+// barrier; after_split(): called when w is free (the next row's loads).
+template <int G, class GroupSync, class After>
+__device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, uint32_t (&w)[16], const uint32_t (&am)[4], int lane,
+                                          uint8_t* xu, uint32_t* l1s, GroupSync group_sync, After after_split,
+                                          uint64_t (&v)[32]) {
+  constexpr int full_l = G == 1 ? 10 : G == 2 ? 11 : 12;
+  uint32_t l1 = unit_l1(w);
+  if constexpr (G > 1) {
+    if (lane == 0) l1s[u.wg] = l1;
+    group_sync();
+    l1 = 0;
+#pragma unroll
+    for (int i = 0; i < G; ++i) l1 += l1s[i];
+  }
+  bool ok = l1 < kL1Slow;
+  const int k = ok ? split_k(l1, u.l) : 0;
+  if (k > 0) ok = __all_sync(0xffffffffu, unit_on_grid(w, k));
+  if (u.l >= 8)
+    unit_phase1<true>(w, am, u.l, k, lane, xu);
+  else
+    unit_phase1<false>(w, am, u.l, k, lane, xu);
+  after_split();
+  group_sync();
+  const uint8_t* xg = xu - u.wg * kUnitBytes;
+  if (u.l == full_l)
+    unit_phase2<G, true>(xg, u.tg, u.l, v);
+  else
+    unit_phase2<G, false>(xg, u.tg, u.l, v);
+  return ok;
+}
+
+// Largest |y| of the warp, as fp32 bits, or 0 if it is certainly not the largest of the
+// warps that share `lead` (zero before the row's first warp).
+__device__ __forceinline__ uint32_t unit_max(const uint64_t (&v)[32], int l, uint32_t* lead, int lane, float c_hi,
+                                             float c_lo) {
+  uint32_t mine;
+  const uint32_t wm = warp_sum_max(v, mine);
+  uint32_t m = __float_as_uint(__fmul_rn(__uint_as_float(wm), __int_as_float((127 - (l >> 1)) << 23)));
+  if (l & 1) {
+    // 2^-j fl(S) / sqrt 2, rounded twice, is within 2 units of y: only warps that are not
+    // clearly below another form their largest y exactly.
+    m = __float_as_uint(__fmul_rn(__uint_as_float(m), c_hi));
+    uint32_t seen = 0u;
+    if (lane == 0) seen = atomicMax(lead, m);
+    seen = __shfl_sync(0xffffffffu, seen, 0);
+    m = seen > m + 8u ? 0u
+                      : __reduce_max_sync(0xffffffffu, __float_as_uint(largest_rotated(v, wm, mine == wm, l, c_hi, c_lo)));
+  }
+  return m;
+}
+
+// The thread's codes (kRQY: rotated values) to their places; s: the row's scale.
+template <int MODE, int G>
+__device__ __forceinline__ void unit_store(const RQArgs& a, const UnitGeom<G>& u, const uint64_t (&v)[32], float amax,
+                                           float s, const RowOut& dst) {
+  using RL = RunLayout<G>;
+  const float p2 = __int_as_float((127 - (u.l >> 1)) << 23);   // 2^-(l / 2)
+  const float r = __fmul_rn((u.l & 1) ? __fmul_rn(p2, a.c_hi) : p2, amax > 0.f ? __frcp_rn(s) : 0.f);
+  const float margin = a.bits == 4 ? 0x1p-17f : 0x1p-13f;
+  const int kb = u.eg + RL::low(u.tg);
+  uint8_t* at = dst.at<MODE>(kb);
+  const size_t step = dst.step256<MODE>();
+#pragma unroll
+  for (int e = 0; e < 32; e += 8) {
+    float q[8];
+    if constexpr (MODE == kRQY) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float h, o;
+        f2_unpack(v[e + i], h, o);
+        q[i] = pair_to_rotated(h, o, u.l, a.c_hi, a.c_lo);
+      }
+    } else {
+      pair_codes(v, e, u.l, s, r, margin, a.c_hi, a.c_lo, q);
+    }
+#pragma unroll
+    for (int c = 0; c < 8 / RL::R; ++c) {
+      if (kb + 256 * (e / RL::R + c) < u.store_end) store_codes_at<MODE, RL::R>(dst, at, q + c * RL::R);
+      at += step;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- fused decode launch
+// Row `row` of the token rows, or its share `part` of `cpr` (1 or 2 CTAs a row, up to 8 units
+// each), by the 8 converter warps of one CTA of the fused GEMM, into the operand planes:
+// a unit per warp, the row maximum through `sh` (32 words, zero before), and between the two
+// CTAs of a row through its line of a.pmax in global memory (words 0, 1: 1 + the bits of
+// each maximum, 0 = not yet written; words 4, 5 the same for rows in 64-bit integers).
+__device__ __forceinline__ uint32_t row_max_exchange(uint32_t* slots, int part, uint32_t mine, long long wait_cycles,
+                                                     int* err) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(slots + part), "r"(mine + 1u) : "memory");
+  const long long t0 = clock64();
+  while (true) {
+    uint32_t o;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(o) : "l"(slots + (part ^ 1)) : "memory");
+    if (o != 0u) return max(mine, o - 1u);
+    if (clock64() - t0 > wait_cycles) {   // bounded: the error word is set and the own maximum stands in
+      atomicCAS(err, 0, (int)kDevTimeoutRowMax);
+      return mine;
+    }
+    __nanosleep(20);
+  }
+}
+
+template <int G, class Sync>
+__device__ __forceinline__ void fused_rotate_row(const RQArgs& a, int row, int part, int cpr, int wpc, uint8_t* smem,
+                                                 uint32_t* sh, int wc, int lane, Sync sync, long long wait_cycles,
+                                                 int* err) {
+  uint32_t* const red = sh;            // [8] warp maxima
+  uint32_t* const l1s = sh + 8;        // [8]
+  uint32_t* const lead = sh + 16;
+  uint32_t* const bc = sh + 17;
+  const int tid = wc * 32 + lane;
+  const UnitGeom<G> u(a, part * wpc + wc, lane, a.KB * 128);
+  RowOut dst;
+  dst.p = static_cast<uint8_t*>(a.out);
+  dst.plane = (size_t)a.KB * a.rows_out * 128;
+  dst.kb_stride = (size_t)a.rows_out * 128;
+  dst.row = row;
+  dst.bits = a.bits;
+  // debug builds: the row is one of the planes' (site 4), its units lie inside it (site 5)
+  // and its slots are one of the 64 lines (site 6)
+  const bool act = wc < wpc && u.in && DPTQ_CHECK(row < a.rows_in && row < a.rows_out, err, 4) &&
+                   DPTQ_CHECK(u.load_end <= a.K && u.store_end <= a.KB * 128, err, 5);
+  uint64_t v[32];
+  uint32_t m = 0u;
+  if (act) {
+    uint32_t w[16], am[4];
+    unit_load(a.x + (size_t)row * a.K, u.e0, u.load_end, lane, w);
+    mma_hadamard_a(u.l, lane, am);
+    if (a.signs != nullptr) unit_signs(a.signs, u.e0, u.load_end, lane, w);
+    const bool ok = unit_sums<G>(u, w, am, lane, smem + wc * kUnitBytes, l1s + wc - u.wg,
+                                 [&] {
+                                   if constexpr (G == 1)
+                                     __syncwarp();
+                                   else
+                                     asm volatile("bar.sync %0, %1;" ::"r"(2 + wc / G), "n"(32 * G) : "memory");
+                                 },
+                                 [] {}, v);
+    m = unit_max(v, u.l, lead, lane, a.c_hi, a.c_lo);
+    if (!ok) m = kRowSlow;
+  }
+  if (lane == 0) red[wc] = m;
+  sync();
+  m = __reduce_max_sync(0xffffffffu, red[lane & 7]);
+  uint32_t* const slots = a.pmax + kRowMaxStride * row;
+  auto across = [&](uint32_t mine, int off) -> uint32_t {   // the row's maximum over its CTAs
+    if (cpr == 1 || !DPTQ_CHECK(row < 64 && part < cpr && cpr <= 2, err, 6)) return mine;
+    if (tid == 0) *bc = row_max_exchange(slots + off, part, mine, wait_cycles, err);
+    sync();
+    return *(volatile uint32_t*)bc;
+  };
+  m = across(m, 0);
+  const float qmaxf = (float)((1 << (a.bits - 1)) - 1);
+  if (m == kRowSlow) {
+    const int k0 = UnitGeom<G>::first(a, part * wpc), k1 = UnitGeom<G>::first(a, (part + 1) * wpc);
+    rotate_slow_row<kRQAct>(a, row, k0, k1, kUnit * G, smem, tid, 256, sync, dst, [&](float mine) {
+      const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mine));
+      sync();
+      if (lane == 0) red[wc] = wm;
+      sync();
+      const float rm = __uint_as_float(across(__reduce_max_sync(0xffffffffu, red[lane & 7]), 4));
+      if (part == 0 && tid == 0) a.scales[row] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
+      return rm;
+    });
+    if (part == cpr - 1) {
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int kz = a.K + 4 * tid; kz < a.KB * 128; kz += 4 * 256) store_codes<kRQAct, 4>(dst, kz, zero);
+    }
+    return;
+  }
+  const float amax = __uint_as_float(m);
+  const float s = __fdiv_rn(amax, qmaxf);
+  if (part == 0 && tid == 0) a.scales[row] = s;
+  if (act) unit_store<kRQAct, G>(a, u, v, amax, s, dst);
 }
 
 }  // namespace dptq

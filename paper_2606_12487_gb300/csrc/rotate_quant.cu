@@ -41,33 +41,21 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
   extern __shared__ __align__(16) uint8_t rm_smem[];
-  __shared__ uint32_t red[2][16];    // [row parity][warp]: fp32 bits of the largest |y|, or kSlow
+  constexpr int kBatch = 1024;       // rows between looks at the left-over ones (32 words)
+  __shared__ uint32_t red[2][16];    // [row parity][warp]: fp32 bits of the largest |y|, or kRowSlow
   __shared__ uint32_t xmax[2][8];    // the same of the cluster's CTAs
   __shared__ uint32_t l1s[16];
   __shared__ uint32_t lead[2];       // [row parity]: largest |y| so far, nearly (odd log2 blocks)
-  constexpr uint32_t kSlow = 0xFFFFFFFFu;
-  constexpr int kBatch = 1024;       // rows between looks at the left-over ones (32 words)
   __shared__ uint32_t slow_rows[kBatch / 32];
   pdl_launch_dependents();
   pdl_wait();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int W = blockDim.x >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NT = blockDim.x, W = NT >> 5;
   const int rank = csize > 1 ? (int)(blockIdx.x % csize) : 0;   // one-dimensional clusters
   const int ncl = (int)gridDim.x / csize;
   const int K = a.K, K_pad = a.KB * 128;
-  const int tail_start = a.nfull << a.log2B;
-  const UnitMap um = unit_map(K, a.tail, G);
-  const int wg = warp % G, tg = wg * 32 + lane;   // warp and thread within the group
-  const int Ug = rank * W + warp - wg;            // the group's first unit (whole groups are in or out)
-  const bool main_unit = Ug < um.nmain;
-  const int eg = main_unit ? Ug * kUnit : Ug < um.units ? tail_start + (Ug - um.nmain) * kUnit : K_pad;
-  const int e0 = eg + wg * kUnit;
-  const int load_end = main_unit ? tail_start : K;
-  const int store_end = main_unit && a.tail ? tail_start : MODE == kRQAct ? K_pad : K;
-  const int l = main_unit ? a.log2B : a.log2T;
-  constexpr int full_l = G == 1 ? 10 : G == 2 ? 11 : 12;
+  const UnitGeom<G> u(a, rank * W + warp, lane, MODE == kRQAct ? K_pad : K);
   uint8_t* const xu = rm_smem + warp * kUnitBytes;
-  uint8_t* const xg = xu - wg * kUnitBytes;
   auto group_sync = [&] {
     if constexpr (G == 1)
       __syncwarp();
@@ -78,11 +66,11 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
   int xpar = 0;
   auto cluster_max = [&](uint32_t v) -> uint32_t {
     if (csize == 1) return v;
-    if ((int)threadIdx.x < csize) {
+    if (tid < csize) {
       const uint32_t at = smem_u32(&xmax[xpar][rank]);
       asm volatile(
           "{\n\t.reg .b32 r;\n\tmapa.shared::cluster.u32 r, %0, %1;\n\tst.shared::cluster.u32 [r], %2;\n\t}\n" ::"r"(at),
-          "r"(threadIdx.x), "r"(v)
+          "r"(tid), "r"(v)
           : "memory");
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -92,163 +80,99 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
     return m;
   };
   uint32_t am[4];
-  mma_hadamard_a(l, lane, am);
-  const int bits = a.bits;
-  const float qmaxf = (float)((1 << (bits - 1)) - 1);
-  const float margin = bits == 4 ? 0x1p-17f : 0x1p-13f;
+  mma_hadamard_a(u.l, lane, am);
+  const float qmaxf = (float)((1 << (a.bits - 1)) - 1);
   RowOut dst;
   dst.plane = (size_t)a.KB * a.rows_out * 128;
   dst.kb_stride = (size_t)a.rows_out * 128;
-  dst.bits = bits;
-
-  const float p2 = __int_as_float((127 - (l >> 1)) << 23);   // 2^-(l / 2)
-  if (threadIdx.x < 2) lead[threadIdx.x] = 0u;
-  if (threadIdx.x < kBatch / 32) slow_rows[threadIdx.x] = 0u;
-  __syncthreads();
-
+  dst.bits = a.bits;
   auto row_out = [&](int r) {
     dst.row = r;
     dst.p = static_cast<uint8_t*>(a.out);
-    if (MODE == kRQPublic) dst.p += (size_t)r * (bits == 4 ? K / 2 : K);
+    if (MODE == kRQPublic) dst.p += (size_t)r * (a.bits == 4 ? K / 2 : K);
     if (MODE == kRQY) dst.p += (size_t)r * K * 4;
   };
+  if (tid < 2) lead[tid] = 0u;
+  if (tid < kBatch / 32) slow_rows[tid] = 0u;
+  __syncthreads();
 
   // Batches of up to kBatch rows: all of them by the pairs, then the ones left over.
   int par = 0;
 #pragma unroll 1
   for (int row0 = (int)blockIdx.x / csize; row0 < a.rows_out; row0 += kBatch * ncl) {
-  bool any_slow = false;
-  uint32_t w[16];
-  if (row0 < a.rows_in) unit_load(a.x + (size_t)row0 * K, e0, load_end, lane, w);
+    bool any_slow = false;
+    uint32_t w[16];
+    if (row0 < a.rows_in) unit_load(a.x + (size_t)row0 * K, u.e0, u.load_end, lane, w);
 #pragma unroll 1
-  for (int it = 0; it < kBatch; ++it, par ^= 1) {
-    const int row = row0 + it * ncl;
-    if (row >= a.rows_out) break;
-    row_out(row);
-    if (row >= a.rows_in) {   // padding row (operand planes): zero codes and scale
-      if (MODE == kRQAct) {
-        const float zero[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int k = 4 * (rank * (int)blockDim.x + (int)threadIdx.x); k < K_pad; k += 4 * csize * (int)blockDim.x)
-          store_codes<kRQAct, 4>(dst, k, zero);
-        if (rank == 0 && threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = 0.f;
-      }
-      continue;
-    }
-    if (a.signs != nullptr) unit_signs(a.signs, e0, load_end, lane, w);
-    uint32_t l1 = unit_l1(w);
-    if constexpr (G > 1) {
-      if (lane == 0) l1s[warp] = l1;
-      group_sync();
-      l1 = 0;
-#pragma unroll
-      for (int i = 0; i < G; ++i) l1 += l1s[warp - wg + i];
-    }
-    bool slow = l1 >= kL1Slow;
-    const int k = slow ? 0 : split_k(l1, l);
-    if (k > 0) slow = !__all_sync(0xffffffffu, unit_on_grid(w, k));
-    if (l >= 8)
-      unit_phase1<true>(w, am, l, k, lane, xu);
-    else
-      unit_phase1<false>(w, am, l, k, lane, xu);
-    if (it + 1 < kBatch && row + ncl < a.rows_in) unit_load(a.x + (size_t)(row + ncl) * K, e0, load_end, lane, w);
-    group_sync();
-    uint64_t v[32];
-    if (l == full_l)
-      unit_phase2<G, true>(xg, tg, l, v);
-    else
-      unit_phase2<G, false>(xg, tg, l, v);
-    uint32_t m = 0u;
-    if constexpr (MODE != kRQY) {
-      uint32_t mine;
-      const uint32_t wm = warp_sum_max(v, mine);
-      m = __float_as_uint(__fmul_rn(__uint_as_float(wm), p2));
-      if (l & 1) {
-        // 2^-j fl(S) / sqrt 2, rounded twice, is within 2 units of y: only warps that are not
-        // clearly below another form their largest y exactly.
-        m = __float_as_uint(__fmul_rn(__uint_as_float(m), a.c_hi));
-        uint32_t seen = 0u;
-        if (lane == 0) seen = atomicMax(&lead[par], m);
-        seen = __shfl_sync(0xffffffffu, seen, 0);
-        m = seen > m + 8u ? 0u
-                          : __reduce_max_sync(0xffffffffu, __float_as_uint(largest_rotated(
-                                                               v, wm, mine == wm, l, a.c_hi, a.c_lo)));
-      }
-    }
-    if (slow) m = kSlow;
-    if (lane == 0) red[par][warp] = m;
-    if (threadIdx.x == 0) lead[par ^ 1] = 0u;
-    __syncthreads();
-    m = __reduce_max_sync(0xffffffffu, lane < W ? red[par][lane] : 0u);
-    m = cluster_max(m);
-    if (m == kSlow) {   // left for the loop below
-      if (threadIdx.x == 0) slow_rows[it >> 5] |= 1u << (it & 31);
-      any_slow = true;
-      continue;
-    }
-    const float amax = __uint_as_float(m);
-    const float s = __fdiv_rn(amax, qmaxf);
-    const float rs = amax > 0.f ? __frcp_rn(s) : 0.f;
-    if (MODE != kRQY && rank == 0 && threadIdx.x == 0 && a.scales != nullptr) a.scales[row] = s;
-    const float r = __fmul_rn((l & 1) ? __fmul_rn(p2, a.c_hi) : p2, rs);
-    using RL = RunLayout<G>;
-    const int kb = eg + RL::low(tg);
-    uint8_t* at = dst.at<MODE>(kb);
-    const size_t step = dst.step256<MODE>();
-#pragma unroll
-    for (int e = 0; e < 32; e += 8) {
-      float q[8];
-      if constexpr (MODE == kRQY) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float h, o;
-          f2_unpack(v[e + i], h, o);
-          q[i] = pair_to_rotated(h, o, l, a.c_hi, a.c_lo);
+    for (int it = 0; it < kBatch; ++it, par ^= 1) {
+      const int row = row0 + it * ncl;
+      if (row >= a.rows_out) break;
+      row_out(row);
+      if (row >= a.rows_in) {   // padding row (operand planes): zero codes and scale
+        if (MODE == kRQAct) {
+          const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+          for (int k = 4 * (rank * NT + tid); k < K_pad; k += 4 * csize * NT) store_codes<kRQAct, 4>(dst, k, zero);
+          if (rank == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = 0.f;
         }
-      } else {
-        pair_codes(v, e, l, s, r, margin, a.c_hi, a.c_lo, q);
+        continue;
       }
-#pragma unroll
-      for (int c = 0; c < 8 / RL::R; ++c) {
-        const int kk = kb + 256 * (e / RL::R + c);
-        if (kk < store_end) store_codes_at<MODE, RL::R>(dst, at, q + c * RL::R);
-        at += step;
+      if (a.signs != nullptr) unit_signs(a.signs, u.e0, u.load_end, lane, w);
+      uint64_t v[32];
+      const bool ok = unit_sums<G>(
+          u, w, am, lane, xu, l1s + warp - u.wg, group_sync,
+          [&] {
+            if (it + 1 < kBatch && row + ncl < a.rows_in)
+              unit_load(a.x + (size_t)(row + ncl) * K, u.e0, u.load_end, lane, w);
+          },
+          v);
+      uint32_t m = MODE == kRQY ? 0u : unit_max(v, u.l, &lead[par], lane, a.c_hi, a.c_lo);
+      if (!ok) m = kRowSlow;
+      if (lane == 0) red[par][warp] = m;
+      if (tid == 0) lead[par ^ 1] = 0u;
+      __syncthreads();
+      m = __reduce_max_sync(0xffffffffu, lane < W ? red[par][lane] : 0u);
+      m = cluster_max(m);
+      if (m == kRowSlow) {   // left for the loop below
+        if (tid == 0) slow_rows[it >> 5] |= 1u << (it & 31);
+        any_slow = true;
+        continue;
       }
+      const float amax = __uint_as_float(m);
+      const float s = __fdiv_rn(amax, qmaxf);
+      if (MODE != kRQY && rank == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = s;
+      unit_store<MODE, G>(a, u, v, amax, s, dst);
     }
-  }
-  if (!any_slow) continue;
-  const int u0 = rank * W, u1 = u0 + W;
-  auto first = [&](int u) { return u < um.nmain ? u * kUnit : u == um.nmain ? tail_start : K; };
+    if (!any_slow) continue;
+    const int k0 = UnitGeom<G>::first(a, rank * W), k1 = UnitGeom<G>::first(a, (rank + 1) * W);
 #pragma unroll 1
-  for (int it = 0; it < kBatch; ++it) {
-    const int row = row0 + it * ncl;
-    if (row >= a.rows_out) break;
-    __syncthreads();
-    if (!((slow_rows[it >> 5] >> (it & 31)) & 1u)) continue;
-    row_out(row);
-    rotate_slow_row<MODE>(a, row, min(first(u0), K), min(first(u1), K), kUnit * G, rm_smem, dst, [&](float mine) {
-      const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mine));
+    for (int it = 0; it < kBatch; ++it) {
+      const int row = row0 + it * ncl;
+      if (row >= a.rows_out) break;
       __syncthreads();
-      if (lane == 0) red[0][warp] = wm;
-      __syncthreads();
-      const float rm = __uint_as_float(cluster_max(__reduce_max_sync(0xffffffffu, lane < W ? red[0][lane] : 0u)));
-      if (MODE != kRQY && rank == 0 && threadIdx.x == 0 && a.scales != nullptr)
-        a.scales[row] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
-      return rm;
-    });
-    if (MODE == kRQAct && rank == csize - 1) {
-      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int kz = K + 4 * (int)threadIdx.x; kz < K_pad; kz += 4 * (int)blockDim.x) store_codes<kRQAct, 4>(dst, kz, zero);
+      if (!((slow_rows[it >> 5] >> (it & 31)) & 1u)) continue;
+      row_out(row);
+      rotate_slow_row<MODE>(a, row, k0, k1, kUnit * G, rm_smem, tid, NT, [] { __syncthreads(); }, dst, [&](float mine) {
+        const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mine));
+        __syncthreads();
+        if (lane == 0) red[0][warp] = wm;
+        __syncthreads();
+        const float rm = __uint_as_float(cluster_max(__reduce_max_sync(0xffffffffu, lane < W ? red[0][lane] : 0u)));
+        if (rank == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
+        return rm;
+      });
+      if (MODE == kRQAct && rank == csize - 1) {
+        const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int kz = K + 4 * tid; kz < K_pad; kz += 4 * NT) store_codes<kRQAct, 4>(dst, kz, zero);
+      }
     }
-  }
-  __syncthreads();
-  if (threadIdx.x < kBatch / 32) slow_rows[threadIdx.x] = 0u;
-  __syncthreads();
+    __syncthreads();
+    if (tid < kBatch / 32) slow_rows[tid] = 0u;
+    __syncthreads();
   }
 }
 
-// Warps that share a Hadamard block of the row.
-int rotate_group(const RQArgs& a) {
-  const int b = a.nfull > 0 ? a.B : a.tail;
+int rotate_group(int K, int B, int tail) {
+  const int b = K > tail ? B : tail;
   return b <= kUnit ? 1 : b / kUnit;
 }
 
@@ -263,8 +187,7 @@ cudaError_t launch_rotate_mma_g(const RQArgs& a, cudaStream_t s, bool pdl) {
   const int units = unit_map(a.K, a.tail, G).units;
   const int csize = ceil_div(units, 16);
   const int W = round_up(ceil_div(units, csize), G);
-  // The exchange, and (rows rotated in 64-bit integers) a padded block of 1024 G values.
-  const int smem = std::max(W * kUnitBytes, G * (kUnit + kUnit / 16) * 8);
+  const int smem = W * kUnitBytes;   // the exchange, or (64-bit integers) a block of 1024 G values
   int sms = 0;
   cudaError_t e = device_sms(&sms);
   if (e == cudaSuccess) e = ensure_max_dyn_smem(rotate_mma_kernel<MODE, G>);
@@ -295,7 +218,7 @@ cudaError_t launch_rotate_mma_g(const RQArgs& a, cudaStream_t s, bool pdl) {
 
 template <int MODE>
 cudaError_t launch_rotate_mma(const RQArgs& a, cudaStream_t s, bool pdl) {
-  switch (rotate_group(a)) {
+  switch (rotate_group(a.K, a.B, a.tail)) {
     case 1: return launch_rotate_mma_g<MODE, 1>(a, s, pdl);
     case 2: return launch_rotate_mma_g<MODE, 2>(a, s, pdl);
     default: return launch_rotate_mma_g<MODE, 4>(a, s, pdl);
@@ -311,7 +234,7 @@ size_t rotate_quant_smem(int K, int chunk) {
 cudaError_t launch_rotate_quant(RQMode mode, const RQArgs& a, cudaStream_t s, bool pdl) {
   // Activations take the tensor-core kernel; a Paley tail and the weight packer (16
   // consecutive codes a thread) the per-row kernel.
-  if (a.tail_p == 1 && rows_kernel_allowed()) {
+  if (a.tail_p <= 1 && rows_kernel_allowed()) {
     switch (mode) {
       case kRQPublic: return launch_rotate_mma<kRQPublic>(a, s, pdl);
       case kRQAct: return launch_rotate_mma<kRQAct>(a, s, pdl);

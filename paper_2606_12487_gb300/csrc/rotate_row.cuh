@@ -1,7 +1,7 @@
 // rotate_row.cuh -- the per-row body of the fused online block-Hadamard rotation +
 // symmetric per-row quantization (Section 2, Eq. 4 then Eq. 2; Section 4.2 per-token /
-// per-channel symmetric), shared by the standalone kernel (rotate_quant.cu) and the
-// fused decode GEMM (qgemm.cu).  Exact 64-bit fixed-point Walsh-Hadamard butterflies
+// per-channel symmetric) in 64-bit integers: the weight packer, rows with a Paley tail, and
+// the pieces that the tensor-core rotation (rotate_mma.cuh) shares.  Exact 64-bit fixed-point Walsh-Hadamard butterflies
 // in registers with two shared-memory transposes per 4096-element chunk, one correctly
 // rounded conversion to fp32 including 1/sqrt(block), row absmax by warp shuffles,
 // IEEE-division rounding to the integer grid, and one of four writers:
@@ -520,626 +520,6 @@ __device__ __forceinline__ void rotate_quant_row(const RQArgs& a, int row, unsig
     }
   }
 #undef RQ_TRACE
-}
-
-// ---------------------------------------------------------------- fused decode launch
-// Element index of value e of thread t in the layout the butterflies of a chunk end in:
-// 0 = round A only (blocks of at most 16), 1 = rounds A and B (at most 256), 2 = all.
-__device__ __forceinline__ int rq_pos(int layout, int t, int e) {
-  return layout == 2 ? 256 * e + t : layout == 1 ? 256 * (t >> 4) + 16 * e + (t & 15) : 16 * t + e;
-}
-
-// Raw fp16 words of thread `tid`'s 16 consecutive values of the chunk at c0 (round A
-// layout, i = 16 tid + e); zeros past the chunk's length.
-__device__ __forceinline__ void rq_load16(const uint4* src, int c0, int len, int tid, uint4 (&u)[2]) {
-  const int i0 = tid * 16;
-  if (i0 < len) {
-    u[0] = src[(c0 + i0) / 8];
-    u[1] = src[(c0 + i0) / 8 + 1];
-  } else {
-    u[0] = make_uint4(0u, 0u, 0u, 0u);
-    u[1] = u[0];
-  }
-}
-
-// The 16 raw fp16 values to exact fixed point, with the randomized-Hadamard signs.
-__device__ __forceinline__ void rq_fix16(const RQArgs& a, const uint4 (&u)[2], int c0, int len, int tid,
-                                         long long (&f)[16]) {
-  const uint32_t w[8] = {u[0].x, u[0].y, u[0].z, u[0].w, u[1].x, u[1].y, u[1].z, u[1].w};
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    f[2 * k] = half_to_fixed(w[k] & 0xFFFFu);
-    f[2 * k + 1] = half_to_fixed(w[k] >> 16);
-  }
-  if (a.signs != nullptr && tid * 16 < len) apply_signs(a.signs + c0 + tid * 16, f);
-}
-
-// The exact butterflies of one chunk (elements c0 .. c0 + len - 1 of the row), starting
-// from f[] in the round A layout; returns the layout f[] ends in (see rq_pos).
-template <class Sync>
-__device__ __forceinline__ int rq_bfly(const RQArgs& a, int c0, int len, int tail_start, long long (&f)[16],
-                                       long long* sx, int tid, Sync sync) {
-  unsigned long long* const tr = DPTQ_TRACE_BUF();
-  (void)tr;
-#define RQC_T(slot) \
-  do {              \
-    if (tid == 0 && c0 == 0) DPTQ_TRACE_CLOCK(tr, slot); \
-  } while (0)
-  auto lg = [&](int i) { return (c0 + i < tail_start) ? a.log2B : a.log2T; };
-  auto bfly = [&](int h) {
-#pragma unroll
-    for (int e = 0; e < 16; ++e)
-      if ((e & h) == 0) {
-        const long long p = f[e], q = f[e + h];
-        f[e] = p + q;
-        f[e + h] = p - q;
-      }
-  };
-  const int i0 = tid * 16;
-  RQC_T(171);
-  {
-    const int L = lg(i0 < len ? i0 : 0);
-    if (L >= 4) {
-      bfly(1);
-      bfly(2);
-      bfly(4);
-      bfly(8);
-    } else {
-#pragma unroll
-      for (int bit = 0; bit < 4; ++bit)
-        if (bit < L) bfly(1 << bit);
-    }
-  }
-  RQC_T(172);
-  const int maxlg = (c0 + len > tail_start) ? max(a.log2B, a.log2T) : a.log2B;
-  if (maxlg <= 4) return 0;
-  sync();   // the previous readers of sx are done
-#pragma unroll
-  for (int e = 0; e < 16; ++e) sx[pad_idx(i0 + e)] = f[e];
-  sync();
-  const int iB = 256 * (tid >> 4) + (tid & 15);
-#pragma unroll
-  for (int e = 0; e < 16; ++e) f[e] = sx[pad_idx(iB + 16 * e)];
-  RQC_T(173);
-  {
-    const int L = lg(iB);
-    if (L >= 8) {
-      bfly(1);
-      bfly(2);
-      bfly(4);
-      bfly(8);
-    } else {
-#pragma unroll
-      for (int bit = 4; bit < 8; ++bit)
-        if (bit < L) bfly(1 << (bit - 4));
-    }
-  }
-  RQC_T(174);
-  if (maxlg <= 8) return 1;
-#pragma unroll
-  for (int e = 0; e < 16; ++e) sx[pad_idx(iB + 16 * e)] = f[e];
-  sync();
-#pragma unroll
-  for (int e = 0; e < 16; ++e) f[e] = sx[pad_idx(256 * e + tid)];
-  RQC_T(175);
-  if (c0 + len <= tail_start && a.log2B == 12) {
-    bfly(1);
-    bfly(2);
-    bfly(4);
-    bfly(8);
-  } else if (c0 + len <= tail_start) {
-#pragma unroll
-    for (int bit = 8; bit < 12; ++bit)
-      if (bit < a.log2B) bfly(1 << (bit - 8));
-  } else {
-#pragma unroll
-    for (int bit = 8; bit < 12; ++bit) {
-      const int h = 1 << (bit - 8);
-#pragma unroll
-      for (int e = 0; e < 16; ++e)
-        if ((e & h) == 0 && bit < lg(256 * e + tid)) {
-          const long long p = f[e], q = f[e + h];
-          f[e] = p + q;
-          f[e + h] = p - q;
-        }
-    }
-  }
-  RQC_T(176);
-#undef RQC_T
-  return 2;
-}
-
-// Load, fix and butterflies of one chunk: the same arithmetic as rotate_quant_row.
-template <class Sync>
-__device__ __forceinline__ int rq_chunk(const RQArgs& a, const uint4* src, int c0, int len, int tail_start,
-                                        long long (&f)[16], long long* sx, int tid, Sync sync) {
-  uint4 u[2];
-  rq_load16(src, c0, len, tid, u);
-  rq_fix16(a, u, c0, len, tid, f);
-  return rq_bfly(a, c0, len, tail_start, f, sx, tid, sync);
-}
-
-// The same butterflies as rq_bfly with a small code footprint, for code that runs once
-// per launch (the fused decode rotation), where every instruction is fetched cold: the
-// three rounds share one body (a transpose through sx between rounds, then the round's
-// four levels on the 16 values in registers), so rounds B and C run from instructions
-// that round A brought into the instruction cache.  Returns the layout f[] ends in.
-template <class Sync>
-__device__ __forceinline__ int rq_bfly_compact(const RQArgs& a, int c0, int len, int tail_start, long long (&f)[16],
-                                            long long* sx, int tid, Sync sync) {
-  const int maxlg = (c0 + len > tail_start) ? max(a.log2B, a.log2T) : a.log2B;
-  const int rounds = maxlg <= 4 ? 1 : maxlg <= 8 ? 2 : 3;
-  // Blocks are B-sized before tail_start and tail-sized after, so only chunks that reach
-  // the tail can mix block sizes.
-  const bool mixed = c0 + len > tail_start && a.log2T != a.log2B;
-  // Padded index of value e of this thread in layout r: pad_idx(rq_pos(r, tid, e)) =
-  // pb[r] + ps[r] e, since every layout is linear in e (strides 1, 16, 256) and the
-  // padding adds one slot per 16 elements.
-  const int pb0 = 17 * tid;
-  const int ib1 = 256 * (tid >> 4) + (tid & 15);
-  const int pb1 = ib1 + (ib1 >> 4);
-  const int pb2 = tid + (tid >> 4);
-#pragma unroll 1
-  for (int r = 0; r < rounds; ++r) {
-    if (r > 0) {
-      const int wb = r == 1 ? pb0 : pb1, ws = r == 1 ? 1 : 17;
-      const int rb = r == 1 ? pb1 : pb2, rs = r == 1 ? 17 : 272;
-      sync();   // the previous readers of sx are done
-      long long* wp = sx + wb;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) wp[ws * e] = f[e];
-      sync();
-      const long long* rp = sx + rb;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) f[e] = rp[rs * e];
-    }
-    const int base = 4 * r;
-    if (!mixed && a.log2B >= base + 4) {   // every element's block spans the round's 4 levels
-#pragma unroll
-      for (int bit = 0; bit < 4; ++bit) {
-        const int h = 1 << bit;
-#pragma unroll
-        for (int e = 0; e < 16; ++e)
-          if ((e & h) == 0) {
-            const long long p = f[e], q = f[e + h];
-            f[e] = p + q;
-            f[e + h] = p - q;
-          }
-      }
-    } else {
-      // A level applies to an element while it is below the log2 of the element's block.
-#pragma unroll
-      for (int bit = 0; bit < 4; ++bit) {
-        const int lvl = base + bit;
-        const int h = 1 << bit;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          if ((e & h) == 0) {
-            const int i = rq_pos(r, tid, e);
-            const int lg = (c0 + i < tail_start) ? a.log2B : a.log2T;
-            if (lvl < lg) {
-              const long long p = f[e], q = f[e + h];
-              f[e] = p + q;
-              f[e + h] = p - q;
-            }
-          }
-        }
-      }
-    }
-  }
-  return rounds - 1;
-}
-
-__device__ __forceinline__ uint32_t e4m3_byte(float v) { return e4m3x2(v, 0.f) & 0xFFu; }
-
-static_assert(kRQPartSmemBytes == kChunkPadded * 8 + 2 * kChunk + 16 * 8, "part scratch layout");
-
-// ---- one row's rotation split over the parts of the fused decode launch
-// Each of the np parts of a row rotates only its own outputs, so the parts share the
-// work instead of repeating it; the row absmax, which every code depends on, is then
-// exchanged between the parts through one slot per part in global memory.
-//   * Whole blocks (kPartBlocks): the row splits into np ranges of whole 128-aligned
-//     granules (a granule is max(B, 128) elements: whole Hadamard blocks), each at most
-//     4096 elements, rotated like one chunk of rotate_quant_row.
-//   * Block slices (kPartSlice4 / kPartSlice8): when a row has fewer blocks than parts,
-//     each block of B = n L elements is shared by n parts.  With Sylvester's ordering
-//     H_B = H_n (x) H_L, so output slice p' of the block is H_L applied to
-//     v = sum_a H_n[p'][a] x_a, x_a the a-th L-element slice of the block's input: a part
-//     combines the n input slices at its L positions (exact) and runs the L-point
-//     butterflies, L = 256 V (V = 4 or 8 values per thread).
-enum : int { kPartBlocks = 1, kPartSlice4 = 4, kPartSlice8 = 8 };
-
-// Granule range [g0, g1) of `part` when ng granules are split over np parts.
-__device__ __forceinline__ void part_granules(int ng, int np, int part, int& g0, int& g1) {
-  g0 = part * ng / np;
-  g1 = (part + 1) * ng / np;
-}
-
-// Row absmax over the parts.  Thread 0 of the part stores 1 + the bits of its own
-// maximum (non-negative floats order as their bit patterns; 0 marks an empty slot) in
-// slot [row][part] (one 128-byte line per row), then reads the row's first four slots,
-// pausing between reads so that the pollers of a line leave the store of the last part
-// a way in, until the first np are set; the
-// slots are cleared for the next launch once every part of the launch is past this
-// point.  A slot holds only its own value, so relaxed accesses suffice.  Bounded: on
-// timeout the error word is set and the part's own maximum stands in.
-__device__ __forceinline__ float part_absmax_exchange(uint32_t* slots, int np, int part, float mine,
-                                                      long long wait_cycles, int* err) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(slots + part), "r"(__float_as_uint(mine) + 1u) : "memory");
-  const long long t0 = clock64();
-  while (true) {
-    uint32_t v[4];
-    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                 : "l"(slots)
-                 : "memory");
-    bool all = true;
-    uint32_t m = 0u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (i < np) {
-        all = all && v[i] != 0u;
-        m = v[i] > m ? v[i] : m;
-      }
-    if (all) return __uint_as_float(m - 1u);
-    if (clock64() - t0 > wait_cycles) {
-      atomicCAS(err, 0, (int)kDevTimeoutRowMax);
-      return mine;
-    }
-    __nanosleep(100);
-  }
-}
-
-// The part's largest |y| from the fp32 of each thread's largest |y| (`tmax`, >= 0): one
-// redux per warp on the bit patterns, the 8 warp maxima through `redf`, then the
-// exchange between the parts (thread 0) and its broadcast.  Two barriers.
-template <class Sync>
-__device__ __forceinline__ float part_row_absmax(const RQArgs& a, int row, int part, float tmax, float* redf, int tid,
-                                                 Sync sync, long long wait_cycles, int* err) {
-  const uint32_t wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(tmax));
-  if ((tid & 31) == 0) redf[tid >> 5] = __uint_as_float(wmax);
-  sync();
-  if (tid == 0) {
-    float pm = redf[0];
-#pragma unroll
-    for (int w = 1; w < kRQThreads / 32; ++w) pm = fmaxf(pm, redf[w]);
-    // debug builds: one of the 64 slot lines and a part of the row (site 6)
-    redf[8] = DPTQ_CHECK(row < 64 && part < a.np && a.np <= 4, err, 6)
-                  ? part_absmax_exchange(a.pmax + kRowMaxStride * row, a.np, part, pm, wait_cycles, err)
-                  : pm;
-  }
-  sync();
-  return redf[8];
-}
-
-// Codes k .. k + 3 of `row` (k % 4 == 0) into the GEMM operand planes (the 128-byte
-// swizzled K-major layout of rotate_quant_row<kRQAct>).
-__device__ __forceinline__ void part_store4(const RQArgs& a, int row, int k, uint32_t w0, uint32_t w1, int* err) {
-  uint8_t* act = static_cast<uint8_t*>(a.out);
-  // debug builds: inside the operand planes (site 4)
-  if (!DPTQ_CHECK(row < a.rows_out && k >= 0 && k + 4 <= a.KB * 128 && (k & 3) == 0, err, 4)) return;
-  const int kb = k >> 7, j = (k >> 4) & 7;
-  const size_t off = ((size_t)kb * a.rows_out + row) * 128 + ((j ^ (row & 7)) << 4) + (k & 15);
-  *reinterpret_cast<uint32_t*>(act + off) = w0;
-  if (a.bits == 8) *reinterpret_cast<uint32_t*>(act + (size_t)a.KB * a.rows_out * 128 + off) = w1;
-}
-
-// Padding row (row >= rows_in): zero codes, the K_pad / 4 words split evenly over the
-// parts, and a zero scale.
-__device__ __forceinline__ void part_zero_row(const RQArgs& a, int row, int part, int tid, int* err) {
-  const int W = a.KB * 32;
-  for (int w = W * part / a.np + tid; w < W * (part + 1) / a.np; w += kRQThreads) part_store4(a, row, 4 * w, 0u, 0u, err);
-  if (part == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = 0.f;
-}
-
-// Staged E4M3 byte(s) of one code: plane 0 (A4, or the A8 hi part) and plane 1 (A8 lo).
-__device__ __forceinline__ void part_code_bytes(float q, int bits, uint32_t& b0, uint32_t& b1) {
-  if (bits == 4) {
-    b0 = e4m3_byte(q);
-    b1 = 0u;
-  } else {
-    const float m = fabsf(q);
-    const float h = __fmul_rn(floorf(__fmul_rn(m, 0.0625f)), 16.f);
-    b0 = e4m3_byte(__fadd_rn(copysignf(h, q), 0.0f));   // + 0: no negative zeros
-    b1 = e4m3_byte(__fadd_rn(copysignf(__fsub_rn(m, h), q), 0.0f));
-  }
-}
-
-// Whole blocks: this part's granules [c0, c0 + len) of the row (len <= 4096), rotated as
-// one chunk (16 values per thread, the three-round butterflies of rq_bfly_compact), its
-// codes staged in shared memory and stored as 32-bit words of four consecutive codes.
-// smem: kRQPartSmemBytes, 16-byte aligned; 256 threads meet at sync(); the caller
-// synchronizes before reusing smem.
-template <class Sync>
-__device__ __forceinline__ void rotate_quant_part_blocks(const RQArgs& a, int row, int part, unsigned char* smem,
-                                                         int tid, Sync sync, long long wait_cycles, int* err) {
-  long long* sx = reinterpret_cast<long long*>(smem);
-  uint8_t* stg = smem;   // staged codes [2][4096] (plane 1 at +4096), in sx once its readers are done
-  float* redf = reinterpret_cast<float*>(smem + (size_t)kChunkPadded * 8 + 2 * kChunk);
-  unsigned long long* const tr = DPTQ_TRACE_BUF();
-  (void)tr;
-  if (row >= a.rows_in) {
-    part_zero_row(a, row, part, tid, err);
-    return;
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 170);
-  const int K = a.K;
-  const int tail_start = a.nfull << a.log2B;
-  const int gr = a.B > 128 ? a.B : 128;
-  int g0, g1;
-  part_granules((K + gr - 1) / gr, a.np, part, g0, g1);
-  const int c0 = min(K, g0 * gr);
-  const int len = min(K, g1 * gr) - c0;   // 0 .. 4096, a multiple of 32
-  long long f[16];
-  {
-    uint4 u[2];
-    rq_load16(reinterpret_cast<const uint4*>(a.x + (size_t)row * K), c0, len, tid, u);
-    rq_fix16(a, u, c0, len, tid, f);
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 171);
-  const int L = len > 0 ? rq_bfly_compact(a, c0, len, tail_start, f, sx, tid, sync) : 2;
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 176);
-  // Block size of the part's values: one size unless the part reaches into the tail
-  // block from a whole block.  Values past len are zero (whole zero blocks).
-  const bool mixed = c0 < tail_start && c0 + len > tail_start;
-  const int lgp = c0 >= tail_start ? a.log2T : a.log2B;
-  float tmax;
-  if (!mixed) {
-    long long m[8];   // pairwise tree of |S|
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const long long p = f[e] < 0 ? -f[e] : f[e], q = f[e + 8] < 0 ? -f[e + 8] : f[e + 8];
-      m[e] = p > q ? p : q;
-    }
-#pragma unroll
-    for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-      for (int e = 0; e < w; ++e) m[e] = m[e] > m[e + w] ? m[e] : m[e + w];
-    tmax = m[0] ? fixed_to_rotated(m[0], lgp, a.c_hi, a.c_lo) : 0.f;
-  } else {
-    long long mB = 0, mT = 0;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const long long v = f[e] < 0 ? -f[e] : f[e];
-      if (c0 + rq_pos(L, tid, e) < tail_start)
-        mB = v > mB ? v : mB;
-      else
-        mT = v > mT ? v : mT;
-    }
-    tmax = fmaxf(mB ? fixed_to_rotated(mB, a.log2B, a.c_hi, a.c_lo) : 0.f,
-                 mT ? fixed_to_rotated(mT, a.log2T, a.c_hi, a.c_lo) : 0.f);
-  }
-  // The fp32 values, converted before the exchange so that their arithmetic overlaps it
-  // (the conversion is odd and monotone: the fp32 of the largest |S| is the largest |y|).
-  // This code runs once per launch from a cold instruction cache, so the uniform choices
-  // (one block size or two, even or odd log2) are taken once, outside the unrolled loops.
-  float y[16];
-  if (!mixed && (lgp & 1) == 0) {
-    const float sc = __int_as_float((127 - 24 - (lgp >> 1)) << 23);   // 2^-(24 + lgp / 2), exact
-#pragma unroll
-    for (int e = 0; e < 16; ++e) y[e] = __fmul_rn(ll_to_float_rn(f[e]), sc);
-  } else if (!mixed) {
-#pragma unroll
-    for (int e = 0; e < 16; ++e) y[e] = fixed_times_const(f[e], lgp >> 1, a.c_hi, a.c_lo);
-  } else {   // a part that reaches from a whole block into the tail block (rare)
-#pragma unroll
-    for (int e = 0; e < 16; ++e)
-      y[e] = fixed_to_rotated(f[e], (c0 + rq_pos(L, tid, e) < tail_start) ? a.log2B : a.log2T, a.c_hi, a.c_lo);
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 140);
-  const float amax = part_row_absmax(a, row, part, tmax, redf, tid, sync, wait_cycles, err);   // also ends sx's reads
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 141);
-  const int bits = a.bits;
-  const float qmaxf = (float)((1 << (bits - 1)) - 1), qminf = -(float)(1 << (bits - 1));
-  const float s = __fdiv_rn(amax, qmaxf);
-  const bool nz = amax > 0.f;
-  const float rs = nz ? __frcp_rn(s) : 0.f;
-  if (part == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = nz ? s : 0.f;
-  // Codes into the staging bytes at their positions; A4 and A8 each in a loop of their own.
-  const int ib = L == 2 ? tid : L == 1 ? 256 * (tid >> 4) + (tid & 15) : 16 * tid;   // position of value 0
-  const int is = L == 2 ? 256 : L == 1 ? 16 : 1;                                       // and the stride
-  if (bits == 4) {
-#pragma unroll
-    for (int g4 = 0; g4 < 4; ++g4) {
-      const float yy[4] = {y[4 * g4], y[4 * g4 + 1], y[4 * g4 + 2], y[4 * g4 + 3]};
-      float q[4] = {0.f, 0.f, 0.f, 0.f};
-      if (nz) quant_code4(yy, s, rs, qminf, qmaxf, q);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = ib + is * (4 * g4 + j);
-        if (i < len) stg[i] = (uint8_t)e4m3_byte(q[j]);
-      }
-    }
-  } else {
-#pragma unroll
-    for (int g4 = 0; g4 < 4; ++g4) {
-      const float yy[4] = {y[4 * g4], y[4 * g4 + 1], y[4 * g4 + 2], y[4 * g4 + 3]};
-      float q[4] = {0.f, 0.f, 0.f, 0.f};
-      if (nz) quant_code4(yy, s, rs, qminf, qmaxf, q);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = ib + is * (4 * g4 + j);
-        if (i < len) {
-          uint32_t b0, b1;
-          part_code_bytes(q[j], 8, b0, b1);
-          stg[i] = (uint8_t)b0;
-          stg[kChunk + i] = (uint8_t)b1;
-        }
-      }
-    }
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 142);
-  sync();
-  // Word j of this thread, found directly from the layout: L = 2 (value e at 256 e + t),
-  // L = 1 (256 (t >> 4) + 16 e + (t & 15)), L = 0 (16 t + e).
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int i = L == 2 ? 4 * (j * kRQThreads + tid) : L == 1 ? 256 * (tid >> 4) + 4 * (j * 16 + (tid & 15)) : 16 * tid + 4 * j;
-    if (i < len)
-      part_store4(a, row, c0 + i, *reinterpret_cast<const uint32_t*>(stg + i),
-                  *reinterpret_cast<const uint32_t*>(stg + kChunk + i), err);
-  }
-  if (part == a.np - 1)   // k in [K, K_pad): zero codes
-    for (int k = K + 4 * tid; k < a.KB * 128; k += 4 * kRQThreads) part_store4(a, row, k, 0u, 0u, err);
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 143);
-}
-
-// Block slices: output slice ps of block blk (B = n L, L = 256 V), thread t owning slice
-// positions V t .. V t + V - 1.  v = sum_a (-1)^popc(ps & a) x_a (exact), then the L-point
-// butterflies: log2 V levels in registers, 5 across the lanes (shuffles), 3 across the 8
-// warps (one exchange through shared memory, groups of 8 values on 32 V threads); the
-// codes go out as words without staging.  smem as rotate_quant_part_blocks.
-template <int V, class Sync>
-__device__ __forceinline__ void rotate_quant_part_slice(const RQArgs& a, int row, int part, unsigned char* smem,
-                                                        int tid, Sync sync, long long wait_cycles, int* err) {
-  static_assert(V == 4 || V == 8, "4 or 8 values per thread");
-  constexpr int L = 256 * V;
-  constexpr int U = L / 8;   // threads of the warp-level step
-  long long* sx = reinterpret_cast<long long*>(smem);   // [L], unpadded
-  float* redf = reinterpret_cast<float*>(smem + (size_t)kChunkPadded * 8 + 2 * kChunk);
-  unsigned long long* const tr = DPTQ_TRACE_BUF();
-  (void)tr;
-  if (row >= a.rows_in) {
-    part_zero_row(a, row, part, tid, err);
-    return;
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 170);
-  const int n = a.B / L;   // parts per block: 2 or 4
-  const int ps = part % n;
-  const int k0 = (part / n) * a.B + V * tid;   // this thread's position in input slice 0
-  // debug builds: the n slices lie inside the row (site 5); a failed check reads slice 0
-  const bool in_row = DPTQ_CHECK(k0 + (n - 1) * L + V <= a.K && n <= 4, err, 5);
-  const __half* xr = a.x + (size_t)row * a.K + (in_row ? k0 : 0);
-  uint32_t raw[4][V / 2];   // the n slices' V fp16 values, all requested before any use
-#pragma unroll
-  for (int sl = 0; sl < 4; ++sl)
-    if (sl < n) {
-      if constexpr (V == 4) {
-        const uint2 w = *reinterpret_cast<const uint2*>(xr + sl * L);
-        raw[sl][0] = w.x;
-        raw[sl][1] = w.y;
-      } else {
-        const uint4 w = *reinterpret_cast<const uint4*>(xr + sl * L);
-        raw[sl][0] = w.x;
-        raw[sl][1] = w.y;
-        raw[sl][2] = w.z;
-        raw[sl][3] = w.w;
-      }
-    }
-  long long v[V];
-#pragma unroll
-  for (int i = 0; i < V; ++i) v[i] = 0;
-#pragma unroll
-  for (int sl = 0; sl < 4; ++sl)
-    if (sl < n) {
-      uint32_t sg = 0u;   // sign bits of the randomized Hadamard, one per value
-      if (a.signs != nullptr) {
-        const int8_t* sp = a.signs + k0 + sl * L;
-#pragma unroll
-        for (int i = 0; i < V; ++i) sg |= (sp[i] < 0 ? 1u : 0u) << i;
-      }
-      const bool neg = __popc(ps & sl) & 1;   // H_n[ps][sl] = -1
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        long long t = half_to_fixed(i & 1 ? raw[sl][i >> 1] >> 16 : raw[sl][i >> 1] & 0xFFFFu);
-        if ((sg >> i) & 1u) t = -t;
-        v[i] = neg ? v[i] - t : v[i] + t;
-      }
-    }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 171);
-#pragma unroll
-  for (int h = 1; h < V; h <<= 1)
-#pragma unroll
-    for (int i = 0; i < V; ++i)
-      if ((i & h) == 0) {
-        const long long p = v[i], q = v[i + h];
-        v[i] = p + q;
-        v[i + h] = p - q;
-      }
-  const int lane = tid & 31;
-#pragma unroll
-  for (int b = 0; b < 5; ++b) {
-    const bool up = (lane >> b) & 1;   // the higher position of the pair
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-      const long long o = __shfl_xor_sync(0xffffffffu, v[i], 1 << b);
-      v[i] = up ? o - v[i] : v[i] + o;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < V; i += 2) *reinterpret_cast<longlong2*>(sx + V * tid + i) = make_longlong2(v[i], v[i + 1]);
-  sync();
-  if (tid < U) {
-    long long w[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) w[k] = sx[tid + U * k];
-#pragma unroll
-    for (int h = 1; h < 8; h <<= 1)
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if ((k & h) == 0) {
-          const long long p = w[k], q = w[k + h];
-          w[k] = p + q;
-          w[k + h] = p - q;
-        }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) sx[tid + U * k] = w[k];
-  }
-  sync();
-#pragma unroll
-  for (int i = 0; i < V; i += 2) {
-    const longlong2 t = *reinterpret_cast<const longlong2*>(sx + V * tid + i);
-    v[i] = t.x;
-    v[i + 1] = t.y;
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 176);
-  long long mx = 0;
-#pragma unroll
-  for (int i = 0; i < V; ++i) {
-    const long long t = v[i] < 0 ? -v[i] : v[i];
-    mx = t > mx ? t : mx;
-  }
-  const float tmax = mx ? fixed_to_rotated(mx, a.log2B, a.c_hi, a.c_lo) : 0.f;
-  float y[V];   // exact 0 for S = 0; even or odd log2 B chosen once, outside the loop
-  if ((a.log2B & 1) == 0) {
-    const float sc = __int_as_float((127 - 24 - (a.log2B >> 1)) << 23);
-#pragma unroll
-    for (int i = 0; i < V; ++i) y[i] = __fmul_rn(ll_to_float_rn(v[i]), sc);
-  } else {
-#pragma unroll
-    for (int i = 0; i < V; ++i) y[i] = fixed_times_const(v[i], a.log2B >> 1, a.c_hi, a.c_lo);
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 140);
-  const float amax = part_row_absmax(a, row, part, tmax, redf, tid, sync, wait_cycles, err);
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 141);
-  const int bits = a.bits;
-  const float qmaxf = (float)((1 << (bits - 1)) - 1), qminf = -(float)(1 << (bits - 1));
-  const float s = __fdiv_rn(amax, qmaxf);
-  const bool nz = amax > 0.f;
-  const float rs = nz ? __frcp_rn(s) : 0.f;
-  if (part == 0 && tid == 0 && a.scales != nullptr) a.scales[row] = nz ? s : 0.f;
-  const int kout = (part / n) * a.B + ps * L + V * tid;   // first output position of this thread
-#pragma unroll
-  for (int g4 = 0; g4 < V / 4; ++g4) {
-    const float yy[4] = {y[4 * g4], y[4 * g4 + 1], y[4 * g4 + 2], y[4 * g4 + 3]};
-    float q[4] = {0.f, 0.f, 0.f, 0.f};
-    if (nz) quant_code4(yy, s, rs, qminf, qmaxf, q);
-    uint32_t w0 = 0u, w1 = 0u;
-    if (bits == 4) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w0 |= e4m3_byte(q[j]) << (8 * j);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t b0, b1;
-        part_code_bytes(q[j], 8, b0, b1);
-        w0 |= b0 << (8 * j);
-        w1 |= b1 << (8 * j);
-      }
-    }
-    part_store4(a, row, kout + 4 * g4, w0, w1, err);
-  }
-  if (tid == 0) DPTQ_TRACE_CLOCK(tr, 143);
 }
 
 }  // namespace dptq
