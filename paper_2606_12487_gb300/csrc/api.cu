@@ -350,14 +350,6 @@ bool fused_allowed() {
   return on;
 }
 
-bool l2_prefetch_allowed() {
-  static const bool on = [] {
-    const char* v = std::getenv("DPTQ_L2PF");
-    return !(v && v[0] == '0');
-  }();
-  return on;
-}
-
 // Decode grids of one CTA per whole weight tile when the tiles fit the SMs (default), or,
 // with DPTQ_DECODE_WHOLE_TILES=0, every SM with split tiles (tuning).
 bool decode_whole_tiles() {
@@ -792,11 +784,11 @@ dptq_status dptq_get_packed(dptq_handle h, void* wq_host, float* sw_host) {
         const int e = kk & 15;  // position in the 16-weight chunk
         const size_t chunk = (((size_t)(n >> 7) * h->KB + (kk >> 7)) * kWTileBytes) + ((kk & 127) >> 5) * 2048 +
                              (n & 127) * 16 + (((kk & 127) >> 4) & 1) * 8;
-        const int word = e >> 3, i = e & 3, high = (e & 7) >= 4;
-        const uint8_t byte = t[chunk + word * 4 + i];
-        const int nib = high ? (byte >> 4) & 0xF : byte & 0xF;
-        const int mag = nib & 7;
-        code[d] = (nib & 8) ? -mag : mag;
+        const int i = e & 3, high = (e & 7) >= 4;
+        const uint8_t* word = t.data() + chunk + (e >> 3) * 4;
+        const int mag = high ? (word[i] >> 4) & 7 : word[i] & 7;
+        const int neg = high ? (word[(i + 1) & 3] >> 3) & 1 : word[i] >> 7;
+        code[d] = neg ? -mag : mag;
       }
       dst[(size_t)n * (h->K / 2) + k / 2] = (uint8_t)((code[0] & 0xF) | ((code[1] & 0xF) << 4));
     }

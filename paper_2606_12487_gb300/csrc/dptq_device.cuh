@@ -147,6 +147,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// Two barriers at once: their answers come back together, where two waits in a row cost two
+// round trips to shared memory.  The first barrier's phase orders the second's (it is
+// asked again only once the first is complete).
+__device__ __forceinline__ bool mbar_wait2(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1,
+                                           volatile int* abort_flag, int* err, int code,
+                                           long long limit = kWaitTimeoutCycles) {
+  const bool r0 = mbar_try_wait(b0, p0), r1 = mbar_try_wait(b1, p1);
+  if (r0 && r1) return true;
+  return mbar_wait(b0, p0, abort_flag, err, code, limit) && mbar_wait(b1, p1, abort_flag, err, code, limit);
+}
+
 // The same wait for a whole, converged warp: every lane polls, the result is the same
 // for all lanes, and lane 0 decides a time-out.  The phase waited on must not be able to
 // advance twice while the warp polls (true for every ring here: its next phase needs an
@@ -169,6 +180,16 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
       return false;
     }
   }
+}
+
+// The same wait for two barriers at once: their answers come back together, where two
+// waits in a row cost two round trips to shared memory.
+__device__ __forceinline__ bool mbar_wait2_warp(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1,
+                                                volatile int* abort_flag, int* err, int code,
+                                                long long limit = kWaitTimeoutCycles) {
+  const bool r0 = mbar_try_wait(b0, p0), r1 = mbar_try_wait(b1, p1);
+  if (__all_sync(0xffffffffu, r0 && r1)) return true;
+  return mbar_wait_warp(b0, p0, abort_flag, err, code, limit) && mbar_wait_warp(b1, p1, abort_flag, err, code, limit);
 }
 
 // One lane of a converged warp (the lowest) gets true.  Single-thread tcgen05 and bulk
@@ -200,12 +221,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       " [%0], [%1], %2, [%3], %4;" ::"r"(smem_u32(dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
-}
-
-// Bring `bytes` of global memory at `src` into L2 without copying it anywhere (both
-// 16-byte aligned / a multiple of 16); no completion is tracked.
-__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
 // ------------------------------------------------------------------ tcgen05 / TMEM

@@ -11,7 +11,7 @@ struct dptq_linear {
   int device;
   int N, K, K_pad, KB, N_pad;
   int had_block;
-  uint8_t* wt;  // [N_pad/128][KB][4 chunks of 32 k][128 rows][16 B] sign-magnitude nibbles
+  uint8_t* wt;  // [N_pad/128][KB][4 chunks of 32 k][128 rows][16 B] sign-magnitude weights
   float* sw;    // [N_pad]
   int8_t* signs;  // randomized Hadamard diagonal [K] on the device, or null (plain block Hadamard)
 };
@@ -105,7 +105,7 @@ cudaError_t launch_policy(const PolicyArgs& a, int num_sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ GEMM
 struct GemmArgs {
-  const uint8_t* wt;   // [NTw][KB][4][128][16] packed sign-magnitude nibbles (chunk-major tiles)
+  const uint8_t* wt;   // [NTw][KB][4][128][16] packed sign-magnitude weights (chunk-major tiles)
   const uint8_t* act;  // [planes][KB][M_pad][128] E4M3, rows pre-swizzled
   const float* sa;     // [>= M] per-token scales
   const float* sw;     // [>= N] per-channel scales
@@ -128,7 +128,6 @@ struct GemmArgs {
   long long sk_iters;  // stream-K iterations (tiles after dp_tiles, times KI)
   uint32_t tmem_cols;
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
-  long long l2_prefetch;  // weight bytes past the first ring stages each CTA requests into L2 up front (0: none)
   // Fused decode launches only: the rotation + quantization of the M_pad token rows
   // (written to `act` / `sa` by the converter warps of CTAs 0, 1, ...: CTA row * rq_cpr +
   // part) and the two grid counters [rows ready, CTAs done] that order it before the GEMM
@@ -179,8 +178,6 @@ long long wait_cycles_setting();
 // for n more published token rows than any CTA publishes, so that its bounded wait runs
 // out (returns n once, then 0).
 int take_rows_shortfall();
-// Decode GEMM launches prefetch their weight share into L2 unless DPTQ_L2PF=0.
-bool l2_prefetch_allowed();
 bool decode_whole_tiles();   // DPTQ_DECODE_WHOLE_TILES=0: decode grids never shrink to one CTA per tile
 bool a8_tile128();   // DPTQ_A8_TILE128=1: A8 prefill on 128-token tiles (weights widened into shared memory)
 // Activation rows are rotated by the tensor-core kernel unless DPTQ_ROWS_KERNEL=0 (the

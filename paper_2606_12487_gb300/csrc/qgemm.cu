@@ -5,9 +5,9 @@
 //
 // sm_103a exposes no integer tcgen05 MMA, so the integers travel through FP8 E4M3,
 // where they are exact:
-//   * a weight code q in [-7, 7] is stored as a sign-magnitude nibble; the nibble
-//     placed in the low bits of a byte (sign moved to bit 7) is the E4M3 subnormal
-//     q * 2^-9, so widening is two mask-and-shift operations per four weights;
+//   * a weight code q in [-7, 7] is stored as a magnitude of three bits and a sign; a byte
+//     with the magnitude in its low bits and the sign in bit 7 is the E4M3 subnormal
+//     q * 2^-9, so widening is a mask, after a rotation for every second word;
 //   * a 4-bit activation code is an E4M3 normal number;
 //   * an 8-bit activation code c is split into c = hi + lo with hi = sign*16*(|c|>>4)
 //     and lo = sign*(|c|&15), both exact in E4M3, and both planes are multiplied into
@@ -130,14 +130,11 @@ struct Ring {
   }
 };
 
-// Widen four sign-magnitude nibbles (low halves of the bytes of w) to E4M3 subnormals.
-__device__ __forceinline__ uint32_t widen_lo(uint32_t w) {
-  return (w & 0x07070707u) | ((w << 4) & 0x80808080u);
-}
-// ... and the four high halves (whose sign bit already sits at bit 7).
-__device__ __forceinline__ uint32_t widen_hi(uint32_t w) {
-  return ((w >> 4) & 0x07070707u) | (w & 0x80808080u);
-}
+// Widen the eight weights of a packed word to E4M3 subnormals, four to a word (the packer's
+// layout: each half is one mask, the second after a rotation; half the instructions of two
+// masks and two shifts).
+__device__ __forceinline__ uint32_t widen_lo(uint32_t w) { return w & 0x87878787u; }
+__device__ __forceinline__ uint32_t widen_hi(uint32_t w) { return __funnelshift_r(w, w, 4) & 0x87878787u; }
 
 // Where the widened weights (the MMA's A operand) live: tensor memory for two-block
 // stages (decode) and for 192-token tiles, whose two accumulators (384 columns) leave
@@ -173,11 +170,10 @@ struct Smem {
 // RG != 0 (decode, two-block stages) makes the launch FUSED: it first rotates and quantizes
 // the token rows itself (RG = 1, 2 or 4 warps per Hadamard block, rotate_mma.cuh).  CTA
 // row * rq_cpr + part takes a row, or half of one of more than 8 units, with its 8 converter
-// warps, in the shared memory of the copy ring, which this CTA fills only afterwards; its
-// weight share is requested into L2 meanwhile.  The other CTAs fill their rings from the
-// start.  The rows are published on a grid counter; every activation producer waits for all
-// of them; the epilogue reads the token scales after the same point, and the last CTA to get
-// there resets the counters and the slots.
+// warps, in the shared memory of the copy ring, which this CTA fills only afterwards; the
+// other CTAs fill their rings from the start.  The rows are published on a grid counter;
+// every activation producer waits for all of them; the epilogue reads the token scales after
+// the same point, and the last CTA to get there resets the counters and the slots.
 template <int NT, int KPS, int RG>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a) {
   constexpr bool FUSED = RG != 0;
@@ -188,7 +184,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   // Two-block stages with the widened weights in tensor memory: the converter warps form
   // two groups of four (one warp per TMEM lane quarter) that take alternate stages, each
   // warp widening both k-blocks of its quarter, so that two stages convert at once.
-  constexpr bool kAltConv = kATmem && KPS == 2;
+  // (wide tiles: all eight on the same stage, a k-block per group).
+  constexpr bool kPairConv = kATmem && KPS == 2;
+  constexpr bool kAltConv = kPairConv && NT <= 64;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = a.stages;
@@ -274,44 +272,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     const uint32_t a_tx = (uint32_t)(KPS * a.planes) * act_bytes;
     const size_t plane_stride = (size_t)a.KB * a.M_pad * 128;
     const size_t kb_stride = (size_t)a.M_pad * 128;
-    // Decode launches: once the ring's first S stages are requested, the weight producer
-    // requests the rest of its CTA's share (up to a cap) into L2, so that HBM streams the
-    // weights while the ring is still full (the token rows are being rotated, or the
-    // previous kernel finishes).  Units are visited in processing order; each unit's
-    // weight range is contiguous (tile-major, k-blocks consecutive) and, with one token
-    // tile, belongs to this CTA.
-    auto prefetch_share = [&](long long skip) {   // skip: bytes fetched by the ring directly
-      if (!(wprod && leader && a.l2_prefetch > 0)) return;
-      UnitIter pit;
-      pit.init(a);
-      Unit pu;
-      long long budget = a.l2_prefetch;
-      while (budget > 0 && pit.next(pu)) {
-        const int tile_n = pu.tile / a.m_tiles;
-        const uint8_t* base = a.wt + ((size_t)tile_n * a.KB + (size_t)pu.i0 * KPS) * kWTileBytes;
-        long long len = (long long)(pu.i1 - pu.i0) * w_bytes;
-        if (skip >= len) {
-          skip -= len;
-          continue;
-        }
-        base += skip;
-        len -= skip;
-        skip = 0;
-        if (len > budget) len = budget;
-        budget -= len;
-        for (long long off = 0; off < len; off += 32768)
-          bulk_prefetch_l2(base + off, (uint32_t)(len - off < 32768 ? len - off : 32768));
-      }
-    };
     // The activation producer starts once the previous kernel has finished and, in a fused
     // launch, every token row has been quantized.
     bool ok = true;
     const bool rotates = FUSED && (int)blockIdx.x < a.rq_items;
-    if (rotates) {   // the ring's memory holds the row until it is quantized
-      prefetch_share(0);
-      __syncwarp();
+    if (rotates)   // the ring's memory holds the row until it is quantized
       ok = mbar_wait_warp(rdone, 0, abort_flag, a.err, kDevTimeoutGrid, a.wait_cycles);
-    }
     if (!wprod && ok) {
       pdl_wait();
       if constexpr (FUSED) {
@@ -372,7 +338,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
             if (DPTQ_CHECK(nt < a.n_wtiles && (it + 1) * KPS <= a.KB, a.err, 1))
               bulk_g2s(sm.wpack(s), wsrc, w_bytes, &full[s], pol_w);
             if (g < kTraceStages) DPTQ_TRACE_POINT(tr, 24 + g);
-            if (g == S - 1 && !rotates) prefetch_share((long long)S * w_bytes);
           } else {
             mbar_arrive_expect_tx(&afull[s], a_tx);
             // debug builds: the stage's token tile lies inside the operand planes (site 2)
@@ -439,12 +404,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         const bool tgm = kTraceStages > 10 && leader && gm >= 8 && gm < 11;   // stages whose steps are clocked (trace builds)
         (void)tgm;
         if (tgm) DPTQ_TRACE_CLOCK(tr, 200 + 8 * (gm - 8));
-        if (!mbar_wait_warp(&afull[s], rg.ph, abort_flag, a.err, kDevTimeoutFull, a.wait_cycles)) {
-          ok = false;
-          break;
-        }
-        if (tgm) DPTQ_TRACE_CLOCK(tr, 201 + 8 * (gm - 8));
-        if (!mbar_wait_warp(&cfull[c], rc.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
+        if (!mbar_wait2_warp(&cfull[c], rc.ph, &afull[s], rg.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -485,7 +445,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
           if (tgm) DPTQ_TRACE_CLOCK(tr, 205 + 8 * (gm - 8));
           if (gm < kTraceStages) DPTQ_TRACE_POINT(tr, 88 + gm);
         }
-        __syncwarp();
         if (tgm) DPTQ_TRACE_CLOCK(tr, 206 + 8 * (gm - 8));
         fresh = 0;
         --seg_left;
@@ -546,49 +505,40 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         // copy (stage gc - S, converted by the other group) is still in flight.  With
         // S >= CS, that copy has landed and been consumed once the MMA of stage gc - CS
         // is done.
-        if (gc >= CS && !mbar_wait(&empty[rl.s], rl.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
-          ok = false;
-          break;
-        }
-        if (tgc) DPTQ_TRACE_CLOCK(tr, 181 + 6 * (gc - 8));
-        if (!mbar_wait(&full[s], rg.ph, abort_flag, a.err, kDevTimeoutFull, a.wait_cycles)) {
+        const bool fresh = gc < CS;   // the slot's first use: only the copy is waited for
+        if (!mbar_wait2(fresh ? &full[s] : &empty[rl.s], fresh ? rg.ph : rl.ph, &full[s], rg.ph, abort_flag, a.err,
+                        kDevTimeoutConv, a.wait_cycles)) {
           ok = false;
           break;
         }
         if (tgc) DPTQ_TRACE_CLOCK(tr, 182 + 6 * (gc - 8));
         if ((kAltConv ? tid_grp == 0 : ctid == 0) && gc < kTraceStages) DPTQ_TRACE_POINT(tr, 40 + gc);
         const uint8_t* __restrict__ wp = sm.wpack(s);
-        if constexpr (kAltConv) {
+        if constexpr (kPairConv) {
           // Warp of lane quarter q widens both k-blocks of rows 32q..32q+31: each thread
           // reads its row's 2 x 64 packed bytes (4 chunks of 32 k per block) and stores
           // 2 x 32 columns of its TMEM lane.
           tc_fence_after();
           const int q = warp & 3;
           const uint8_t* src = wp + (q * 32 + lane) * 16;
-          uint4 w[8];
+          // One k-block per step, not unrolled: the loop then fits the instruction cache that
+          // the MMA issuer, on the same scheduler, also runs from.
+#pragma unroll 1
+          for (int h = kAltConv ? 0 : grp; h < (kAltConv ? 2 : grp + 1); ++h) {
+            uint4 w[4];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) w[j] = *reinterpret_cast<const uint4*>(src + (j >> 2) * kWTileBytes + (j & 3) * 2048);
-#ifdef DPTQ_TRACE
-          if (tgc) {
-            volatile uint32_t sink = w[0].x ^ w[7].w;
-            (void)sink;
-            DPTQ_TRACE_CLOCK(tr, 183 + 6 * (gc - 8));
-          }
-#endif
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
+            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(src + h * kWTileBytes + j * 2048);
             uint32_t v[32];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const uint4 ww = w[4 * h + j];
-              v[8 * j + 0] = widen_lo(ww.x);
-              v[8 * j + 1] = widen_hi(ww.x);
-              v[8 * j + 2] = widen_lo(ww.y);
-              v[8 * j + 3] = widen_hi(ww.y);
-              v[8 * j + 4] = widen_lo(ww.z);
-              v[8 * j + 5] = widen_hi(ww.z);
-              v[8 * j + 6] = widen_lo(ww.w);
-              v[8 * j + 7] = widen_hi(ww.w);
+              v[8 * j + 0] = widen_lo(w[j].x);
+              v[8 * j + 1] = widen_hi(w[j].x);
+              v[8 * j + 2] = widen_lo(w[j].y);
+              v[8 * j + 3] = widen_hi(w[j].y);
+              v[8 * j + 4] = widen_lo(w[j].z);
+              v[8 * j + 5] = widen_hi(w[j].z);
+              v[8 * j + 6] = widen_lo(w[j].w);
+              v[8 * j + 7] = widen_hi(w[j].w);
             }
             tmem_st32(tmem_base + ((uint32_t)(q * 32) << 16) + a.a_col0 + (uint32_t)((c * KPS + h) * 32), v);
           }
@@ -1109,10 +1059,6 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   if ((long long)a.sk_iters * G + G >= (1LL << 32) || tiles >= (1LL << 31)) return false;
   a.tmem_cols = cols;
   a.out_vec = 0;
-  // Decode plans (one token tile of at most 64, weights streamed once): each CTA may
-  // request up to 512 KB of its share into L2 ahead of the ring (76 MB over 152 SMs,
-  // within the 129 MB L2).
-  a.l2_prefetch = (nt <= 64 && m_tiles == 1 && l2_prefetch_allowed()) ? 512LL * 1024 : 0;
   a.rq = RQArgs{};
   a.gsync = nullptr;
   // Fused: the grid holds four CTAs per token row (padding included), or two; a launch whose

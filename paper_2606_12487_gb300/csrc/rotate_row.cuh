@@ -488,28 +488,32 @@ __device__ __forceinline__ void rotate_quant_row(const RQArgs& a, int row, unsig
         }
       }
     } else if constexpr (MODE == kRQWeights) {
-      // 16 weights -> 8 bytes.  Nibble = sign (bit 3) | magnitude (bits 0-2); word 0
-      // byte i holds k0+i (low nibble) and k0+4+i (high nibble), word 1 holds k0+8+i
-      // and k0+12+i, so that the GEMM widens a word with two masks per half.  A tile of
-      // 128 rows x 128 k is stored as 4 column chunks of 32 k, each [128 rows][16 B].
+      // 16 weights -> 8 bytes: weights k0 .. k0 + 7 in word 0, k0 + 8 .. in word 1.  Byte i of a
+      // word holds weight i (magnitude in bits 0-2, sign in bit 7) and the magnitude of weight
+      // 4 + i (bits 4-6), whose sign is bit 3 of the next byte (of byte 0 for i = 3): the word
+      // and the word rotated right by 4 then both show four sign-magnitude bytes under one
+      // mask.  A tile of 128 rows x 128 k is stored as 4 column chunks of 32 k, each
+      // [128 rows][16 B].
       uint8_t* wt = static_cast<uint8_t*>(a.out);
       const int nchunks = a.KB * 8;
       for (int ch = tid; ch < nchunks; ch += kRQThreads) {
         const int kb = ch >> 3, j = ch & 7;
         const int k0 = ch * 16;
-        uint32_t nib[16];
+        uint32_t mag[16], neg[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           const int k = k0 + e;
           int c = (nz && k < K) ? quantize(sy[k], s, rs, qmin, qmax) : 0;
           c = c < -7 ? -7 : c;   // unreachable for symmetric RTN (|W'/s| <= 7)
-          nib[e] = (c < 0 ? 8u : 0u) | (uint32_t)(c < 0 ? -c : c);
+          mag[e] = (uint32_t)(c < 0 ? -c : c);
+          neg[e] = c < 0 ? 1u : 0u;
         }
         uint32_t w0 = 0, w1 = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          w0 |= (nib[i] | (nib[4 + i] << 4)) << (8 * i);
-          w1 |= (nib[8 + i] | (nib[12 + i] << 4)) << (8 * i);
+          const int j = 8 * ((i + 1) & 3) + 3;   // sign of the second weight
+          w0 |= ((mag[i] | (neg[i] << 7) | (mag[4 + i] << 4)) << (8 * i)) | (neg[4 + i] << j);
+          w1 |= ((mag[8 + i] | (neg[8 + i] << 7) | (mag[12 + i] << 4)) << (8 * i)) | (neg[12 + i] << j);
         }
         // tile [16-byte chunk j / 2][row][16 B]: the 32 rows a warp reads side by side
         // are contiguous
