@@ -127,6 +127,7 @@ struct GemmArgs {
   int dp_tiles;        // tiles processed whole, round-robin, before the stream-K part
   long long sk_iters;  // stream-K iterations (tiles after dp_tiles, times KI)
   uint32_t tmem_cols;
+  int cl;              // CTAs of a cluster that share a weight tile's k range (1: no cluster)
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
   // Fused decode launches only: the rotation + quantization of the M_pad token rows
   // (written to `act` / `sa` by the converter warps of CTAs 0, 1, ...: CTA row * rq_cpr +

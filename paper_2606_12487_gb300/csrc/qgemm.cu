@@ -35,6 +35,7 @@
 // Work: whole tiles round-robin first (`dp_tiles`), then the remaining tiles' k-blocks
 // split evenly over the CTAs (stream-K), so every SM streams the same number of
 // weight bytes.
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
@@ -60,6 +61,7 @@ constexpr int kConvBytes = 128 * 128;   // one weight tile widened to E4M3
 constexpr int kMaxStages = 8;
 constexpr int kMaxConvSlots = 4;
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in dynamic shared memory per CTA
+constexpr int kCluster = 4;   // CTAs of a cluster that split a weight tile
 constexpr int kBarrierBytes = 2048;   // barriers and flags, token scales (tiles <= 64), output transpose (1 KB)
 
 struct Unit {
@@ -167,6 +169,81 @@ struct Smem {
   __device__ __forceinline__ uint8_t* end(int S) const { return slot(S); }
 };
 
+// A tile whose k range the kCluster CTAs of a cluster share: CTA r finishes tokens
+// r NT / 4 .. of it.  Each CTA sends the others their tokens' partial sums (exact integers in
+// fp32: their order does not matter) straight into their shared memory and adds what it
+// receives to its own accumulators: one store and one barrier wait, where partial sums in
+// global memory take reductions, a fence, an atomic and a read back (LLaMA-2-7B o at
+// M = 32: 3.9 us from the last MMA to the exit).  Run by the four epilogue warps; `tb`: the
+// warp's accumulators; n: this thread's channel.
+template <int NT, int KPS>
+__device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT, KPS>& sm, uint64_t* bars, uint64_t* xbar,
+                                               __half* xpose, const float* sa_sh, uint32_t tb, int n, int nt, int q,
+                                               int lane, volatile int* abort_flag) {
+  constexpr int TQ = NT / kCluster;          // tokens a CTA finishes: 4, 8 or 16
+  float* recv = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kBarrierBytes);   // [3][TQ / 4][128][4]
+  const uint32_t rank = blockIdx.x % kCluster;
+  const int ch = q * 32 + lane;
+  cluster_wait();   // the others' barriers are initialized
+  float own[TQ];
+#pragma unroll
+  for (int c0 = 0; c0 < NT; c0 += 16) {
+    uint32_t r[16];
+    tmem_ld16(tb + (uint32_t)c0, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {            // tokens c0 + 4 j .. + 3
+      const uint32_t dst = (uint32_t)((c0 + 4 * j) / TQ);
+      const int g = ((c0 + 4 * j) % TQ) / 4;
+      if (dst == rank) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) own[4 * g + i] = __uint_as_float(r[4 * j + i]);
+      } else {
+        const uint32_t from = rank - (rank > dst ? 1u : 0u);   // this CTA's place among the senders
+        const uint32_t at = smem_u32(recv + ((from * (TQ / 4) + g) * 128 + ch) * 4);
+        st_async_v4(cluster_map(at, dst), cluster_map(smem_u32(xbar), dst), r[4 * j], r[4 * j + 1], r[4 * j + 2],
+                    r[4 * j + 3]);
+      }
+    }
+  }
+  tc_fence_before();
+  const float swn = n < a.N ? a.sw[n] : 0.f;
+  if (!mbar_wait(xbar, 0, abort_flag, a.err, kDevTimeoutTmemFull, a.wait_cycles)) return false;
+  const int t0 = (int)rank * TQ;
+#pragma unroll
+  for (int g = 0; g < TQ / 4; ++g) {
+    float f[4] = {own[4 * g], own[4 * g + 1], own[4 * g + 2], own[4 * g + 3]};
+#pragma unroll
+    for (int k = 0; k < kCluster - 1; ++k) {
+      const float4 p = *reinterpret_cast<const float4*>(recv + ((k * (TQ / 4) + g) * 128 + ch) * 4);
+      f[0] += p.x;
+      f[1] += p.y;
+      f[2] += p.z;
+      f[3] += p.w;
+    }
+    const int m0 = t0 + 4 * g;
+    __half* xw = xpose + q * 128;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float v = f[i] * 512.f;   // fp32(acc), exact
+      if (a.acc_out != nullptr && n < a.N && m0 + i < a.M) a.acc_out[(size_t)(m0 + i) * a.N + n] = __float2int_rn(v);
+      const __half h = __float2half_rn(__fmul_rn(__fmul_rn(v, sa_sh[m0 + i]), swn));
+      if (a.out_vec)
+        xw[i * 32 + lane] = h;
+      else if (n < a.N && m0 + i < a.M)
+        a.out[(size_t)(m0 + i) * a.N + n] = h;
+    }
+    if (a.out_vec) {   // 4 tokens x 32 channels through shared memory, 8 bytes a lane
+      __syncwarp();
+      const uint2 val = *reinterpret_cast<const uint2*>(xw + (lane >> 3) * 32 + (lane & 7) * 4);
+      __syncwarp();
+      const int m = m0 + (lane >> 3), nn = nt * 128 + q * 32 + (lane & 7) * 4;
+      if (m < a.M && nn < a.N) *reinterpret_cast<uint2*>(a.out + (size_t)m * a.N + nn) = val;
+    }
+  }
+  return true;
+}
+
 // RG != 0 (decode, two-block stages) makes the launch FUSED: it first rotates and quantizes
 // the token rows itself (RG = 1, 2 or 4 warps per Hadamard block, rotate_mma.cuh).  CTA
 // row * rq_cpr + part takes a row, or half of one of more than 8 units, with its 8 converter
@@ -187,6 +264,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   // (wide tiles: all eight on the same stage, a k-block per group).
   constexpr bool kPairConv = kATmem && KPS == 2;
   constexpr bool kAltConv = kPairConv && NT <= 64;
+  // Clusters of kCluster CTAs, each with a quarter of a weight tile's k range (small N).
+  constexpr bool kClusterTiles = NT <= 64 && KPS == 2;
+  constexpr uint32_t kXchBytes = (kCluster - 1) * (NT / kCluster) * 128 * 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = a.stages;
@@ -203,7 +283,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   uint64_t* esync = drain + 1;   // epilogue-group barrier (4 warps), bounded waits
   uint64_t* aready = esync + 1;  // fused: all token rows are quantized (producer -> epilogue)
   uint64_t* rdone = aready + 1;  // fused: this CTA's row is quantized, the ring's memory is free
-  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(rdone + 1);
+  uint64_t* xbar = rdone + 1;    // cluster: the other CTAs' partial sums landed
+  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(xbar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_sh + 1);
   volatile int* flags = reinterpret_cast<volatile int*>(tmem_base_sh + 2);   // epilogue: 2 units x 2
   float* sa_sh = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);   // token scales (NT <= 64)
@@ -233,6 +314,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     mbar_init(esync, kNumEpiWarps);
     mbar_init(aready, 1);
     mbar_init(rdone, 1);
+    mbar_init(xbar, 1);
     if (FUSED) rot_sh[16] = 0u;
     *abort_flag = 0;
     for (int i = 0; i < 4; ++i) flags[i] = 0;
@@ -245,6 +327,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  const bool clustered = kClusterTiles && a.cl > 1;
+  if (clustered) {
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(xbar, kXchBytes);
+    cluster_arrive();   // this CTA's barrier may be counted on by the others
+  }
   const uint32_t tmem_base = *tmem_base_sh;
   if (threadIdx.x == 0) DPTQ_TRACE_POINT(tr, 1);
   pdl_launch_dependents();
@@ -252,6 +339,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   UnitIter iter;
   iter.init(a);
   Unit un;
+  bool cluster_waited = false;   // this thread has waited for the cluster's first barrier
 
   if (warp == 0 || warp == kActWarp) {
     // ------------------------------------------------------------ producers
@@ -678,6 +766,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       if (!mbar_wait(&tfull[b], tpar, abort_flag, a.err, kDevTimeoutTmemFull, a.wait_cycles)) break;
       if (etid == 0 && u < 4) DPTQ_TRACE_POINT(tr, 104 + u);
       tc_fence_after();
+      if constexpr (kClusterTiles) {
+        if (clustered) {
+          epi_ok = cluster_finish<NT, KPS>(a, sm, bars, xbar, xpose, sa_sh, tmem_base + lane_base + (uint32_t)(b * NT), n,
+                                           nt, q, lane, abort_flag);
+          cluster_waited = true;
+          break;
+        }
+      }
       const int nseg = (un.i1 - 1) / a.seg_iters - un.i0 / a.seg_iters + 1;
       const uint32_t tb = tmem_base + lane_base + (uint32_t)(b * NT * a.segs);
       // debug builds: a split tile's slot is one of the grid's (site 3)
@@ -917,6 +1013,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     if (etid == 0) DPTQ_TRACE_VALUE(tr, 122, u);
   }
 
+  if (clustered) {
+    // No CTA leaves while another may still store into its shared memory.  (A CTA that has
+    // received everything knows that; after an abort, stores may be on their way.)
+    if (*abort_flag) __nanosleep(20000);
+    if (!cluster_waited) cluster_wait();
+    cluster_arrive();
+    cluster_wait();
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -991,7 +1095,9 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   // A fused launch needs two-block stages (weights widened into TMEM) and a ring that holds
   // the eight units of a row's rotation.
   if (fused && (kps != 2 || nt > 64)) return false;
-  auto smem_total = [&](int st) { return smem_for(nt, kps, st, planes, smem_conv); };
+  // Decode tiles may be finished by clusters, which receive partial sums in shared memory.
+  const int xch = nt <= 64 && kps == 2 && segs == 1 ? (kCluster - 1) * (nt / kCluster) * 128 * 4 : 0;
+  auto smem_total = [&](int st) { return smem_for(nt, kps, st, planes, smem_conv) + xch; };
   int stages = kMaxStages;
   while (stages > 2 && smem_total(stages) > kSmemLimit) --stages;
   if (smem_total(stages) > kSmemLimit) return false;
@@ -1031,6 +1137,9 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   }
   long long dp = 0;
   if (tiles >= 2LL * G) dp = (tiles / G - 1) * G;
+
+  // Every tile split evenly over four CTAs: a cluster finishes it.
+  a.cl = xch > 0 && m_tiles == 1 && dp == 0 && G == kCluster * tiles ? kCluster : 1;
 
   plan.fused = fused;
   plan.a_tmem = a_tmem;
@@ -1102,12 +1211,44 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
   cfg.blockDim = dim3(kGemmThreads);
   cfg.dynamicSmemBytes = (size_t)plan.smem_bytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (pdl && pdl_allowed()) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = (pdl && pdl_allowed()) ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RG>, plan.args);
+  GemmArgs args = plan.args;
+  if (args.cl > 1) {
+    cudaLaunchAttribute* c = &attr[n];
+    c->id = cudaLaunchAttributeClusterDimension;
+    c->val.clusterDim.x = (unsigned)args.cl;
+    c->val.clusterDim.y = 1;
+    c->val.clusterDim.z = 1;
+    // All CTAs have to be resident at once (a fused launch's wait for one another's rows).
+    // Asked once per kernel and device, for the largest shared memory.
+    static std::atomic<int> most[64];   // resident clusters + 1 (0: not asked yet)
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int m = dev < 64 ? most[dev].load() : 1;
+    if (m == 0) {
+      cudaLaunchConfig_t probe = cfg;
+      probe.dynamicSmemBytes = kSmemLimit;
+      cudaLaunchAttribute only = *c;
+      probe.attrs = &only;
+      probe.numAttrs = 1;
+      e = cudaOccupancyMaxActiveClusters(&m, qgemm_kernel<NT, KPS, RG>, &probe);
+      if (e != cudaSuccess) return e;
+      most[dev].store(++m);
+    }
+    if ((m - 1) * args.cl >= plan.grid)
+      ++n;
+    else
+      args.cl = 1;   // the tiles' parts meet in global memory instead
+  }
+  cfg.numAttrs = (unsigned)n;
+  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RG>, args);
 }
 
 cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
