@@ -763,6 +763,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         if (!epi_sync()) break;
         sa_mt = mt;
       }
+      // Split tile: whether every other contributor is already in is asked while the MMAs
+      // still run, and once more after them if not.
+      volatile int* const flag = flags + 2 * (u & 1);   // [0]: all others in, [1]: last
+      const bool split = un.slot >= 0 && !clustered;
+      if (split) {
+        if (etid == 0) *flag = ld_acquire_gpu(a.counters + un.slot) == (uint32_t)(un.contributors - 1);
+        if (!epi_sync()) break;
+      }
       if (!mbar_wait(&tfull[b], tpar, abort_flag, a.err, kDevTimeoutTmemFull, a.wait_cycles)) break;
       if (etid == 0 && u < 4) DPTQ_TRACE_POINT(tr, 104 + u);
       tc_fence_after();
@@ -782,12 +790,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       // Split tile.  If every other contributor has already added its part to the slot,
       // this CTA finishes the tile straight from its accumulators (slot + own part);
       // otherwise it adds its part and the last contributor to arrive finishes.
-      volatile int* const flag = flags + 2 * (u & 1);   // [0]: all others in, [1]: last
       bool finish = wsl == nullptr;
       if (wsl != nullptr) {
-        if (etid == 0) *flag = ld_acquire_gpu(a.counters + un.slot) == (uint32_t)(un.contributors - 1);
-        if (!epi_sync()) break;
         finish = *flag != 0;
+        if (!finish) {
+          if (!epi_sync()) break;   // every warp has read the early answer
+          if (etid == 0) *flag = ld_acquire_gpu(a.counters + un.slot) == (uint32_t)(un.contributors - 1);
+          if (!epi_sync()) break;
+          finish = *flag != 0;
+        }
         if (etid == 0) DPTQ_TRACE_POINT(tr, 3);
       }
       // Output of 16 tokens of this thread's channel.  With a 16-byte aligned `out`, each
