@@ -1,0 +1,74 @@
+"""Edges of the KV4 quantizer's and the policy's packed arithmetic: NaN and infinities (no
+value disturbs its neighbours in a word), ties, ragged group counts, tiny and infinite
+scales."""
+import numpy as np
+import pytest
+
+import parity
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_12487_gb300 import dptq
+    dptq.load()
+    return dptq
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 128), (3, 128), (5, 640), (257, 1024)])
+def test_kv4_ties_and_non_finite_values(dp, orc, rows, cols):
+    rng = np.random.default_rng(rows + cols)
+    x = (rng.integers(-14, 15, (rows, cols)) * 0.5).astype(np.float16)   # half the values tie
+    x[:, ::128] = 7.0                                                    # s = 1
+    x[0, :128] = 0
+    x[-1, 64:128] *= np.float16(2.0 ** -20)
+    c_ref, s_ref = orc.kv4_quantize(x, 128)
+    bad = x.copy()
+    bad[-1, 5], bad[-1, 77] = np.nan, -np.nan
+    for src in (x, bad):
+        codes = torch.empty((rows, cols // 2), dtype=torch.uint8, device="cuda")
+        sc = torch.empty((rows, cols // 128), dtype=torch.float32, device="cuda")
+        dp.dptq_kv4_quantize(torch.from_numpy(src).cuda(), 128, codes, sc)
+        c = parity.unpack_public_a4(codes.cpu().numpy(), cols)
+        want = np.where(np.isnan(src), -1, c_ref)
+        assert np.array_equal(c, want) and np.array_equal(sc.cpu().numpy(), s_ref)
+    # an infinite value: infinite scale, code -1 for it and 0 for the other values of its group
+    inf = x.copy()
+    inf[-1, 9] = np.inf
+    dp.dptq_kv4_quantize(torch.from_numpy(inf).cuda(), 128, codes, sc)
+    c = parity.unpack_public_a4(codes.cpu().numpy(), cols)
+    assert np.isinf(sc.cpu().numpy()[-1, 0]) and c[-1, 9] == -1 and np.all(np.delete(c[-1, :128], 9) == 0)
+    assert np.array_equal(c[-1, 128:], c_ref[-1, 128:]) and np.array_equal(c[:-1], c_ref[:-1])
+
+
+@pytest.mark.parametrize("d", [4, 1028, 4096])
+@pytest.mark.parametrize("bits", [4, 8])
+def test_policy_ties_tiny_and_infinite_values(dp, orc, d, bits):
+    L, T = 4, 9
+    rng = np.random.default_rng(d + bits)
+    x = (rng.integers(-14, 15, (L, T, d)) * 0.5).astype(np.float32)
+    dx = (rng.integers(-3, 4, (L, T, d)) * 0.25).astype(np.float32)
+    x[1] *= np.float32(1e-39)                       # subnormal sums: the reciprocal overflows
+    dx[1] *= np.float32(1e-39)
+    x[2] += rng.standard_normal((T, d)).astype(np.float32)
+    ref = [orc.residual_stats(x[l], dx[l], bits, 1e-6) for l in range(L)]
+    jr = torch.empty((L,), dtype=torch.float64, device="cuda")
+    snr = torch.empty((L,), dtype=torch.float64, device="cuda")
+    mask = torch.empty((L,), dtype=torch.uint8, device="cuda")
+    dp.dptq_sensitivity_policy(torch.from_numpy(x).cuda(), torch.from_numpy(dx).cuda(), bits, 1e-6, 0.1, 20.0, jr, snr,
+                               mask)
+    for l in (0, 2, 3):
+        assert abs(jr[l].item() - ref[l][0]) <= 1e-5 * abs(ref[l][0]) and abs(snr[l].item() - ref[l][1]) <= 1e-3
+    # an infinite update: the scale is infinite, inf * 0 of the finite values' codes is NaN, and so
+    # is its layer's SNR (IEEE, term by term); the other layers keep theirs
+    dx[3, 2, 1] = np.inf
+    before = snr.clone()
+    dp.dptq_sensitivity_policy(torch.from_numpy(x).cuda(), torch.from_numpy(dx).cuda(), bits, 1e-6, 0.1, 20.0, jr, snr,
+                               mask)
+    assert np.isinf(jr[3].item()) and np.isnan(snr[3].item())
+    assert np.allclose(snr[:3].cpu().numpy(), before[:3].cpu().numpy(), rtol=1e-12, equal_nan=True)
+    dp.dptq_last_device_error()
