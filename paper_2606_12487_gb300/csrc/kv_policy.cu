@@ -301,7 +301,10 @@ __global__ void __launch_bounds__(kPolThreads) policy_stats_kernel(const PolicyA
 // 2^-24).  Thread 0 records each finished token's three sums; every 32 tokens the lanes
 // of warp 0 form the tokens' JR and SNR terms in parallel (fp32; the fp64 unit of this
 // GPU is far slower) and add them per layer to the fp64 outputs, one atomic per layer.
-constexpr int kPolStages = 3;
+// Two stages: three CTAs an SM, whose barriers then overlap (32 layers x 512 tokens x 4096:
+// 97 us; three stages, two CTAs: 115 us; 384 or 512 threads a CTA: 114, 135 us).
+constexpr int kPolStages = 2;
+constexpr int kPolStagedThreads = 256;
 constexpr int kPolMaxStagedD = 4096;
 
 // Warp 0, converged: token i of the batch (i < nb, first item `item0`) has its sums in
@@ -335,10 +338,10 @@ __device__ __forceinline__ void pol_batch(const PolicyArgs& a, const float (*tok
   }
 }
 
-__global__ void __launch_bounds__(kPolThreads) policy_stats_staged_kernel(const PolicyArgs a) {
+__global__ void __launch_bounds__(kPolStagedThreads) policy_stats_staged_kernel(const PolicyArgs a) {
   extern __shared__ __align__(128) uint8_t pol_smem[];
   __shared__ uint64_t full[kPolStages];
-  __shared__ float part[2][4][kPolThreads / 32];   // [iteration parity][amax, |x|^2, |dx|^2, |err|^2][warp]
+  __shared__ float part[2][4][kPolStagedThreads / 32];   // [iteration parity][amax, |x|^2, |dx|^2, |err|^2][warp]
   __shared__ float tok[32][3];                      // finished tokens' |x|^2, |dx|^2, |err|^2
   __shared__ int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -377,48 +380,74 @@ __global__ void __launch_bounds__(kPolThreads) policy_stats_staged_kernel(const 
     if (j >= 1) {   // pass 2 of token j - 1
       const float* xs = reinterpret_cast<const float*>(pol_smem + (size_t)((j - 1) % kPolStages) * stage_bytes);
       const float* ds = xs + a.d;
+      const uint64_t nr2 = f2_pack(-r, -r), s2 = f2_pack(s, s), bias2 = f2_pack(12582912.f, 12582912.f), zero2 = 0u;
+      const bool fin = fmaxf(s, r) < __int_as_float(0x7F800000);   // both finite
+      uint64_t ne2 = 0u;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = 4 * (tid + kPolThreads * i);
+      for (int i = 0; i < kPolMaxStagedD / (4 * kPolStagedThreads); ++i) {
+        const int k = 4 * (tid + kPolStagedThreads * i);
         if (k < a.d) {
-          const float4 xv = *reinterpret_cast<const float4*>(xs + k);
-          const float4 dv = *reinterpret_cast<const float4*>(ds + k);
-          const float xe[4] = {xv.x, xv.y, xv.z, xv.w}, de[4] = {dv.x, dv.y, dv.z, dv.w};
-          float u[4], c[4] = {0.f, 0.f, 0.f, 0.f};
+          const ulonglong2 xp = *reinterpret_cast<const ulonglong2*>(xs + k), dp = *reinterpret_cast<const ulonglong2*>(ds + k);
+          const uint64_t x2[2] = {xp.x, xp.y}, d2[2] = {dp.x, dp.y};
+          uint64_t u2[2], c2[2];
+          float dm = 0.f;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) u[e] = __fadd_rn(xe[e], de[e]);
-          if (nzs) quant_code4(u, s, r, qminf, qmaxf, c);
+          for (int h = 0; h < 2; ++h) {
+            u2[h] = f2_add(x2[h], d2[h]);
+            c2[h] = f2_sub(bias2, f2_fma(u2[h], nr2, bias2));   // rint(u r), +0 for zero
+            float m0, m1;
+            f2_unpack(f2_fma(u2[h], nr2, c2[h]), m0, m1);
+            dm = fmaxf(dm, fmaxf(fabsf(m0), fabsf(m1)));
+          }
+          if (__any_sync(__activemask(), dm >= 0.5f - 0x1p-15f) || !fin) {   // near a tie, or an infinite scale or reciprocal
+            float u[4], c[4] = {0.f, 0.f, 0.f, 0.f};
+            f2_unpack(u2[0], u[0], u[1]);
+            f2_unpack(u2[1], u[2], u[3]);
+            if (nzs) quant_code4(u, s, r, qminf, qmaxf, c);
+            c2[0] = f2_pack(c[0], c[1]);
+            c2[1] = f2_pack(c[2], c[3]);
+          }
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float bv = __fsub_rn(u[e], xe[e]);
-            const float av = __fsub_rn(u[e], bv);
-            const float res = __fadd_rn(__fsub_rn(xe[e], av), __fsub_rn(de[e], bv));   // x + dx - u, exact
-            const float err = __fsub_rn(__fmaf_rn(s, c[e], -u[e]), res);
-            ne = __fmaf_rn(err, err, ne);
+          for (int h = 0; h < 2; ++h) {
+            const uint64_t bv = f2_sub(u2[h], x2[h]);
+            const uint64_t av = f2_sub(u2[h], bv);
+            const uint64_t res = f2_add(f2_sub(x2[h], av), f2_sub(d2[h], bv));   // x + dx - u, exact
+            const uint64_t err = f2_sub(f2_fma(s2, c2[h], f2_sub(zero2, u2[h])), res);
+            ne2 = f2_fma(err, err, ne2);
           }
         }
       }
+      float n0, n1;
+      f2_unpack(ne2, n0, n1);
+      ne = n0 + n1;
     }
     if (j < cnt) {   // pass 1 of token j
       const int st = j % kPolStages;
       if (mbar_wait_warp(&full[st], (uint32_t)(j / kPolStages) & 1u, &abort_flag, a.err, kDevTimeoutFull)) {
         const float* xs = reinterpret_cast<const float*>(pol_smem + (size_t)st * stage_bytes);
         const float* ds = xs + a.d;
+        uint64_t nx2 = 0u, nd2 = 0u;   // two sums each, on packed pairs
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k = 4 * (tid + kPolThreads * i);
+        for (int i = 0; i < kPolMaxStagedD / (4 * kPolStagedThreads); ++i) {
+          const int k = 4 * (tid + kPolStagedThreads * i);
           if (k < a.d) {
-            const float4 xv = *reinterpret_cast<const float4*>(xs + k);
-            const float4 dv = *reinterpret_cast<const float4*>(ds + k);
-            const float xe[4] = {xv.x, xv.y, xv.z, xv.w}, de[4] = {dv.x, dv.y, dv.z, dv.w};
+            const ulonglong2 xp = *reinterpret_cast<const ulonglong2*>(xs + k), dp = *reinterpret_cast<const ulonglong2*>(ds + k);
+            const uint64_t x2[2] = {xp.x, xp.y}, d2[2] = {dp.x, dp.y};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              nx = __fmaf_rn(xe[e], xe[e], nx);
-              nd = __fmaf_rn(de[e], de[e], nd);
-              am = fmaxf(am, fabsf(__fadd_rn(xe[e], de[e])));
+            for (int h = 0; h < 2; ++h) {
+              nx2 = f2_fma(x2[h], x2[h], nx2);
+              nd2 = f2_fma(d2[h], d2[h], nd2);
+              float u0, u1;
+              f2_unpack(f2_add(x2[h], d2[h]), u0, u1);
+              am = fmaxf(am, fmaxf(fabsf(u0), fabsf(u1)));
             }
           }
         }
+        float n0, n1;
+        f2_unpack(nx2, n0, n1);
+        nx = n0 + n1;
+        f2_unpack(nd2, n0, n1);
+        nd = n0 + n1;
       }
     }
 #pragma unroll
@@ -443,7 +472,7 @@ __global__ void __launch_bounds__(kPolThreads) policy_stats_staged_kernel(const 
     }
     float amax = part[j & 1][0][0];
 #pragma unroll
-    for (int w = 1; w < kPolThreads / 32; ++w) amax = fmaxf(amax, part[j & 1][0][w]);
+    for (int w = 1; w < kPolStagedThreads / 32; ++w) amax = fmaxf(amax, part[j & 1][0][w]);
     s = __fdiv_rn(amax, qmaxf);
     nzs = amax > 0.f;
     r = nzs ? __frcp_rn(s) : 0.f;
@@ -451,7 +480,7 @@ __global__ void __launch_bounds__(kPolThreads) policy_stats_staged_kernel(const 
       if (lane == 0) {
         float sx = 0.f, sd = 0.f, se = 0.f;
 #pragma unroll
-        for (int w = 0; w < kPolThreads / 32; ++w) {
+        for (int w = 0; w < kPolStagedThreads / 32; ++w) {
           sx += part[j & 1][1][w];
           sd += part[j & 1][2][w];
           se += part[j & 1][3][w];
@@ -504,12 +533,12 @@ cudaError_t launch_policy(const PolicyArgs& a, int num_sms, cudaStream_t s) {
     e = ensure_max_dyn_smem(policy_stats_staged_kernel);
     int per_sm = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, policy_stats_staged_kernel, kPolThreads, smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, policy_stats_staged_kernel, kPolStagedThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     long long blocks = (long long)num_sms * per_sm;
     if (blocks > items) blocks = items;
-    policy_stats_staged_kernel<<<(unsigned)blocks, kPolThreads, smem, s>>>(a);
+    policy_stats_staged_kernel<<<(unsigned)blocks, kPolStagedThreads, smem, s>>>(a);
   } else {
     long long blocks = items < (long long)num_sms * 8 ? items : (long long)num_sms * 8;
     if (blocks < 1) blocks = 1;
