@@ -589,7 +589,7 @@ dptq_status prepare_qlinear(dptq_handle h, int M, int bits, cudaStream_t s, int*
   if (st != DPTQ_OK) return st;
   if (M == 0) return DPTQ_OK;
   if ((st = ensure_scratch(*dev, 0, 0, s, sc)) != DPTQ_OK) return st;
-  if (!plan_gemm(M, h->N, h->K_pad, bits, (*sc)->num_sms, *plan)) return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan");
+  if (!plan_launch(M, h->N, h->K_pad, bits, (*sc)->num_sms, *plan)) return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan");
   const int planes = bits == 8 ? 2 : 1;
   return ensure_scratch(*dev, (size_t)planes * h->K_pad * plan->M_pad, plan->M_pad, s, sc);
 }
@@ -676,7 +676,7 @@ dptq_status dptq_qgemm_codes(dptq_handle h, const void* codes, const float* scal
   Scratch* sc = nullptr;
   if ((st = ensure_scratch(dev, 0, 0, s, &sc)) != DPTQ_OK) return st;
   GemmPlan plan;
-  if (!plan_gemm(M, h->N, h->K_pad, bits, sc->num_sms, plan)) return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan");
+  if (!plan_launch(M, h->N, h->K_pad, bits, sc->num_sms, plan)) return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan");
   const int planes = bits == 8 ? 2 : 1;
   if ((st = ensure_scratch(dev, (size_t)planes * h->K_pad * plan.M_pad, 0, s, &sc)) != DPTQ_OK) return st;
   CodesArgs c{};
@@ -731,20 +731,42 @@ dptq_status dptq_sensitivity_policy(const float* x, const float* dx, int L, int 
   return DPTQ_OK;
 }
 
-dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused, int* info, int info_len) {
+namespace {
+void write_plan(const GemmPlan& plan, int* info, int len) {
+  const GemmArgs& g = plan.args;
+  const long long sk = g.sk_iters;
+  const int v[DPTQ_LAUNCH_PLAN_LEN] = {plan.nt, plan.kps, plan.M_pad, plan.grid, plan.smem_bytes, g.stages,
+                                       g.conv_slots, plan.a_tmem ? 1 : 0, g.nbuf, g.segs, g.seg_iters,
+                                       (int)g.tmem_cols, (int)g.a_col0, g.KI, g.n_wtiles, g.m_tiles, g.dp_tiles,
+                                       sk > 0x7fffffffLL ? 0x7fffffff : (int)sk, g.rq_np, plan.fused ? 1 : 0,
+                                       g.sk_ctas, g.cl};
+  for (int i = 0; i < len; ++i) info[i] = v[i];
+}
+dptq_status check_plan_args(int M, int N, int K, int bits, int num_sms, const int* info, int info_len, int want) {
   if (M < 1 || N < 1 || K < 1 || num_sms < 1) return fail(DPTQ_ERR_INVALID_ARG, "sizes must be >= 1");
   if (bits != 4 && bits != 8) return fail(DPTQ_ERR_INVALID_ARG, "bits must be 4 or 8");
-  if (info == nullptr || info_len < DPTQ_PLAN_INFO_LEN) return fail(DPTQ_ERR_INVALID_ARG, "info too short");
+  if (info == nullptr || info_len < want) return fail(DPTQ_ERR_INVALID_ARG, "info too short");
+  return DPTQ_OK;
+}
+}  // namespace
+
+dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused, int* info, int info_len) {
+  const dptq_status st = check_plan_args(M, N, K, bits, num_sms, info, info_len, DPTQ_PLAN_INFO_LEN);
+  if (st != DPTQ_OK) return st;
   GemmPlan plan{};
   if (!plan_gemm(M, N, round_up(K, kKBlock), bits, num_sms, plan, fused != 0))
     return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
-  const GemmArgs& g = plan.args;
-  const long long sk = g.sk_iters;
-  const int v[DPTQ_PLAN_INFO_LEN] = {plan.nt, plan.kps, plan.M_pad, plan.grid, plan.smem_bytes, g.stages,
-                                     g.conv_slots, plan.a_tmem ? 1 : 0, g.nbuf, g.segs, g.seg_iters,
-                                     (int)g.tmem_cols, (int)g.a_col0, g.KI, g.n_wtiles, g.m_tiles, g.dp_tiles,
-                                     sk > 0x7fffffffLL ? 0x7fffffff : (int)sk, g.rq_np, plan.fused ? 1 : 0};
-  for (int i = 0; i < DPTQ_PLAN_INFO_LEN; ++i) info[i] = v[i];
+  write_plan(plan, info, DPTQ_PLAN_INFO_LEN);
+  return DPTQ_OK;
+}
+
+dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int* info, int info_len) {
+  const dptq_status st = check_plan_args(M, N, K, bits, num_sms, info, info_len, DPTQ_LAUNCH_PLAN_LEN);
+  if (st != DPTQ_OK) return st;
+  GemmPlan plan{};
+  if (!plan_launch(M, N, round_up(K, kKBlock), bits, num_sms, plan))
+    return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
+  write_plan(plan, info, DPTQ_LAUNCH_PLAN_LEN);
   return DPTQ_OK;
 }
 

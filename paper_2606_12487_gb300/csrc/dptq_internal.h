@@ -126,6 +126,7 @@ struct GemmArgs {
   uint32_t a_col0;     // first TMEM column of the widened-weight slots (A operand in TMEM)
   int dp_tiles;        // tiles processed whole, round-robin, before the stream-K part
   long long sk_iters;  // stream-K iterations (tiles after dp_tiles, times KI)
+  int sk_ctas;         // CTAs that share them evenly (as many as tiles: whole tiles)
   uint32_t tmem_cols;
   int cl;              // CTAs of a cluster that share a weight tile's k range (1: no cluster)
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
@@ -151,6 +152,7 @@ struct GemmPlan {
   int M_pad;
   int grid;
   int smem_bytes;
+  double cost;     // estimated microseconds (more than 64 tokens; 0 otherwise)
   GemmArgs args;
 };
 
@@ -159,6 +161,9 @@ struct GemmPlan {
 // `fused` plans the decode kernel that rotates and quantizes the rows itself: two k-blocks
 // per stage; false if it does not fit.
 bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused = false);
+// The plan of a two-launch call: plan_gemm's, or for more than 64 tokens 64-token tiles on the
+// same operand planes where they are estimated to be faster.
+bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan);
 // Warps that share a Hadamard block of a row in the tensor-core rotation (1, 2 or 4; K, B and
 // a power-of-two tail).
 int rotate_group(int K, int B, int tail);

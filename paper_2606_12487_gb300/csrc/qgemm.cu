@@ -77,10 +77,10 @@ struct Unit {
 // checks this); 32-bit divisions keep the per-unit cost low.
 struct UnitIter {
   uint32_t cta, G, KI, dp_tiles, dp_next;
-  uint32_t sk_iters, it, it_end;
+  uint32_t skG, sk_iters, it, it_end;   // the stream-K part: CTAs that share it, its iterations
 
-  __device__ __forceinline__ uint32_t sk_begin(uint32_t c) const { return (c * sk_iters) / G; }
-  __device__ __forceinline__ uint32_t cta_of(uint32_t i) const { return ((i + 1) * G - 1) / sk_iters; }
+  __device__ __forceinline__ uint32_t sk_begin(uint32_t c) const { return (c * sk_iters) / skG; }
+  __device__ __forceinline__ uint32_t cta_of(uint32_t i) const { return ((i + 1) * skG - 1) / sk_iters; }
   __device__ __forceinline__ void init(const GemmArgs& a) {
     cta = blockIdx.x;
     G = gridDim.x;
@@ -88,8 +88,10 @@ struct UnitIter {
     dp_tiles = (uint32_t)a.dp_tiles;
     dp_next = cta;
     sk_iters = (uint32_t)a.sk_iters;
-    it = sk_iters > 0 ? sk_begin(cta) : 0;
-    it_end = sk_iters > 0 ? sk_begin(cta + 1) : 0;
+    skG = (uint32_t)a.sk_ctas;
+    const bool shares = sk_iters > 0 && cta < skG;
+    it = shares ? sk_begin(cta) : 0;
+    it_end = shares ? sk_begin(cta + 1) : 0;
   }
   __device__ __forceinline__ bool next(Unit& u) {
     if (dp_next < dp_tiles) {
@@ -1062,11 +1064,33 @@ static int smem_for(int nt, int kps, int stages, int planes, int conv_slots) {
   return 1024 + conv_slots * kps * kConvBytes + stages * kps * (planes * nt * 128 + kWTileBytes) + kBarrierBytes;
 }
 
-bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused) {
+// Launch time of a GEMM of more than 64 tokens in microseconds, by token tile: fixed +
+// stage * stages of the longest CTA, plus `split` when tiles are split (partial sums through
+// L2; `apart` when every tile is, with fewer tiles than SMs).  Fitted to times on GB300 of N =
+// 1024 .. 22016, K = 4096 .. 11008, M = 80 .. 2048, which it meets within about 10 % (64-token
+// stages and 192-token A4 stages hold two k-blocks, the others one).  What the choice gives,
+// A4, against 192-token (M <= 128: 128-token) tiles split evenly over all SMs, GEMM alone:
+//   M = 200, N = K = 4096: 20.8 -> 9.4 us (64-token tiles, whole)
+//   M = 333, N = 1024 / 4096, K = 4096: 16.1 -> 8.8 / 21.6 -> 14.8 us
+//   M = 512, N = K = 4096: 23.9 -> 15.0 us; M = 2048: 38.1 -> 33.0 us (192, whole)
+//   M = 2048, N = 28672, K = 4096: 163 -> 157 us (192, 17 whole waves)
+struct TileCost {
+  double stage, fixed, split, apart;
+};
+static TileCost tile_cost(int nt, int planes) {
+  if (nt == 64) return planes == 1 ? TileCost{0.336, 4.0, 4.5, 4.5} : TileCost{0.42, 4.5, 4.5, 4.5};
+  if (nt == 192) return planes == 1 ? TileCost{0.515, 7.6, 8.0, 11.0} : TileCost{0.42, 7.3, 8.0, 11.0};
+  return planes == 1 ? TileCost{0.41, 8.0, 5.0, 5.0} : TileCost{0.45, 8.0, 5.0, 5.0};
+}
+
+// `nt` forces the token tile (0: by M), `M_pad` the padded tokens of the operand planes (0: a
+// multiple of the tile).
+static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused, int nt_forced,
+                       int M_pad_forced) {
   GemmArgs& a = plan.args;
   const int KB = K_pad / kKBlock;
   const int planes = bits == 8 ? 2 : 1;
-  int nt = gemm_pick_nt(M, bits, KB);
+  int nt = nt_forced > 0 ? nt_forced : gemm_pick_nt(M, bits, KB);
   int kps = kps_for(nt);
   // A8 192-token tiles take one k-block per stage: a stage holds two 24 KB activation
   // planes, so two-block stages would leave room for only two of them.
@@ -1125,9 +1149,9 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   while (cols < (uint32_t)(acc_cols + a_cols)) cols <<= 1;
 
   const int KI = KB / kps;
-  const int M_pad = round_up(M, nt);
+  const int M_pad = M_pad_forced > 0 ? M_pad_forced : round_up(M, nt);
   const int n_wtiles = ceil_div(N, 128);
-  const int m_tiles = M_pad / nt;
+  const int m_tiles = ceil_div(M, nt);
   const long long tiles = (long long)n_wtiles * m_tiles;
   const long long iters = tiles * KI;
   int G = (int)(iters < num_sms ? iters : num_sms);
@@ -1147,7 +1171,23 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
       G = (int)(4 * tiles);
   }
   long long dp = 0;
+  int sk_ctas = G;
   if (tiles >= 2LL * G) dp = (tiles / G - 1) * G;
+  plan.cost = 0.0;
+  if (M > 64) {
+    // Whole tiles in waves, the last one on as many CTAs as it has tiles; or all but the last
+    // waves whole and the rest split evenly over the SMs.
+    const TileCost c = tile_cost(nt, planes);
+    const int P = (int)(tiles < num_sms ? tiles : num_sms);
+    const double whole = c.fixed + c.stage * KI * ceil_div(tiles, P);
+    const double even = c.fixed + (tiles < num_sms ? c.apart : c.split) + c.stage * ((double)tiles * KI / G);
+    plan.cost = whole < even ? whole : even;
+    if (whole <= even) {
+      G = P;
+      dp = tiles / G * G;
+      sk_ctas = (int)(tiles - dp);
+    }
+  }
 
   // Every tile split evenly over four CTAs: a cluster finishes it.
   a.cl = xch > 0 && m_tiles == 1 && dp == 0 && G == kCluster * tiles ? kCluster : 1;
@@ -1175,6 +1215,7 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   a.conv_slots = conv_slots;
   a.dp_tiles = (int)dp;
   a.sk_iters = (tiles - dp) * KI;
+  a.sk_ctas = sk_ctas;
   // 32-bit work enumeration on the device (UnitIter).
   if ((long long)a.sk_iters * G + G >= (1LL << 32) || tiles >= (1LL << 31)) return false;
   a.tmem_cols = cols;
@@ -1202,6 +1243,22 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   a.rq_items = 0;
   a.rq_shortfall = 0;
   a.wait_cycles = kWaitTimeoutCycles;
+  return true;
+}
+
+bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused) {
+  return plan_tiles(M, N, K_pad, bits, num_sms, plan, fused, 0, 0);
+}
+
+bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan) {
+  if (!plan_gemm(M, N, K_pad, bits, num_sms, plan)) return false;
+  if (M <= 64 || K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;
+  // The operand planes keep the rows of the wide tiles (192 and 128 are multiples of 64), so
+  // that one quantized matrix serves layers of any N.
+  GemmPlan narrow;
+  if (plan_tiles(M, N, K_pad, bits, num_sms, narrow, false, 64, plan.M_pad) && narrow.nt == 64 &&
+      narrow.cost < plan.cost)
+    plan = narrow;
   return true;
 }
 

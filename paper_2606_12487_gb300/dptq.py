@@ -25,7 +25,7 @@ EXPORTS = ("dptq_pack_weights", "dptq_rotate_quant_act", "dptq_rotate_act", "dpt
            "dptq_qgemm_codes", "dptq_reserve", "dptq_get_packed", "dptq_get_shape",
            "dptq_last_device_error", "dptq_destroy", "dptq_status_str", "dptq_last_error_message",
            "dptq_pack_weights_rh", "dptq_rotate_quant_act_rh", "dptq_rotate_act_rh", "dptq_kv4_quantize",
-           "dptq_sensitivity_policy", "dptq_plan_info", "dptq_scratch_buffers")
+           "dptq_sensitivity_policy", "dptq_plan_info", "dptq_launch_plan", "dptq_scratch_buffers")
 
 
 class DptqError(RuntimeError):
@@ -73,6 +73,7 @@ def load(build_if_missing: bool = True):
                 "dptq_sensitivity_policy": ([P, P, I, I, I, I, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                              P, P, P, P], I),
                 "dptq_plan_info": ([I, I, I, I, I, I, ctypes.POINTER(I), I], I),
+                "dptq_launch_plan": ([I, I, I, I, I, ctypes.POINTER(I), I], I),
                 "dptq_scratch_buffers": ([ctypes.POINTER(P), ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(I), I,
                                           ctypes.POINTER(I)], I),
             }
@@ -292,6 +293,14 @@ def dptq_plan_info(M: int, N: int, K: int, bits: int, num_sms: int, fused: bool 
     buf = (ctypes.c_int * len(PLAN_INFO_FIELDS))()
     _check(load().dptq_plan_info(M, N, K, bits, num_sms, 1 if fused else 0, buf, len(PLAN_INFO_FIELDS)))
     return dict(zip(PLAN_INFO_FIELDS, list(buf)))
+
+
+def dptq_launch_plan(M: int, N: int, K: int, bits: int, num_sms: int) -> dict:
+    """The plan that a two-launch call takes (host only): PLAN_INFO_FIELDS, "sk_ctas", "cluster"."""
+    fields = PLAN_INFO_FIELDS + ("sk_ctas", "cluster")
+    buf = (ctypes.c_int * len(fields))()
+    _check(load().dptq_launch_plan(M, N, K, bits, num_sms, buf, len(fields)))
+    return dict(zip(fields, list(buf)))
 
 
 def dptq_get_packed(layer: QLinear):
