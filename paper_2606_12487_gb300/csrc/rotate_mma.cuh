@@ -40,6 +40,7 @@ namespace dptq {
 
 constexpr int kUnit = 1024;            // elements of one warp
 constexpr int kUnitBytes = kUnit * 8;  // its (hi, lo) pairs in the exchange
+constexpr int kStageBytes = kUnit * 2;  // its halves, waiting for their turn
 constexpr uint32_t kRowSlow = 0x7FFFFFFFu;   // in place of a maximum: the row leaves the pair form
 
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
@@ -107,6 +108,21 @@ __host__ __device__ __forceinline__ constexpr int xch_granule(int i) {
   return (i >> 1) ^ ((i >> 4) & 1) ^ ((((i >> 8) ^ (i >> 5)) & 1) << 1) ^ (((i >> 9) & 1) << 2);
 }
 
+// 16 bytes at granule (base's) ^ g of a unit, g a constant: the low three bits by an exclusive
+// or of the address (units are 128-byte aligned), the rest, which the base leaves zero, as
+// an immediate offset.
+__device__ __forceinline__ void xch_store(uint32_t base, int g, const float4& v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"((base ^ (16 * (g & 7))) + 16 * (g & ~7)), "f"(v.x),
+               "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void xch_load(uint32_t base, int g, int off, uint64_t& a, uint64_t& b) {
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];"
+               : "=l"(a), "=l"(b)
+               : "r"((base ^ (16 * (g & 7))) + 16 * (g & ~7) + off)
+               : "memory");
+}
+
 // The units of a row: whole blocks first, then the tail block in units of its own.
 struct UnitMap {
   int nmain;   // units of whole blocks (a multiple of G)
@@ -133,51 +149,58 @@ __device__ __forceinline__ float pair_to_rotated(float hi, float lo, int l, floa
 }
 
 // ---------------------------------------------------------------- rotation of one unit
-// The 16 halves-pairs of this lane (w[4 j + m]: elements 64 j + 2 m, 2 m + 1 of its run).
+// First element of the lane's four runs of eight halves, 64 elements apart.
 __device__ __forceinline__ int unit_lane_offset(int lane) {
   return (lane & 3) * 8 + ((lane >> 2) & 1) * 32 + (lane >> 3) * 256;
 }
-__device__ __forceinline__ void unit_load(const __half* row, int e0, int end, int lane, uint32_t (&w)[16]) {
+__device__ __forceinline__ void unit_load(const __half* row, int e0, int end, int lane, uint4 (&w)[4]) {
   const int o = e0 + unit_lane_offset(lane);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (o + 64 * j < end) v = __ldg(reinterpret_cast<const uint4*>(row + o + 64 * j));
-    w[4 * j] = v.x;
-    w[4 * j + 1] = v.y;
-    w[4 * j + 2] = v.z;
-    w[4 * j + 3] = v.w;
-  }
+  for (int j = 0; j < 4; ++j)
+    w[j] = o + 64 * j < end ? __ldg(reinterpret_cast<const uint4*>(row + o + 64 * j)) : make_uint4(0u, 0u, 0u, 0u);
 }
-__device__ __forceinline__ void unit_signs(const int8_t* signs, int e0, int end, int lane, uint32_t (&w)[16]) {
+// The signs of a lane's eight halves at offset o (inside the row) applied to them.
+__device__ __forceinline__ void run_signs(const int8_t* signs, int o, uint4& v) {
+  const uint2 s = __ldg(reinterpret_cast<const uint2*>(signs + o));
+  v.x ^= __byte_perm(s.x, 0u, 0x1404) & 0x80008000u;   // bytes 0, 1 to the sign bits
+  v.y ^= __byte_perm(s.x, 0u, 0x3424) & 0x80008000u;
+  v.z ^= __byte_perm(s.y, 0u, 0x1404) & 0x80008000u;
+  v.w ^= __byte_perm(s.y, 0u, 0x3424) & 0x80008000u;
+}
+// Asynchronous copies of the lane's four runs to its own 16-byte places of `stg` (2048 bytes a
+// warp, [run][lane]; zeros past the row): the next row waits there, not in registers.
+__device__ __forceinline__ void unit_prefetch(const __half* row, int e0, int end, int lane, uint8_t* stg) {
   const int o = e0 + unit_lane_offset(lane);
+  const uint32_t at = smem_u32(stg) + 16 * lane;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    if (o + 64 * j < end) {
-      const uint2 s = __ldg(reinterpret_cast<const uint2*>(signs + o + 64 * j));
-      w[4 * j] ^= __byte_perm(s.x, 0u, 0x1404) & 0x80008000u;   // bytes 0, 1 to the sign bits
-      w[4 * j + 1] ^= __byte_perm(s.x, 0u, 0x3424) & 0x80008000u;
-      w[4 * j + 2] ^= __byte_perm(s.y, 0u, 0x1404) & 0x80008000u;
-      w[4 * j + 3] ^= __byte_perm(s.y, 0u, 0x3424) & 0x80008000u;
-    }
+    const bool in = o + 64 * j < end;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at + 512 * j),
+                 "l"(row + (in ? o + 64 * j : 0)), "r"(in ? 16 : 0)
+                 : "memory");
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // An upper bound of the unit's sum of |x| in units of 1/4, at least 2^22 when the sum is
 // not known to be below 2^20 (also for infinities and NaN).  Eight binary16 additions in a
 // row lose at most 7 2^-11 of their sum; the factor 1 + 2^-7 covers that and the fp32 steps.
 constexpr uint32_t kL1Slow = 1u << 22;
-__device__ __forceinline__ uint32_t unit_l1(const uint32_t (&w)[16]) {
-  __half2 s0 = __habs2(as_half2(w[0])), s1 = __habs2(as_half2(w[8]));
+template <class Run>
+__device__ __forceinline__ uint32_t unit_l1(Run run) {
+  __half2 s[2];
 #pragma unroll
-  for (int i = 1; i < 8; ++i) {
-    s0 = __hadd2_rn(s0, __habs2(as_half2(w[i])));
-    s1 = __hadd2_rn(s1, __habs2(as_half2(w[8 + i])));
+  for (int j = 0; j < 4; ++j) {
+    const uint4 v = run(j);
+    const __half2 h[4] = {__habs2(as_half2(v.x)), __habs2(as_half2(v.y)), __habs2(as_half2(v.z)), __habs2(as_half2(v.w))};
+    s[j >> 1] = (j & 1) ? __hadd2_rn(s[j >> 1], h[0]) : h[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) s[j >> 1] = __hadd2_rn(s[j >> 1], h[i]);
   }
-  const float2 a = __half22float2(s0), b = __half22float2(s1);
-  const float s = (a.x + a.y) + (b.x + b.y);
+  const float2 a = __half22float2(s[0]), b = __half22float2(s[1]);
+  const float t = (a.x + a.y) + (b.x + b.y);
   uint32_t v = kL1Slow;
-  if (s < 500000.f) v = (uint32_t)(int)(s * 4.04f) + 2u;   // 4 (1 + 2^-7) < 4.04
+  if (t < 500000.f) v = (uint32_t)(int)(t * 4.04f) + 2u;   // 4 (1 + 2^-7) < 4.04
   return __reduce_add_sync(0xffffffffu, v);
 }
 // k of the block from the sum of its units' bounds.
@@ -187,13 +210,19 @@ __device__ __forceinline__ int split_k(uint32_t l1q, int l) {
   return k > 0 ? k : 0;
 }
 // Whether every value is a multiple of 2^(k - 24) (k >= 1).
-__device__ __forceinline__ bool unit_on_grid(const uint32_t (&w)[16], int k) {
+template <class Run>
+__device__ __forceinline__ bool unit_on_grid(Run run, int k) {
   const __half2 c = __half2half2(__ushort_as_half((unsigned short)((k - 14 + 15) << 10)));   // 2^(k - 14)
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const __half2 m = __hmin2(__habs2(as_half2(w[i])), c);
-    ok = ok && as_u32(__hsub2_rn(__hadd2_rn(m, c), c)) == as_u32(m);
+  for (int j = 0; j < 4; ++j) {
+    const uint4 v = run(j);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __half2 m = __hmin2(__habs2(as_half2(w[i])), c);
+      ok = ok && as_u32(__hsub2_rn(__hadd2_rn(m, c), c)) == as_u32(m);
+    }
   }
   return ok;
 }
@@ -201,21 +230,22 @@ __device__ __forceinline__ bool unit_on_grid(const uint32_t (&w)[16], int k) {
 // Split, MMAs and the butterflies of bits 0 .. 7, then the unit's pairs into the exchange
 // (`xu`: the unit's 8192 bytes).  FULL: l >= 8, every level applies; a level under a
 // condition costs a register move for each of its additions.
-template <bool FULL>
-__device__ __forceinline__ void unit_phase1(const uint32_t (&w)[16], const uint32_t (&am)[4], int l, int k, int lane,
-                                            uint8_t* xu) {
+template <bool FULL, class Run>
+__device__ __forceinline__ void unit_phase1(Run run, const uint32_t (&am)[4], int l, int k, int lane, uint8_t* xu) {
   // C = T = 2^(10 + u): |x| + C for |x| <= T rounds to a multiple of 2^u; larger values
   // are multiples of 2^u already.
   const __half2 c = __half2half2(__ushort_as_half((unsigned short)((11 - l + k + 15) << 10)));
   uint64_t h[8][2], o[8][2];   // [instance 2 j + b2][bit 0]: pairs over bit 5
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
+    const uint4 wv = run(j);
+    const uint32_t w[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
     for (int b2 = 0; b2 < 2; ++b2) {
       uint32_t hi[2], lo[2];
 #pragma unroll
       for (int b1 = 0; b1 < 2; ++b1) {
-        const uint32_t x = w[4 * j + 2 * b2 + b1];
+        const uint32_t x = w[2 * b2 + b1];
         const __half2 m = __hmin2(__habs2(as_half2(x)), c);
         const __half2 r = __hsub2_rn(__hadd2_rn(m, c), c);
         lo[b1] = as_u32(__hsub2_rn(m, r)) ^ (x & 0x80008000u);
@@ -247,7 +277,7 @@ __device__ __forceinline__ void unit_phase1(const uint32_t (&w)[16], const uint3
   }
   // bit 5 and the stores: element bits 1 = g0, 3 = g1, 4 = g2, 8 = q0, 9 = q1
   const int g = lane >> 2, q = lane & 3;
-  const int gb = xch_granule(((g & 1) << 1) | ((g >> 1) << 3) | (q << 8));
+  const uint32_t base = smem_u32(xu) + 16 * xch_granule(((g & 1) << 1) | ((g >> 1) << 3) | (q << 8));
 #pragma unroll
   for (int n = 0; n < 8; ++n) {
     float h00, h01, h10, h11, o00, o01, o10, o11;   // [bit 0][bit 5]
@@ -264,10 +294,8 @@ __device__ __forceinline__ void unit_phase1(const uint32_t (&w)[16], const uint3
       v1 = make_float4(h01, o01, h11, o11);
     }
     const int i = ((n & 1) << 2) | ((n >> 1) << 6);
-    // (gb ^ low) + high: gb and the constant share no bit of 8 and up
-    const int g0 = xch_granule(i), g1 = xch_granule(i | 32);
-    *reinterpret_cast<float4*>(xu + 16 * (gb ^ (g0 & 7)) + 16 * (g0 & ~7)) = v0;
-    *reinterpret_cast<float4*>(xu + 16 * (gb ^ (g1 & 7)) + 16 * (g1 & ~7)) = v1;
+    xch_store(base, xch_granule(i), v0);
+    xch_store(base, xch_granule(i | 32), v1);
   }
 }
 
@@ -285,16 +313,12 @@ struct RunLayout {
 template <int G, bool FULL>
 __device__ __forceinline__ void unit_phase2(const uint8_t* xg, int t, int l, uint64_t (&v)[32]) {
   using RL = RunLayout<G>;
-  const int gb = xch_granule(RL::low(t));
+  const uint32_t base = smem_u32(xg) + 16 * xch_granule(RL::low(t));
 #pragma unroll
   for (int c = 0; c < RL::C; ++c) {
 #pragma unroll
     for (int e = 0; e < RL::R; e += 2) {
-      const int gc = xch_granule(256 * (c & 3) + e);
-      const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(xg + 16 * (gb ^ (gc & 7)) + (c >> 2) * kUnitBytes +
-                                                                16 * (gc & ~7));
-      v[c * RL::R + e] = p.x;
-      v[c * RL::R + e + 1] = p.y;
+      xch_load(base, xch_granule(256 * (c & 3) + e), (c >> 2) * kUnitBytes, v[c * RL::R + e], v[c * RL::R + e + 1]);
     }
   }
 #pragma unroll
@@ -307,45 +331,53 @@ __device__ __forceinline__ void unit_phase2(const uint8_t* xg, int t, int l, uin
   }
 }
 
-// Largest |fl(S)| of the warp's values, as fp32 bits; `mine`: the lane's.
-__device__ __forceinline__ uint32_t warp_sum_max(const uint64_t (&v)[32], uint32_t& mine) {
-  float m0 = 0.f, m1 = 0.f;
+// Largest |fl(S)| of the warp's values, as fp32 bits; part[g]: the lane's over values 8 g .. 8 g + 7.
+__device__ __forceinline__ uint32_t warp_sum_max(const uint64_t (&v)[32], float (&part)[4]) {
 #pragma unroll
-  for (int e = 0; e < 32; e += 2) {
-    float h, o, h2, o2;
-    f2_unpack(v[e], h, o);
-    f2_unpack(v[e + 1], h2, o2);
-    m0 = fmaxf(m0, fabsf(__fadd_rn(h, o)));
-    m1 = fmaxf(m1, fabsf(__fadd_rn(h2, o2)));
+  for (int g = 0; g < 4; ++g) {
+    part[g] = 0.f;
+#pragma unroll
+    for (int e = 8 * g; e < 8 * g + 8; e += 2) {
+      float h, o, h2, o2;
+      f2_unpack(v[e], h, o);
+      f2_unpack(v[e + 1], h2, o2);
+      part[g] = fmaxf(part[g], fmaxf(fabsf(__fadd_rn(h, o)), fabsf(__fadd_rn(h2, o2))));
+    }
   }
-  mine = __float_as_uint(fmaxf(m0, m1));
-  return __reduce_max_sync(0xffffffffu, mine);
+  return __reduce_max_sync(0xffffffffu,
+                           __float_as_uint(fmaxf(fmaxf(part[0], part[1]), fmaxf(part[2], part[3]))));
 }
 
-// Largest |y| over the values whose |fl(S)| is `wm` (odd l: 1 / sqrt 2 and the sum's own
-// remainder decide y's last bit), in lanes that hold one; 0 in the others.
-__device__ __forceinline__ float largest_rotated(const uint64_t (&v)[32], uint32_t wm, bool has, int l, float c_hi,
-                                                 float c_lo) {
+// Largest |y| over the lane's values whose |fl(S)| is `wm`, 0 if it has none (odd l: 1 / sqrt 2
+// and the sum's own remainder decide y's last bit).  Lanes look only at the eights that hold
+// one.
+__device__ __forceinline__ float largest_rotated(const uint64_t (&v)[32], const float (&part)[4], uint32_t wm, int l,
+                                                 float c_hi, float c_lo) {
   float ym = 0.f;
-  int left = has ? 1 : 0;
-#pragma unroll 1
-  for (int it = 0; it < left; ++it) {   // the it-th such value of the lane
-    float ch = 0.f, cl = 0.f;
-    int c = 0;
 #pragma unroll
-    for (int e = 0; e < 32; ++e) {
-      float h, o;
-      f2_unpack(v[e], h, o);
-      if ((__float_as_uint(__fadd_rn(h, o)) & 0x7FFFFFFFu) == wm) {
-        if (c == it) {
-          ch = h;
-          cl = o;
+  for (int g = 0; g < 4; ++g) {
+    if (__float_as_uint(part[g]) == wm) {
+      int left = 1;
+#pragma unroll 1
+      for (int it = 0; it < left; ++it) {   // the it-th such value
+        float ch = 0.f, cl = 0.f;
+        int c = 0;
+#pragma unroll
+        for (int e = 8 * g; e < 8 * g + 8; ++e) {
+          float h, o;
+          f2_unpack(v[e], h, o);
+          if ((__float_as_uint(__fadd_rn(h, o)) & 0x7FFFFFFFu) == wm) {
+            if (c == it) {
+              ch = h;
+              cl = o;
+            }
+            ++c;
+          }
         }
-        ++c;
+        left = c;
+        ym = fmaxf(ym, fabsf(pair_to_rotated(ch, cl, l, c_hi, c_lo)));
       }
     }
-    left = c;
-    ym = fmaxf(ym, fabsf(pair_to_rotated(ch, cl, l, c_hi, c_lo)));
   }
   return ym;
 }
@@ -447,31 +479,38 @@ __device__ __forceinline__ void store_codes_at(const RowOut& d, uint8_t* p, cons
       put(p, q);
     } else {
       // c = hi + lo, hi = sign * 16 (|c| >> 4): |c| - 7.5 rounds to 16 (|c| >> 4) at a
-      // spacing of 16 (adding 1.5 * 2^27).
+      // spacing of 16 (adding 1.5 * 2^27), and c - sign * 7.5 to its signed value.
       float hi[R], lo[R];
+      const uint64_t big = f2_pack(201326592.f, 201326592.f);
 #pragma unroll
-      for (int e = 0; e < R; ++e) {
-        const float h = __fsub_rn(__fadd_rn(__fadd_rn(fabsf(q[e]), -7.5f), 201326592.f), 201326592.f);
-        hi[e] = h == 0.f ? 0.f : copysignf(h, q[e]);
-        lo[e] = __fsub_rn(q[e], hi[e]);
+      for (int e = 0; e < R; e += 2) {
+        const uint64_t c = f2_pack(q[e], q[e + 1]);
+        const uint64_t h =
+            f2_sub(f2_add(f2_sub(c, f2_pack(copysignf(7.5f, q[e]), copysignf(7.5f, q[e + 1]))), big), big);
+        f2_unpack(h, hi[e], hi[e + 1]);
+        f2_unpack(f2_sub(c, h), lo[e], lo[e + 1]);
       }
       put(p, hi);
       put(p + d.plane, lo);
     }
   } else if constexpr (MODE == kRQPublic) {
-    uint32_t b[R];   // two's complement in the low bits of q + 1.5 * 2^23
-#pragma unroll
-    for (int e = 0; e < R; ++e) b[e] = __float_as_uint(__fadd_rn(q[e], kRoundBias));
+    // Several codes make one exact fp32 sum with a bias that keeps each field positive; the
+    // fields are the low bits after adding 1.5 * 2^23, and flipping each top bit gives two's
+    // complement.
     if (d.bits == 4) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int e = 0; e < R; ++e) w |= (b[e] & 0xFu) << (4 * e);
-      if constexpr (R == 2) *p = (uint8_t)w;
-      if constexpr (R == 4) *reinterpret_cast<uint16_t*>(p) = (uint16_t)w;
-      if constexpr (R == 8) *reinterpret_cast<uint32_t*>(p) = w;
+      auto four = [&](int e) {
+        return __float_as_uint(__fadd_rn(
+            __fmaf_rn(q[e + 3], 4096.f, __fmaf_rn(q[e + 2], 256.f, __fmaf_rn(q[e + 1], 16.f, q[e]))), kRoundBias + 34952.f));
+      };
+      if constexpr (R == 2) *p = (uint8_t)(__float_as_uint(__fadd_rn(__fmaf_rn(q[1], 16.f, q[0]), kRoundBias + 136.f)) ^ 0x88u);
+      if constexpr (R == 4) *reinterpret_cast<uint16_t*>(p) = (uint16_t)(four(0) ^ 0x8888u);
+      if constexpr (R == 8) *reinterpret_cast<uint32_t*>(p) = __byte_perm(four(0), four(4), 0x5410) ^ 0x88888888u;
     } else {
-      auto word = [&](int e) { return __byte_perm(__byte_perm(b[e], b[e + 1], 0x0040), __byte_perm(b[e + 2], b[e + 3], 0x0040), 0x5410); };
-      if constexpr (R == 2) *reinterpret_cast<uint16_t*>(p) = (uint16_t)__byte_perm(b[0], b[1], 0x0040);
+      auto two = [&](int e) {
+        return __float_as_uint(__fadd_rn(__fmaf_rn(q[e + 1], 256.f, q[e]), kRoundBias + 32896.f));
+      };
+      auto word = [&](int e) { return __byte_perm(two(e), two(e + 2), 0x5410) ^ 0x80808080u; };
+      if constexpr (R == 2) *reinterpret_cast<uint16_t*>(p) = (uint16_t)(two(0) ^ 0x8080u);
       if constexpr (R == 4) *reinterpret_cast<uint32_t*>(p) = word(0);
       if constexpr (R == 8) {   // rows start 4-byte aligned at least
         reinterpret_cast<uint32_t*>(p)[0] = word(0);
@@ -598,15 +637,16 @@ struct UnitGeom {
   }
 };
 
-// From the loaded halves to the thread's exact sums; false when the unit's block leaves the
-// pair form (v is then meaningless).  l1s: a word per warp of the group; group_sync: its
-// barrier; after_split(): called when w is free (the next row's loads).
-template <int G, class GroupSync, class After>
-__device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, uint32_t (&w)[16], const uint32_t (&am)[4], int lane,
+// From the lane's halves (raw(j): run j, signs(j, v): the signs applied to it) to the
+// thread's exact sums; false when the unit's block leaves the pair form (v is then
+// meaningless).  l1s: a word per warp of the group; group_sync: its barrier; after_split():
+// called when the halves are no longer needed (the next row's loads).
+template <int G, class Raw, class Signs, class GroupSync, class After>
+__device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, Signs signs, const uint32_t (&am)[4], int lane,
                                           uint8_t* xu, uint32_t* l1s, GroupSync group_sync, After after_split,
                                           uint64_t (&v)[32]) {
   constexpr int full_l = G == 1 ? 10 : G == 2 ? 11 : 12;
-  uint32_t l1 = unit_l1(w);
+  uint32_t l1 = unit_l1(raw);
   if constexpr (G > 1) {
     if (lane == 0) l1s[u.wg] = l1;
     group_sync();
@@ -616,11 +656,16 @@ __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, uint32_t (&w)[16
   }
   bool ok = l1 < kL1Slow;
   const int k = ok ? split_k(l1, u.l) : 0;
-  if (k > 0) ok = __all_sync(0xffffffffu, unit_on_grid(w, k));
+  if (k > 0) ok = __all_sync(0xffffffffu, unit_on_grid(raw, k));
+  auto run = [&](int j) {
+    uint4 x = raw(j);
+    signs(j, x);
+    return x;
+  };
   if (u.l >= 8)
-    unit_phase1<true>(w, am, u.l, k, lane, xu);
+    unit_phase1<true>(run, am, u.l, k, lane, xu);
   else
-    unit_phase1<false>(w, am, u.l, k, lane, xu);
+    unit_phase1<false>(run, am, u.l, k, lane, xu);
   after_split();
   group_sync();
   const uint8_t* xg = xu - u.wg * kUnitBytes;
@@ -635,8 +680,8 @@ __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, uint32_t (&w)[16
 // warps that share `lead` (zero before the row's first warp).
 __device__ __forceinline__ uint32_t unit_max(const uint64_t (&v)[32], int l, uint32_t* lead, int lane, float c_hi,
                                              float c_lo) {
-  uint32_t mine;
-  const uint32_t wm = warp_sum_max(v, mine);
+  float part[4];
+  const uint32_t wm = warp_sum_max(v, part);
   uint32_t m = __float_as_uint(__fmul_rn(__uint_as_float(wm), __int_as_float((127 - (l >> 1)) << 23)));
   if (l & 1) {
     // 2^-j fl(S) / sqrt 2, rounded twice, is within 2 units of y: only warps that are not
@@ -646,7 +691,7 @@ __device__ __forceinline__ uint32_t unit_max(const uint64_t (&v)[32], int l, uin
     if (lane == 0) seen = atomicMax(lead, m);
     seen = __shfl_sync(0xffffffffu, seen, 0);
     m = seen > m + 8u ? 0u
-                      : __reduce_max_sync(0xffffffffu, __float_as_uint(largest_rotated(v, wm, mine == wm, l, c_hi, c_lo)));
+                      : __reduce_max_sync(0xffffffffu, __float_as_uint(largest_rotated(v, part, wm, l, c_hi, c_lo)));
   }
   return m;
 }
@@ -728,11 +773,16 @@ __device__ __forceinline__ void fused_rotate_row(const RQArgs& a, int row, int p
   uint64_t v[32];
   uint32_t m = 0u;
   if (act) {
-    uint32_t w[16], am[4];
+    uint32_t am[4];
+    uint4 w[4];
     unit_load(a.x + (size_t)row * a.K, u.e0, u.load_end, lane, w);
     mma_hadamard_a(u.l, lane, am);
-    if (a.signs != nullptr) unit_signs(a.signs, u.e0, u.load_end, lane, w);
-    const bool ok = unit_sums<G>(u, w, am, lane, smem + wc * kUnitBytes, l1s + wc - u.wg,
+    const int o = u.e0 + unit_lane_offset(lane);
+    const bool ok = unit_sums<G>(u, [&](int j) { return w[j]; },
+                                 [&](int j, uint4& x) {
+                                   if (a.signs != nullptr && o + 64 * j < u.load_end) run_signs(a.signs, o + 64 * j, x);
+                                 },
+                                 am, lane, smem + wc * kUnitBytes, l1s + wc - u.wg,
                                  [&] {
                                    if constexpr (G == 1)
                                      __syncwarp();

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // same row: 33.8 -> 7.3 us.
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
-  extern __shared__ __align__(16) uint8_t rm_smem[];
+  extern __shared__ __align__(128) uint8_t rm_smem[];
   constexpr int kBatch = 1024;       // rows between looks at the left-over ones (32 words)
   __shared__ uint32_t red[2][16];    // [row parity][warp]: fp32 bits of the largest |y|, or kRowSlow
   __shared__ uint32_t xmax[2][8];    // the same of the cluster's CTAs
@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
   const int K = a.K, K_pad = a.KB * 128;
   const UnitGeom<G> u(a, rank * W + warp, lane, MODE == kRQAct ? K_pad : K);
   uint8_t* const xu = rm_smem + warp * kUnitBytes;
+  uint8_t* const stg = rm_smem + W * kUnitBytes + warp * kStageBytes;
   auto group_sync = [&] {
     if constexpr (G == 1)
       __syncwarp();
@@ -101,8 +102,7 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
 #pragma unroll 1
   for (int row0 = (int)blockIdx.x / csize; row0 < a.rows_out; row0 += kBatch * ncl) {
     bool any_slow = false;
-    uint32_t w[16];
-    if (row0 < a.rows_in) unit_load(a.x + (size_t)row0 * K, u.e0, u.load_end, lane, w);
+    if (row0 < a.rows_in) unit_prefetch(a.x + (size_t)row0 * K, u.e0, u.load_end, lane, stg);
 #pragma unroll 1
     for (int it = 0; it < kBatch; ++it, par ^= 1) {
       const int row = row0 + it * ncl;
@@ -116,13 +116,18 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
         }
         continue;
       }
-      if (a.signs != nullptr) unit_signs(a.signs, u.e0, u.load_end, lane, w);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");   // the lane's own copies
       uint64_t v[32];
       const bool ok = unit_sums<G>(
-          u, w, am, lane, xu, l1s + warp - u.wg, group_sync,
+          u, [&](int j) { return *reinterpret_cast<const uint4*>(stg + 512 * j + 16 * lane); },
+          [&](int j, uint4& x) {
+            const int o = u.e0 + unit_lane_offset(lane) + 64 * j;
+            if (a.signs != nullptr && o < u.load_end) run_signs(a.signs, o, x);
+          },
+          am, lane, xu, l1s + warp - u.wg, group_sync,
           [&] {
             if (it + 1 < kBatch && row + ncl < a.rows_in)
-              unit_load(a.x + (size_t)(row + ncl) * K, u.e0, u.load_end, lane, w);
+              unit_prefetch(a.x + (size_t)(row + ncl) * K, u.e0, u.load_end, lane, stg);
           },
           v);
       uint32_t m = MODE == kRQY ? 0u : unit_max(v, u.l, &lead[par], lane, a.c_hi, a.c_lo);
@@ -187,7 +192,8 @@ cudaError_t launch_rotate_mma_g(const RQArgs& a, cudaStream_t s, bool pdl) {
   const int units = unit_map(a.K, a.tail, G).units;
   const int csize = ceil_div(units, 16);
   const int W = round_up(ceil_div(units, csize), G);
-  const int smem = W * kUnitBytes;   // the exchange, or (64-bit integers) a block of 1024 G values
+  // The exchange, or (64-bit integers) a block of 1024 G values; the coming row.
+  const int smem = W * (kUnitBytes + kStageBytes);
   int sms = 0;
   cudaError_t e = device_sms(&sms);
   if (e == cudaSuccess) e = ensure_max_dyn_smem(rotate_mma_kernel<MODE, G>);
