@@ -245,12 +245,14 @@ dptq_status dptq_reserve(int max_M, int max_K, int max_N);
 #define DPTQ_PLAN_INFO_LEN 20
 dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused, int* info, int info_len);
 
-/* The plan that a two-launch call takes (dptq_qlinear_gemm, dptq_qgemm_codes, and dptq_qlinear
- * where it does not run as one launch), in the order of dptq_plan_info, then 20 the CTAs that
- * share the stream-K stages (as many as tiles: whole tiles) and 21 the CTAs of a cluster (4,
- * or 1: none).  Host only; errors as dptq_plan_info. */
+/* The plan that a launch takes, in the order of dptq_plan_info, then 20 the CTAs that share
+ * the stream-K stages (as many as tiles: whole tiles) and 21 the CTAs of a cluster that
+ * share a weight tile (2 or 4, or 1: none).  row_ctas = 0: a GEMM launch (dptq_qlinear_gemm,
+ * dptq_qgemm_codes, and dptq_qlinear where it does not run as one launch); otherwise the
+ * one-launch kernel, with that many CTAs rotating token rows (one per token, two for
+ * K > 8192).  Host only; errors as dptq_plan_info, and INVALID_ARG for row_ctas < 0. */
 #define DPTQ_LAUNCH_PLAN_LEN 22
-dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int* info, int info_len);
+dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int row_ctas, int* info, int info_len);
 
 /* Copy the packed weights out in the public layout: wq_host uint8 [N][K/2] (same
  * nibble format as 4-bit activation codes) and sw_host float [N].  Either may be

@@ -622,8 +622,8 @@ dptq_status dptq_qlinear(dptq_handle h, const void* x_fp16, int M, int bits, voi
   GemmPlan fp;
   int cpr = 0, wpc = 0;
   if (fused_allowed() && h->K_pad <= kFusedMaxKPad && pow2_tail(h->K, h->had_block) &&
-      plan_gemm(M, h->N, h->K_pad, bits, sc->num_sms, fp, true) && fp.M_pad == plan.M_pad && fp.M_pad <= 64 &&
-      fused_rotation_split(h->K, h->had_block, h->K % h->had_block, cpr, wpc)) {
+      plan.M_pad <= 64 && fused_rotation_split(h->K, h->had_block, h->K % h->had_block, cpr, wpc) &&
+      plan_launch(M, h->N, h->K_pad, bits, sc->num_sms, fp, M * cpr) && fp.M_pad == plan.M_pad) {
     int nfull, tail, log2B;
     if ((st = check_shape(h->K, h->had_block, nfull, tail, log2B)) != DPTQ_OK) return st;
     fp.args.rq = make_rq(x_fp16, M, fp.M_pad, h->K, h->KB, h->had_block, nfull, tail, log2B, bits, sc->sa, sc->act);
@@ -760,11 +760,12 @@ dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused
   return DPTQ_OK;
 }
 
-dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int* info, int info_len) {
+dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int row_ctas, int* info, int info_len) {
   const dptq_status st = check_plan_args(M, N, K, bits, num_sms, info, info_len, DPTQ_LAUNCH_PLAN_LEN);
   if (st != DPTQ_OK) return st;
+  if (row_ctas < 0) return fail(DPTQ_ERR_INVALID_ARG, "row_ctas must be >= 0");
   GemmPlan plan{};
-  if (!plan_launch(M, N, round_up(K, kKBlock), bits, num_sms, plan))
+  if (!plan_launch(M, N, round_up(K, kKBlock), bits, num_sms, plan, row_ctas))
     return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
   write_plan(plan, info, DPTQ_LAUNCH_PLAN_LEN);
   return DPTQ_OK;

@@ -161,9 +161,10 @@ struct GemmPlan {
 // `fused` plans the decode kernel that rotates and quantizes the rows itself: two k-blocks
 // per stage; false if it does not fit.
 bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused = false);
-// The plan of a two-launch call: plan_gemm's, or for more than 64 tokens 64-token tiles on the
-// same operand planes where they are estimated to be faster.
-bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan);
+// The plan of a launch: plan_gemm's, for more than 64 tokens 64-token tiles on the same operand
+// planes where they are estimated to be faster, for up to 64 whole or half tiles on fewer
+// CTAs.  items: CTAs that rotate token rows in a fused launch, 0 for a GEMM launch.
+bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, int items = 0);
 // Warps that share a Hadamard block of a row in the tensor-core rotation (1, 2 or 4; K, B and
 // a power-of-two tail).
 int rotate_group(int K, int B, int tail);

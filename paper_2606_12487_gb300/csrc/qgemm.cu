@@ -61,7 +61,7 @@ constexpr int kConvBytes = 128 * 128;   // one weight tile widened to E4M3
 constexpr int kMaxStages = 8;
 constexpr int kMaxConvSlots = 4;
 constexpr int kSmemLimit = 232448;      // 227 KB opt-in dynamic shared memory per CTA
-constexpr int kCluster = 4;   // CTAs of a cluster that split a weight tile
+constexpr int kCluster = 4;   // most CTAs of a cluster that split a weight tile
 constexpr int kBarrierBytes = 2048;   // barriers and flags, token scales (tiles <= 64), output transpose (1 KB)
 
 struct Unit {
@@ -171,20 +171,20 @@ struct Smem {
   __device__ __forceinline__ uint8_t* end(int S) const { return slot(S); }
 };
 
-// A tile whose k range the kCluster CTAs of a cluster share: CTA r finishes tokens
-// r NT / 4 .. of it.  Each CTA sends the others their tokens' partial sums (exact integers in
+// A tile whose k range the CL (2 or 4) CTAs of a cluster share: CTA r finishes tokens
+// r NT / CL .. of it.  Each CTA sends the others their tokens' partial sums (exact integers in
 // fp32: their order does not matter) straight into their shared memory and adds what it
 // receives to its own accumulators: one store and one barrier wait, where partial sums in
 // global memory take reductions, a fence, an atomic and a read back (LLaMA-2-7B o at
 // M = 32: 3.9 us from the last MMA to the exit).  Run by the four epilogue warps; `tb`: the
 // warp's accumulators; n: this thread's channel.
-template <int NT, int KPS>
+template <int NT, int KPS, int CL>
 __device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT, KPS>& sm, uint64_t* bars, uint64_t* xbar,
                                                __half* xpose, const float* sa_sh, uint32_t tb, int n, int nt, int q,
                                                int lane, volatile int* abort_flag) {
-  constexpr int TQ = NT / kCluster;          // tokens a CTA finishes: 4, 8 or 16
-  float* recv = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kBarrierBytes);   // [3][TQ / 4][128][4]
-  const uint32_t rank = blockIdx.x % kCluster;
+  constexpr int TQ = NT / CL;          // tokens a CTA finishes
+  float* recv = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kBarrierBytes);   // [CL - 1][TQ / 4][128][4]
+  const uint32_t rank = blockIdx.x % CL;
   const int ch = q * 32 + lane;
   cluster_wait();   // the others' barriers are initialized
   float own[TQ];
@@ -216,7 +216,7 @@ __device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT,
   for (int g = 0; g < TQ / 4; ++g) {
     float f[4] = {own[4 * g], own[4 * g + 1], own[4 * g + 2], own[4 * g + 3]};
 #pragma unroll
-    for (int k = 0; k < kCluster - 1; ++k) {
+    for (int k = 0; k < CL - 1; ++k) {
       const float4 p = *reinterpret_cast<const float4*>(recv + ((k * (TQ / 4) + g) * 128 + ch) * 4);
       f[0] += p.x;
       f[1] += p.y;
@@ -266,9 +266,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   // (wide tiles: all eight on the same stage, a k-block per group).
   constexpr bool kPairConv = kATmem && KPS == 2;
   constexpr bool kAltConv = kPairConv && NT <= 64;
-  // Clusters of kCluster CTAs, each with a quarter of a weight tile's k range (small N).
+  // Clusters of two or four CTAs, each with its part of a weight tile's k range (small N).
   constexpr bool kClusterTiles = NT <= 64 && KPS == 2;
-  constexpr uint32_t kXchBytes = (kCluster - 1) * (NT / kCluster) * 128 * 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = a.stages;
@@ -331,7 +330,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   tc_fence_after();
   const bool clustered = kClusterTiles && a.cl > 1;
   if (clustered) {
-    if (threadIdx.x == 0) mbar_arrive_expect_tx(xbar, kXchBytes);
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(xbar, (uint32_t)((a.cl - 1) * (NT / a.cl) * 128 * 4));
     cluster_arrive();   // this CTA's barrier may be counted on by the others
   }
   const uint32_t tmem_base = *tmem_base_sh;
@@ -778,8 +777,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       tc_fence_after();
       if constexpr (kClusterTiles) {
         if (clustered) {
-          epi_ok = cluster_finish<NT, KPS>(a, sm, bars, xbar, xpose, sa_sh, tmem_base + lane_base + (uint32_t)(b * NT), n,
-                                           nt, q, lane, abort_flag);
+          const uint32_t acc = tmem_base + lane_base + (uint32_t)(b * NT);
+          epi_ok = a.cl == 2 ? cluster_finish<NT, KPS, 2>(a, sm, bars, xbar, xpose, sa_sh, acc, n, nt, q, lane, abort_flag)
+                             : cluster_finish<NT, KPS, 4>(a, sm, bars, xbar, xpose, sa_sh, acc, n, nt, q, lane, abort_flag);
           cluster_waited = true;
           break;
         }
@@ -1083,10 +1083,11 @@ static TileCost tile_cost(int nt, int planes) {
   return planes == 1 ? TileCost{0.41, 8.0, 5.0, 5.0} : TileCost{0.45, 8.0, 5.0, 5.0};
 }
 
-// `nt` forces the token tile (0: by M), `M_pad` the padded tokens of the operand planes (0: a
-// multiple of the tile).
+// `nt_forced` forces the token tile (0: by M), `M_pad_forced` the padded tokens of the operand
+// planes (0: a multiple of the tile).  items > 0 (decode tiles): the grid needs only that many
+// CTAs for the rows' rotation (fused; 1 otherwise) and may be smaller than the general plan's.
 static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused, int nt_forced,
-                       int M_pad_forced) {
+                       int M_pad_forced, int items = 0) {
   GemmArgs& a = plan.args;
   const int KB = K_pad / kKBlock;
   const int planes = bits == 8 ? 2 : 1;
@@ -1164,9 +1165,15 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
     // tile is at most twice a CTA's fair share of the stages; otherwise stream-K with at
     // most four CTAs per tile.  A fused launch keeps whole tiles only while they leave four
     // CTAs for every token row.
-    const bool rows_fit = !fused || (long long)M_pad * 4 <= tiles;
+    const bool rows_fit = !fused || (items > 0 ? items : 4LL * M_pad) <= tiles;
+    // Half tiles on clusters of two CTAs cost at most five stages more per CTA than an even
+    // split and save its sums in global memory (about 2 us; a stage takes 0.3 us).
+    const bool halves = items > 0 && xch > 0 && 4 * tiles > num_sms && 2 * tiles <= num_sms && 2 * tiles >= items &&
+                        KI >= 2 && (long long)KI * num_sms - 2LL * KI * tiles <= 10LL * num_sms;
     if (decode_whole_tiles() && rows_fit && tiles <= num_sms && (long long)KI * num_sms <= 2 * iters)
       G = (int)tiles;
+    else if (halves)
+      G = (int)(2 * tiles);
     else if (4 * tiles < G)
       G = (int)(4 * tiles);
   }
@@ -1189,8 +1196,8 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
     }
   }
 
-  // Every tile split evenly over four CTAs: a cluster finishes it.
-  a.cl = xch > 0 && m_tiles == 1 && dp == 0 && G == kCluster * tiles ? kCluster : 1;
+  // Every tile split evenly over four or two CTAs: a cluster finishes it.
+  a.cl = xch == 0 || m_tiles != 1 || dp != 0 ? 1 : G == 4 * tiles ? 4 : G == 2 * tiles ? 2 : 1;
 
   plan.fused = fused;
   plan.a_tmem = a_tmem;
@@ -1227,7 +1234,9 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   // A row's rotation takes one of them, or two (rows of more than 8 units), so that most
   // CTAs only stream weights meanwhile and no CTA takes a second row.
   int np = 1;
-  if (fused) {
+  if (fused && items > 0) {
+    np = 2;   // the row's CTAs fit (checked against the general plan)
+  } else if (fused) {
     if ((long long)M_pad * 4 <= G)
       np = 4;
     else if ((long long)M_pad * 2 <= G && K_pad <= 2 * 4096)
@@ -1250,9 +1259,17 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
   return plan_tiles(M, N, K_pad, bits, num_sms, plan, fused, 0, 0);
 }
 
-bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan) {
-  if (!plan_gemm(M, N, K_pad, bits, num_sms, plan)) return false;
-  if (M <= 64 || K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;
+bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, int items) {
+  const bool fused = items > 0;
+  if (!plan_gemm(M, N, K_pad, bits, num_sms, plan, fused)) return false;
+  if (M <= 64) {
+    // The general plan keeps a CTA for each of two or four parts of a row; the rotation takes
+    // `items` CTAs, so whole tiles (or halves in clusters) may run on fewer.
+    GemmPlan p;
+    if (plan_tiles(M, N, K_pad, bits, num_sms, p, fused, 0, 0, fused ? items : 1) && p.grid >= items) plan = p;
+    return true;
+  }
+  if (K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;
   // The operand planes keep the rows of the wide tiles (192 and 128 are multiples of 64), so
   // that one quantized matrix serves layers of any N.
   GemmPlan narrow;

@@ -73,7 +73,7 @@ def load(build_if_missing: bool = True):
                 "dptq_sensitivity_policy": ([P, P, I, I, I, I, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                              P, P, P, P], I),
                 "dptq_plan_info": ([I, I, I, I, I, I, ctypes.POINTER(I), I], I),
-                "dptq_launch_plan": ([I, I, I, I, I, ctypes.POINTER(I), I], I),
+                "dptq_launch_plan": ([I, I, I, I, I, I, ctypes.POINTER(I), I], I),
                 "dptq_scratch_buffers": ([ctypes.POINTER(P), ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(I), I,
                                           ctypes.POINTER(I)], I),
             }
@@ -295,11 +295,12 @@ def dptq_plan_info(M: int, N: int, K: int, bits: int, num_sms: int, fused: bool 
     return dict(zip(PLAN_INFO_FIELDS, list(buf)))
 
 
-def dptq_launch_plan(M: int, N: int, K: int, bits: int, num_sms: int) -> dict:
-    """The plan that a two-launch call takes (host only): PLAN_INFO_FIELDS, "sk_ctas", "cluster"."""
+def dptq_launch_plan(M: int, N: int, K: int, bits: int, num_sms: int, row_ctas: int = 0) -> dict:
+    """The plan that a launch takes (host only): PLAN_INFO_FIELDS, "sk_ctas", "cluster"; row_ctas
+    CTAs of a one-launch call rotate token rows (0: a GEMM launch)."""
     fields = PLAN_INFO_FIELDS + ("sk_ctas", "cluster")
     buf = (ctypes.c_int * len(fields))()
-    _check(load().dptq_launch_plan(M, N, K, bits, num_sms, buf, len(fields)))
+    _check(load().dptq_launch_plan(M, N, K, bits, num_sms, row_ctas, buf, len(fields)))
     return dict(zip(fields, list(buf)))
 
 

@@ -39,11 +39,23 @@ def test_planes_do_not_depend_on_n(M, bits, sms):
         assert dptq.dptq_launch_plan(M, 4096, K, bits, sms)["M_pad"] == wide["M_pad"]
 
 
-@pytest.mark.parametrize("N,K", [(16, 256), (1024, 4096), (4096, 4096), (4096, 11008), (5120, 384), (28672, 4096)])
+@pytest.mark.parametrize("N,K", [(16, 256), (1024, 4096), (4096, 4096), (4096, 11008), (5120, 384), (5120, 5120), (6144, 4096),
+                                 (8192, 8192), (12288, 4096), (28672, 4096)])
 @pytest.mark.parametrize("bits", [4, 8])
-def test_every_stage_once(N, K, bits):
+@pytest.mark.parametrize("fused", [False, True])
+def test_every_stage_once(N, K, bits, fused):
     for M in MS:
-        p = dptq.dptq_launch_plan(M, N, K, bits, 152)
+        rows = M * (2 if K > 8192 else 1) if fused else 0
+        if fused:
+            # accepted exactly where the general one-launch plan is
+            try:
+                dptq.dptq_plan_info(M, N, K, bits, 152, fused=True)
+            except dptq.DptqError:
+                with pytest.raises(dptq.DptqError):
+                    dptq.dptq_launch_plan(M, N, K, bits, 152, rows)
+                continue
+        p = dptq.dptq_launch_plan(M, N, K, bits, 152, rows)
+        assert p["fused"] == int(fused) and p["grid"] >= rows   # a CTA for every row's rotation
         tiles = p["n_wtiles"] * p["m_tiles"]
         assert p["m_tiles"] * p["nt"] >= M and p["m_tiles"] * p["nt"] <= p["M_pad"]
         assert p["smem_bytes"] <= 232448 and p["grid"] <= 152 and p["kps"] * p["KI"] == -(-K // 128)
@@ -57,6 +69,7 @@ def test_every_stage_once(N, K, bits):
             assert all(n == len(q) and slot == q[0][2] and (slot >= 0) == (len(q) > 1) for _, _, slot, n in q)
         slots = {t: q[0][2] for t, q in parts.items() if q[0][2] >= 0}
         assert len(set(slots.values())) == len(slots)          # a slot serves one tile
-        if p["cluster"] > 1:                                   # four CTAs per tile, one tile per CTA
-            assert p["grid"] == 4 * tiles and all(len(q) == 4 for q in parts.values())
-            assert all(t == c // 4 for c, t, *_ in units(p))
+        n = p["cluster"]
+        if n > 1:                                              # n CTAs per tile, one tile per CTA
+            assert n in (2, 4) and p["grid"] == n * tiles and all(len(q) == n for q in parts.values())
+            assert all(t == c // n for c, t, *_ in units(p))
