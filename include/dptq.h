@@ -172,9 +172,9 @@ dptq_status dptq_sensitivity_policy(const float* x, const float* dx, int L, int 
  * exits, so work enqueued earlier and graphs captured earlier (which keep the old
  * addresses) stay valid.
  * For token tiles of up to 64 rows (M <= 64), K <= 16384 and a power-of-two tail block,
- * rotation, quantization and GEMM run as ONE kernel launch: each token row is split over
- * two or four CTAs of the GEMM grid, each rotating and quantizing its own share of the
- * row, and the row maxima are exchanged between them (the environment variable
+ * rotation, quantization and GEMM run as ONE kernel launch wherever the GEMM grid holds
+ * the CTAs that rotate the token rows: one per row, two for K > 8192 (they exchange the
+ * row's maximum), or on small grids one for several rows (the environment variable
  * DPTQ_FUSED=0 selects the two-launch sequence of dptq_qlinear_quantize +
  * dptq_qlinear_gemm); both give the same bits. */
 dptq_status dptq_qlinear(dptq_handle h, const void* x_fp16, int M, int bits, void* out_fp16,
@@ -250,7 +250,7 @@ dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused
  * share a weight tile (2 or 4, or 1: none).  row_ctas = 0: a GEMM launch (dptq_qlinear_gemm,
  * dptq_qgemm_codes, and dptq_qlinear where it does not run as one launch); otherwise the
  * one-launch kernel, with that many CTAs rotating token rows (one per token, two for
- * K > 8192).  Host only; errors as dptq_plan_info, and INVALID_ARG for row_ctas < 0. */
+ * K > 8192, or on small grids one for several tokens).  Host only; errors as dptq_plan_info, and INVALID_ARG for row_ctas < 0. */
 #define DPTQ_LAUNCH_PLAN_LEN 22
 dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int row_ctas, int* info, int info_len);
 

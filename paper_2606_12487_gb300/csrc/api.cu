@@ -618,12 +618,19 @@ dptq_status dptq_qlinear(dptq_handle h, const void* x_fp16, int M, int bits, voi
   dptq_status st = prepare_qlinear(h, M, bits, s, &dev, &plan, &sc);
   if (st != DPTQ_OK || M == 0) return st;
   if (!x_fp16 || !out_fp16) return fail(DPTQ_ERR_INVALID_ARG, "null pointer");
-  // Small M: one launch that rotates and quantizes the rows and runs the GEMM.
+  // Small M: one launch that rotates and quantizes the rows and runs the GEMM, with a CTA (or
+  // two) per row, or else as many rows side by side in a CTA as its warps hold.
   GemmPlan fp;
-  int cpr = 0, wpc = 0;
-  if (fused_allowed() && h->K_pad <= kFusedMaxKPad && pow2_tail(h->K, h->had_block) &&
-      plan.M_pad <= 64 && fused_rotation_split(h->K, h->had_block, h->K % h->had_block, cpr, wpc) &&
-      plan_launch(M, h->N, h->K_pad, bits, sc->num_sms, fp, M * cpr) && fp.M_pad == plan.M_pad) {
+  int cpr = 0, wpc = 0, rpc = 1;
+  bool one = fused_allowed() && plan.M_pad <= 64 && h->K_pad <= kFusedMaxKPad && pow2_tail(h->K, h->had_block) &&
+             fused_rotation_split(h->K, h->had_block, h->K % h->had_block, cpr, wpc);
+  int items = M * cpr;
+  if (one && !plan_launch(M, h->N, h->K_pad, bits, sc->num_sms, fp, items)) {
+    rpc = cpr == 1 ? 8 / wpc : 1;
+    items = ceil_div(M, rpc);
+    one = rpc > 1 && plan_launch(M, h->N, h->K_pad, bits, sc->num_sms, fp, items);
+  }
+  if (one && fp.M_pad == plan.M_pad) {
     int nfull, tail, log2B;
     if ((st = check_shape(h->K, h->had_block, nfull, tail, log2B)) != DPTQ_OK) return st;
     fp.args.rq = make_rq(x_fp16, M, fp.M_pad, h->K, h->KB, h->had_block, nfull, tail, log2B, bits, sc->sa, sc->act);
@@ -631,7 +638,8 @@ dptq_status dptq_qlinear(dptq_handle h, const void* x_fp16, int M, int bits, voi
     fp.args.rq.pmax = sc->pmax;
     fp.args.rq_cpr = cpr;
     fp.args.rq_wpc = wpc;
-    fp.args.rq_items = M * cpr;
+    fp.args.rq_rpc = rpc;
+    fp.args.rq_items = items;
     return run_gemm(h, fp, sc->act, sc->sa, out_fp16, nullptr, sc, s);
   }
   if ((st = quantize_into_scratch(h, x_fp16, M, bits, plan, sc, s)) != DPTQ_OK) return st;

@@ -131,14 +131,14 @@ struct GemmArgs {
   int cl;              // CTAs of a cluster that share a weight tile's k range (1: no cluster)
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
   // Fused decode launches only: the rotation + quantization of the M_pad token rows
-  // (written to `act` / `sa` by the converter warps of CTAs 0, 1, ...: CTA row * rq_cpr +
-  // part) and the two grid counters [rows ready, CTAs done] that order it before the GEMM
+  // (written to `act` / `sa` by the converter warps of CTAs 0 .. rq_items - 1) and the two grid counters [rows ready, CTAs done] that order it before the GEMM
   // (zero between launches).
   RQArgs rq;
   int rq_np;           // CTAs the grid holds per token row (2 or 4)
   int rq_cpr;          // CTAs that share a row's rotation (1 or 2)
   int rq_wpc;          // units of 1024 elements (warps) of a row in each of them, at most 8
-  int rq_items;        // M * rq_cpr: the value the rows-ready counter reaches
+  int rq_rpc;          // rows a CTA rotates side by side (rq_cpr = 1; at most 8 / rq_wpc)
+  int rq_items;        // CTAs that rotate rows: the value the rows-ready counter reaches
   int rq_shortfall;    // test hook: extra items the activation producer waits for (0)
   uint32_t* gsync;
   long long wait_cycles;   // bound of every pipeline wait (SM cycles) before the kernel gives up
@@ -168,8 +168,8 @@ bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan,
 // Warps that share a Hadamard block of a row in the tensor-core rotation (1, 2 or 4; K, B and
 // a power-of-two tail).
 int rotate_group(int K, int B, int tail);
-// How a fused launch splits a row: CTAs per row and units in each.  False for rows of more
-// than 16 units.
+// How a fused launch splits a row: CTAs per row and units (warps) in each.  False for rows of
+// more than 16 units.
 bool fused_rotation_split(int K, int B, int tail, int& cpr, int& wpc);
 cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl);
 

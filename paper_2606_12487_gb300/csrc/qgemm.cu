@@ -247,10 +247,10 @@ __device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT,
 }
 
 // RG != 0 (decode, two-block stages) makes the launch FUSED: it first rotates and quantizes
-// the token rows itself (RG = 1, 2 or 4 warps per Hadamard block, rotate_mma.cuh).  CTA
-// row * rq_cpr + part takes a row, or half of one of more than 8 units, with its 8 converter
-// warps, in the shared memory of the copy ring, which this CTA fills only afterwards; the
-// other CTAs fill their rings from the start.  The rows are published on a grid counter;
+// the token rows itself (RG = 1, 2 or 4 warps per Hadamard block, rotate_mma.cuh).  Each of the
+// first rq_items CTAs takes a row, or half of one of more than 8 units, or (small grids)
+// several, with its 8 converter warps, in the shared memory of the copy ring, which this CTA
+// fills only afterwards; the other CTAs fill their rings from the start.  The rows are published on a grid counter;
 // every activation producer waits for all of them; the epilogue reads the token scales after
 // the same point, and the last CTA to get there resets the counters and the slots.
 template <int NT, int KPS, int RG>
@@ -316,7 +316,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     mbar_init(aready, 1);
     mbar_init(rdone, 1);
     mbar_init(xbar, 1);
-    if (FUSED) rot_sh[16] = 0u;
+    if (FUSED)
+      for (int i = 16; i < 24; ++i) rot_sh[i] = 0u;
     *abort_flag = 0;
     for (int i = 0; i < 4; ++i) flags[i] = 0;
     fence_mbar_init();
@@ -560,8 +561,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       if (ctid == 0) DPTQ_TRACE_POINT(tr, 125);
       if ((int)blockIdx.x < a.rq_items) {
         const auto csync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kConvThreads) : "memory"); };
-        fused_rotate_row<RG>(a.rq, (int)blockIdx.x / a.rq_cpr, (int)blockIdx.x % a.rq_cpr, a.rq_cpr, a.rq_wpc, smem,
-                             rot_sh, warp - kConvWarp0, lane, csync, a.wait_cycles, a.err);
+        fused_rotate_rows<RG>(a.rq, (int)blockIdx.x, a.rq_cpr, a.rq_wpc, a.rq_rpc, smem, rot_sh, warp - kConvWarp0, lane,
+                              csync, a.wait_cycles, a.err);
         if (ctid == 0) DPTQ_TRACE_POINT(tr, 126);
         fence_proxy_async_smem();   // the ring's copies overwrite what was read and written here
         csync();                    // every converter thread's code and scale stores precede the release
@@ -1249,6 +1250,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   a.rq_np = np;
   a.rq_cpr = 0;
   a.rq_wpc = 0;
+  a.rq_rpc = 1;
   a.rq_items = 0;
   a.rq_shortfall = 0;
   a.wait_cycles = kWaitTimeoutCycles;
@@ -1260,13 +1262,21 @@ bool plan_gemm(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, b
 }
 
 bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, int items) {
-  const bool fused = items > 0;
-  if (!plan_gemm(M, N, K_pad, bits, num_sms, plan, fused)) return false;
-  if (M <= 64) {
-    // The general plan keeps a CTA for each of two or four parts of a row; the rotation takes
-    // `items` CTAs, so whole tiles (or halves in clusters) may run on fewer.
+  if (items > 0) {
+    // One launch: the grid holds the CTAs that rotate rows.  The general plan (four or two CTAs a
+    // row) where it exists, or whole tiles, or halves in clusters, on fewer.
     GemmPlan p;
-    if (plan_tiles(M, N, K_pad, bits, num_sms, p, fused, 0, 0, fused ? items : 1) && p.grid >= items) plan = p;
+    const bool general = plan_gemm(M, N, K_pad, bits, num_sms, plan, true);
+    if (plan_tiles(M, N, K_pad, bits, num_sms, p, true, 0, 0, items) && p.grid >= items) {
+      plan = p;
+      return true;
+    }
+    return general && plan.grid >= items;
+  }
+  if (!plan_gemm(M, N, K_pad, bits, num_sms, plan)) return false;
+  if (M <= 64) {
+    GemmPlan p;
+    if (plan_tiles(M, N, K_pad, bits, num_sms, p, false, 0, 0, 1)) plan = p;
     return true;
   }
   if (K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;

@@ -729,11 +729,12 @@ __device__ __forceinline__ void unit_store(const RQArgs& a, const UnitGeom<G>& u
 }
 
 // ---------------------------------------------------------------- fused decode launch
-// Row `row` of the token rows, or its share `part` of `cpr` (1 or 2 CTAs a row, up to 8 units
-// each), by the 8 converter warps of one CTA of the fused GEMM, into the operand planes:
-// a unit per warp, the row maximum through `sh` (32 words, zero before), and between the two
-// CTAs of a row through its line of a.pmax in global memory (words 0, 1: 1 + the bits of
-// each maximum, 0 = not yet written; words 4, 5 the same for rows in 64-bit integers).
+// Token rows by the 8 converter warps of CTA `item` of the fused GEMM, into the operand
+// planes, a unit per warp: `rpc` rows (8 / wpc at most, wpc warps each), or one row, or the
+// half item % 2 of a row of more than 8 units (cpr = 2).  A row's maximum meets in `sh` (32
+// words; 16 .. 23 zero before), and between the two CTAs of a row in its line of a.pmax in
+// global memory (words 0, 1: 1 + the bits of each maximum, 0 = not yet written; words 4, 5
+// the same for rows in 64-bit integers).
 __device__ __forceinline__ uint32_t row_max_exchange(uint32_t* slots, int part, uint32_t mine, long long wait_cycles,
                                                      int* err) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(slots + part), "r"(mine + 1u) : "memory");
@@ -751,15 +752,19 @@ __device__ __forceinline__ uint32_t row_max_exchange(uint32_t* slots, int part, 
 }
 
 template <int G, class Sync>
-__device__ __forceinline__ void fused_rotate_row(const RQArgs& a, int row, int part, int cpr, int wpc, uint8_t* smem,
-                                                 uint32_t* sh, int wc, int lane, Sync sync, long long wait_cycles,
-                                                 int* err) {
+__device__ __forceinline__ void fused_rotate_rows(const RQArgs& a, int item, int cpr, int wpc, int rpc, uint8_t* smem,
+                                                  uint32_t* sh, int wc, int lane, Sync sync, long long wait_cycles,
+                                                  int* err) {
   uint32_t* const red = sh;            // [8] warp maxima
   uint32_t* const l1s = sh + 8;        // [8]
-  uint32_t* const lead = sh + 16;
-  uint32_t* const bc = sh + 17;
+  uint32_t* const lead = sh + 16;      // [8], the row's first warp's
+  uint32_t* const bc = sh + 24;
   const int tid = wc * 32 + lane;
-  const UnitGeom<G> u(a, part * wpc + wc, lane, a.KB * 128);
+  const int part = cpr > 1 ? item % cpr : 0;
+  const int row0 = cpr > 1 ? item / cpr : item * rpc;
+  const int slot = wc / wpc;           // the warp's row of the CTA's
+  const int row = row0 + slot;
+  const UnitGeom<G> u(a, part * wpc + wc - slot * wpc, lane, a.KB * 128);
   RowOut dst;
   dst.p = static_cast<uint8_t*>(a.out);
   dst.plane = (size_t)a.KB * a.rows_out * 128;
@@ -768,7 +773,7 @@ __device__ __forceinline__ void fused_rotate_row(const RQArgs& a, int row, int p
   dst.bits = a.bits;
   // debug builds: the row is one of the planes' (site 4), its units lie inside it (site 5)
   // and its slots are one of the 64 lines (site 6)
-  const bool act = wc < wpc && u.in && DPTQ_CHECK(row < a.rows_in && row < a.rows_out, err, 4) &&
+  const bool act = slot < rpc && row < a.rows_in && u.in && DPTQ_CHECK(row >= 0 && row < a.rows_out, err, 4) &&
                    DPTQ_CHECK(u.load_end <= a.K && u.store_end <= a.KB * 128, err, 5);
   uint64_t v[32];
   uint32_t m = 0u;
@@ -790,42 +795,58 @@ __device__ __forceinline__ void fused_rotate_row(const RQArgs& a, int row, int p
                                      asm volatile("bar.sync %0, %1;" ::"r"(2 + wc / G), "n"(32 * G) : "memory");
                                  },
                                  [] {}, v);
-    m = unit_max(v, u.l, lead, lane, a.c_hi, a.c_lo);
+    m = unit_max(v, u.l, lead + slot, lane, a.c_hi, a.c_lo);
     if (!ok) m = kRowSlow;
   }
   if (lane == 0) red[wc] = m;
   sync();
-  m = __reduce_max_sync(0xffffffffu, red[lane & 7]);
-  uint32_t* const slots = a.pmax + kRowMaxStride * row;
+  // Maximum of the warps of row slot s (any s; the same in every thread).
+  auto slot_max = [&](int s) { return __reduce_max_sync(0xffffffffu, (lane & 7) / wpc == s ? red[lane & 7] : 0u); };
+  // Whether any row of the CTA leaves the pair form, before red is used again.
+  const uint32_t any = __reduce_max_sync(0xffffffffu, red[lane & 7]);
+  m = slot_max(slot);
+  uint32_t* const slots = a.pmax + kRowMaxStride * row0;
   auto across = [&](uint32_t mine, int off) -> uint32_t {   // the row's maximum over its CTAs
-    if (cpr == 1 || !DPTQ_CHECK(row < 64 && part < cpr && cpr <= 2, err, 6)) return mine;
+    if (cpr == 1 || !DPTQ_CHECK(row0 < 64 && part < cpr && cpr <= 2, err, 6)) return mine;
     if (tid == 0) *bc = row_max_exchange(slots + off, part, mine, wait_cycles, err);
     sync();
     return *(volatile uint32_t*)bc;
   };
-  m = across(m, 0);
+  if (cpr > 1) m = across(m, 0);   // (one row: slot 0 in every warp that counts)
   const float qmaxf = (float)((1 << (a.bits - 1)) - 1);
-  if (m == kRowSlow) {
+  if (act && m != kRowSlow) {
+    const float amax = __uint_as_float(m);
+    const float s = __fdiv_rn(amax, qmaxf);
+    if (part == 0 && wc == slot * wpc && lane == 0) a.scales[row] = s;
+    unit_store<kRQAct, G>(a, u, v, amax, s, dst);
+  }
+  if ((cpr > 1 ? m : any) != kRowSlow) return;
+  // Rows in 64-bit integers, one after the other by all the warps.
+  uint32_t slow = 0u;
+  if (cpr > 1)
+    slow = 1u;
+  else
+    for (int sl = 0; sl < rpc; ++sl) slow |= slot_max(sl) == kRowSlow ? 1u << sl : 0u;
+  sync();   // red and the exchange are free
+#pragma unroll 1
+  for (; slow; slow &= slow - 1u) {
+    const int r = row0 + __ffs(slow) - 1;
+    dst.row = r;
     const int k0 = UnitGeom<G>::first(a, part * wpc), k1 = UnitGeom<G>::first(a, (part + 1) * wpc);
-    rotate_slow_row<kRQAct>(a, row, k0, k1, kUnit * G, smem, tid, 256, sync, dst, [&](float mine) {
+    rotate_slow_row<kRQAct>(a, r, k0, k1, kUnit * G, smem, tid, 256, sync, dst, [&](float mine) {
       const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mine));
       sync();
       if (lane == 0) red[wc] = wm;
       sync();
       const float rm = __uint_as_float(across(__reduce_max_sync(0xffffffffu, red[lane & 7]), 4));
-      if (part == 0 && tid == 0) a.scales[row] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
+      if (part == 0 && tid == 0) a.scales[r] = rm > 0.f ? __fdiv_rn(rm, qmaxf) : 0.f;
       return rm;
     });
     if (part == cpr - 1) {
       const float zero[4] = {0.f, 0.f, 0.f, 0.f};
       for (int kz = a.K + 4 * tid; kz < a.KB * 128; kz += 4 * 256) store_codes<kRQAct, 4>(dst, kz, zero);
     }
-    return;
   }
-  const float amax = __uint_as_float(m);
-  const float s = __fdiv_rn(amax, qmaxf);
-  if (part == 0 && tid == 0) a.scales[row] = s;
-  if (act) unit_store<kRQAct, G>(a, u, v, amax, s, dst);
 }
 
 }  // namespace dptq

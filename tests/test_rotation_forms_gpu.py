@@ -95,3 +95,25 @@ def test_operand_planes_hold_the_public_codes(dp, K, B, bits):
     assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
     dp.dptq_last_device_error()
     layer.close()
+
+
+# one row a CTA, two CTAs a row, several rows side by side in a CTA (1, 2 and 4 warps each, a
+# last CTA that is not full), whole tiles and clusters of two and four CTAs
+@pytest.mark.parametrize("M,N,K,B", [(16, 512, 256, 256), (13, 128, 1024, 1024), (64, 256, 2048, 2048),
+                                     (33, 128, 4096, 4096), (64, 1024, 4096, 2048), (7, 4096, 11008, 256),
+                                     (32, 6144, 4096, 4096), (21, 8192, 1536, 512)])
+@pytest.mark.parametrize("bits", [4, 8])
+def test_one_launch_equals_two(dp, M, N, K, B, bits):
+    base = rows_of_every_kind(K)
+    x = torch.from_numpy(np.concatenate([base] * (-(-M // 7)))[:M]).to(DEV)
+    x[7:] *= torch.linspace(0.2, 1.0, max(1, M - 7), device=DEV)[:max(0, M - 7), None].half()
+    layer = dp.dptq_pack_weights(torch.from_numpy(inputs.weights(N, K, layer=3)).to(DEV), B)
+    one = torch.empty((M, N), dtype=torch.float16, device=DEV)
+    two = torch.empty((M, N), dtype=torch.float16, device=DEV)
+    for _ in range(2):
+        dp.dptq_qlinear(layer, x, bits, one)
+    dp.dptq_qlinear_quantize(layer, x, bits)
+    dp.dptq_qlinear_gemm(layer, M, bits, two)
+    assert torch.equal(one.view(torch.int16), two.view(torch.int16))
+    dp.dptq_last_device_error()
+    layer.close()
