@@ -247,11 +247,12 @@ dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused
 
 /* The plan that a launch takes, in the order of dptq_plan_info, then 20 the CTAs that share
  * the stream-K stages (as many as tiles: whole tiles) and 21 the CTAs of a cluster that
- * share a weight tile (2 or 4, or 1: none).  row_ctas = 0: a GEMM launch (dptq_qlinear_gemm,
+ * share a weight tile (2 or 4, or 1: none), 22 the CTAs that share a token tile (2: fields 16, 17 and 20
+ * count pairs of weight tiles and of CTAs; or 1).  row_ctas = 0: a GEMM launch (dptq_qlinear_gemm,
  * dptq_qgemm_codes, and dptq_qlinear where it does not run as one launch); otherwise the
  * one-launch kernel, with that many CTAs rotating token rows (one per token, two for
  * K > 8192, or on small grids one for several tokens).  Host only; errors as dptq_plan_info, and INVALID_ARG for row_ctas < 0. */
-#define DPTQ_LAUNCH_PLAN_LEN 22
+#define DPTQ_LAUNCH_PLAN_LEN 23
 dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int row_ctas, int* info, int info_len);
 
 /* Copy the packed weights out in the public layout: wq_host uint8 [N][K/2] (same

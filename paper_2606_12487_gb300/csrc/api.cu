@@ -747,7 +747,7 @@ void write_plan(const GemmPlan& plan, int* info, int len) {
                                        g.conv_slots, plan.a_tmem ? 1 : 0, g.nbuf, g.segs, g.seg_iters,
                                        (int)g.tmem_cols, (int)g.a_col0, g.KI, g.n_wtiles, g.m_tiles, g.dp_tiles,
                                        sk > 0x7fffffffLL ? 0x7fffffff : (int)sk, g.rq_np, plan.fused ? 1 : 0,
-                                       g.sk_ctas, g.cl};
+                                       g.sk_ctas, g.cl, g.pair};
   for (int i = 0; i < len; ++i) info[i] = v[i];
 }
 dptq_status check_plan_args(int M, int N, int K, int bits, int num_sms, const int* info, int info_len, int want) {

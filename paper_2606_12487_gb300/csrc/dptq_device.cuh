@@ -210,6 +210,13 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
+// Arrive on another CTA's mbarrier (an address of cluster_map).  For tensor-memory stores and
+// bulk copies that this thread has already seen complete: a release at cluster scope would wait
+// for more and takes longer than a whole stage (266 instead of 140 us for M = 2048, N = 28672, K
+// = 4096).
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // 16 bytes into another CTA's shared memory, counted on its mbarrier.
 __device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
@@ -240,16 +247,31 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 
 // ------------------------------------------------------------------ tcgen05 / TMEM
+// (PAIR: by one warp of each CTA of a pair; a kernel uses one group size throughout.)
+template <bool PAIR>
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
-               "r"(ncols)
-               : "memory");
+  if constexpr (PAIR)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
+                 "r"(ncols)
+                 : "memory");
+  else
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
+                 "r"(ncols)
+                 : "memory");
 }
+template <bool PAIR>
 __device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  if constexpr (PAIR)
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  else
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+template <bool PAIR>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+  if constexpr (PAIR)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+  else
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -294,6 +316,28 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// Pairs of CTAs (cta_group::2).  D: this CTA's 128 rows in each CTA's tensor memory; A: the same
+// rows, in the same columns of each CTA's tensor memory; B: half of the columns in each CTA's
+// shared memory, at the same place.  Issued by the pair's first CTA.
+__device__ __forceinline__ void mma_f8_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrive once on the barrier at this place in both CTAs when every MMA issued so far by this
+// thread has completed.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand in the 128-byte swizzle layout
 // (8-row x 128-byte atoms, rows 128 B apart, atoms 1024 B apart; base 1024-aligned).
 __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
@@ -304,12 +348,13 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
          | ((uint64_t)2 << 61);                // swizzle mode: 128-byte
 }
 
-// Instruction descriptor: kind::f8f6f4, A = B = E4M3, D = F32, both K-major, M = 128.
-__host__ __device__ constexpr uint32_t idesc_e4m3_m128(int n) {
+// Instruction descriptor: kind::f8f6f4, A = B = E4M3, D = F32, both K-major, M rows (128,
+// or 256: 128 in each CTA of a pair).
+__host__ __device__ constexpr uint32_t idesc_e4m3(int m, int n) {
   return (1u << 4)                        // D format F32
          | (0u << 7) | (0u << 10)         // A, B format E4M3
          | ((uint32_t)(n >> 3) << 17)     // N / 8
-         | ((uint32_t)(128 >> 4) << 24);  // M / 16
+         | ((uint32_t)(m >> 4) << 24);    // M / 16
 }
 
 // 32 TMEM lanes (one per thread of the warp) x 16 consecutive 32-bit columns.

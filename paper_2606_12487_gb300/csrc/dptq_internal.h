@@ -128,6 +128,8 @@ struct GemmArgs {
   long long sk_iters;  // stream-K iterations (tiles after dp_tiles, times KI)
   int sk_ctas;         // CTAs that share them evenly (as many as tiles: whole tiles)
   uint32_t tmem_cols;
+  int pair;            // 2: pairs of CTAs multiply a token tile by two weight tiles together (dp_tiles,
+                       // sk_iters and sk_ctas count pairs of tiles and of CTAs), else 1
   int cl;              // CTAs of a cluster that share a weight tile's k range (1: no cluster)
   int out_vec;         // `out` is 16-byte aligned: the epilogue stores 8 channels at a time
   // Fused decode launches only: the rotation + quantization of the M_pad token rows

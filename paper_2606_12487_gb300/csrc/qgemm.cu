@@ -81,9 +81,9 @@ struct UnitIter {
 
   __device__ __forceinline__ uint32_t sk_begin(uint32_t c) const { return (c * sk_iters) / skG; }
   __device__ __forceinline__ uint32_t cta_of(uint32_t i) const { return ((i + 1) * skG - 1) / sk_iters; }
-  __device__ __forceinline__ void init(const GemmArgs& a) {
-    cta = blockIdx.x;
-    G = gridDim.x;
+  __device__ __forceinline__ void init(const GemmArgs& a, uint32_t ctas) {   // `ctas` work together
+    cta = blockIdx.x / ctas;
+    G = gridDim.x / ctas;
     KI = (uint32_t)a.KI;
     dp_tiles = (uint32_t)a.dp_tiles;
     dp_next = cta;
@@ -253,7 +253,17 @@ __device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT,
 // fills only afterwards; the other CTAs fill their rings from the start.  The rows are published on a grid counter;
 // every activation producer waits for all of them; the epilogue reads the token scales after
 // the same point, and the last CTA to get there resets the counters and the slots.
-template <int NT, int KPS, int RG>
+//
+// PAIR (192-token tiles): two CTAs multiply a token tile by two weight tiles with MMAs of M =
+// 256 (cta_group::2), each holding half of the tile's tokens.  One CTA's stages are bound by its
+// shared memory: two k-blocks bring 48 KB of codes and 16 KB of weights in and read them out
+// again, 128 KB or 1000 clocks at 128 bytes a clock, of the 990 a stage takes; its MMAs take 768.
+// In a pair it is 80 KB, and what remains above the MMAs is the way round a widened slot (two fit
+// beside the accumulators): commit, widen, tell the first CTA.  That one issues every MMA and its
+// commits arrive in both; the second CTA's converters arrive on its `pfull` themselves (through
+// that CTA's MMA warp: 140.6 instead of 139.3 us at M = 2048, N = 28672, K = 4096), and the MMA
+// warp tells of landed codes and, with a unit's first stage, of a free accumulator.
+template <int NT, int KPS, int RG, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a) {
   constexpr bool FUSED = RG != 0;
   // Two-block stages (token tiles of up to 64, weight streaming) and 192-token tiles
@@ -268,11 +278,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   constexpr bool kAltConv = kPairConv && NT <= 64;
   // Clusters of two or four CTAs, each with its part of a weight tile's k range (small N).
   constexpr bool kClusterTiles = NT <= 64 && KPS == 2;
+  constexpr int kActRows = PAIR ? NT / 2 : NT;   // tokens of a tile in this CTA
+  static_assert(!PAIR || kATmem, "pairs take the widened weights from tensor memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = a.stages;
   const int CS = a.conv_slots;
-  const Smem<NT, KPS> sm(smem, a.planes, kATmem ? 0 : CS);
+  const Smem<kActRows, KPS> sm(smem, a.planes, kATmem ? 0 : CS);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm.end(S));
   uint64_t* full = bars;                     // slot s: weight copies landed
   uint64_t* empty = bars + kMaxStages;       // slot s: MMA done with it
@@ -285,7 +297,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   uint64_t* aready = esync + 1;  // fused: all token rows are quantized (producer -> epilogue)
   uint64_t* rdone = aready + 1;  // fused: this CTA's row is quantized, the ring's memory is free
   uint64_t* xbar = rdone + 1;    // cluster: the other CTAs' partial sums landed
-  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(xbar + 1);
+  uint64_t* pfull = xbar + 1;    // pairs, in the first CTA: the second is ready for the MMAs of slot s
+  uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(pfull + kMaxStages);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_sh + 1);
   volatile int* flags = reinterpret_cast<volatile int*>(tmem_base_sh + 2);   // epilogue: 2 units x 2
   float* sa_sh = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);   // token scales (NT <= 64)
@@ -303,6 +316,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
       mbar_init(&afull[s], 1);
+      mbar_init(&pfull[s], kNumConvWarps + 1);
     }
     for (int c = 0; c < CS; ++c) {
       mbar_init(&cfull[c], kAltConv ? kNumConvWarps / 2 : kNumConvWarps);
@@ -323,15 +337,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_base_sh, a.tmem_cols);
-    tmem_relinquish();
+    tmem_alloc<PAIR>(tmem_base_sh, a.tmem_cols);
+    tmem_relinquish<PAIR>();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const bool clustered = kClusterTiles && a.cl > 1;
+  const bool ksplit = kClusterTiles && a.cl > 1;
+  const int rank = PAIR ? (int)(blockIdx.x & 1u) : 0;
+  const bool clustered = ksplit || PAIR;
   if (clustered) {
-    if (threadIdx.x == 0) mbar_arrive_expect_tx(xbar, (uint32_t)((a.cl - 1) * (NT / a.cl) * 128 * 4));
+    if (ksplit && threadIdx.x == 0) mbar_arrive_expect_tx(xbar, (uint32_t)((a.cl - 1) * (NT / a.cl) * 128 * 4));
     cluster_arrive();   // this CTA's barrier may be counted on by the others
   }
   const uint32_t tmem_base = *tmem_base_sh;
@@ -339,7 +355,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   pdl_launch_dependents();
 
   UnitIter iter;
-  iter.init(a);
+  iter.init(a, PAIR ? 2u : 1u);
   Unit un;
   bool cluster_waited = false;   // this thread has waited for the cluster's first barrier
 
@@ -357,7 +373,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     if (leader && wprod) DPTQ_TRACE_POINT(tr, 117);
     const uint64_t pol_w = l2_policy_evict_first();   // weights are streamed once
     const uint64_t pol_a = l2_policy_evict_last();    // activations are re-read per n-tile
-    const uint32_t act_bytes = (uint32_t)NT * 128;
+    const uint32_t act_bytes = (uint32_t)kActRows * 128;
     const uint32_t w_bytes = (uint32_t)KPS * kWTileBytes;
     const uint32_t a_tx = (uint32_t)(KPS * a.planes) * act_bytes;
     const size_t plane_stride = (size_t)a.KB * a.M_pad * 128;
@@ -405,11 +421,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     Ring rg(S);
     int g = 0;
     while (ok && iter.next(un)) {
-      const int nt = un.tile / a.m_tiles;
-      const int mt = un.tile - nt * a.m_tiles;
+      const int np = un.tile / a.m_tiles;
+      const int mt = un.tile - np * a.m_tiles;
+      const int nt = PAIR ? 2 * np + rank : np;
       if (leader && wprod) DPTQ_TRACE_POINT(tr, 118);
       const uint8_t* wsrc = a.wt + ((size_t)nt * a.KB + (size_t)un.i0 * KPS) * kWTileBytes;
-      const uint8_t* asrc = a.act + ((size_t)un.i0 * KPS * a.M_pad + (size_t)mt * NT) * 128;
+      const uint8_t* asrc = a.act + ((size_t)un.i0 * KPS * a.M_pad + (size_t)mt * NT + (size_t)rank * kActRows) * 128;
       for (int it = un.i0; it < un.i1; ++it, ++g, rg.next(), wsrc += w_bytes, asrc += KPS * kb_stride) {
         const int s = rg.s;
         const bool tg = kTraceStages > 10 && wprod && leader && g >= 8 && g < 11;   // clocked stages (trace builds)
@@ -452,6 +469,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         __syncwarp();
       }
     }
+    if (PAIR && !wprod && ok) {   // the commits that the other CTA's MMAs owe this one have arrived
+      for (int i = 0; i < S; ++i, rg.next())
+        mbar_wait_warp(&empty[rg.s], rg.ph ^ 1u, abort_flag, a.err, kDevTimeoutEmpty, a.wait_cycles);
+    }
     __syncwarp();
     // Do not leave the CTA while copies into its shared memory may be in flight: after an
     // abort, wait (bounded) for the copies this warp armed in the last S stages.
@@ -468,16 +489,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     // the MMAs of the thread that issues it.  Descriptors and TMEM addresses advance by
     // additions, segment boundaries by a countdown.
     const bool leader = elect_one();
-    const uint32_t idesc = idesc_e4m3_m128(NT);
+    const auto commit = [](uint64_t* bar) { PAIR ? mma_commit_pair(bar) : mma_commit(bar); };
+    const uint32_t idesc = idesc_e4m3(PAIR ? 256 : 128, NT);
     const int planes = a.planes;
     // Shared-memory descriptors hold address >> 4 in their low bits, so a byte offset
     // `o` into a region is `desc + (o >> 4)`.
     const uint64_t act_desc0 = sdesc_sw128(smem_u32(sm.act(0, 0, 0)));
     const uint64_t conv_desc0 = kATmem ? 0 : sdesc_sw128(smem_u32(sm.conv(0, 0)));
     const uint32_t slot_step = (uint32_t)(sm.slot_bytes >> 4);
-    const uint32_t act_step = (uint32_t)(Smem<NT, KPS>::kActBytes >> 4);
+    const uint32_t act_step = (uint32_t)(Smem<kActRows, KPS>::kActBytes >> 4);
     const uint32_t a_tmem0 = tmem_base + a.a_col0;
     Ring rg(S), rc(CS);
+    if constexpr (PAIR) {
+      cluster_wait();   // the other CTA's barriers are initialized
+      cluster_waited = true;
+    }
+    const uint32_t peer_full = PAIR ? cluster_map(smem_u32(pfull), 0) : 0;
     int u = 0, mma_done = 0;
     while (iter.next(un)) {
       const int b = a.nbuf == 2 ? (u & 1) : 0;
@@ -494,7 +521,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         const bool tgm = kTraceStages > 10 && leader && gm >= 8 && gm < 11;   // stages whose steps are clocked (trace builds)
         (void)tgm;
         if (tgm) DPTQ_TRACE_CLOCK(tr, 200 + 8 * (gm - 8));
+        if constexpr (PAIR) {
+          if (rank != 0) {   // (its converters tell the first CTA themselves)
+            if (!mbar_wait_warp(&afull[s], rg.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
+              ok = false;
+              break;
+            }
+            tc_fence_before();
+            if (leader) mbar_arrive_remote(peer_full + 8u * (uint32_t)s);
+            continue;
+          }
+        }
         if (!mbar_wait2_warp(&cfull[c], rc.ph, &afull[s], rg.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
+          ok = false;
+          break;
+        }
+        if (PAIR && !mbar_wait_warp(&pfull[s], rg.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -519,7 +561,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks) {   // 4 x (K = 32 FP8 elements = 32 bytes = 8 columns)
                   const uint32_t accumulate = (h | p | ks) ? 1u : (fresh ^ 1u);
-                  if (kATmem)
+                  if (PAIR)
+                    mma_f8_ts_pair(d, at + (uint32_t)(8 * ks), bd + 2 * ks, idesc, accumulate);
+                  else if (kATmem)
                     mma_f8_ts(d, at + (uint32_t)(8 * ks), bd + 2 * ks, idesc, accumulate);
                   else
                     mma_f8(d, ad + 2 * ks, bd + 2 * ks, idesc, accumulate);
@@ -531,7 +575,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
           // One commit per stage: it frees the bulk-copy slot (producer) and tells the
           // converters that widened slot c may be overwritten (they wait on the same
           // barrier, one ring position CS stages back).
-          mma_commit(&empty[s]);
+          commit(&empty[s]);
           if (tgm) DPTQ_TRACE_CLOCK(tr, 205 + 8 * (gm - 8));
           if (gm < kTraceStages) DPTQ_TRACE_POINT(tr, 88 + gm);
         }
@@ -540,14 +584,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         --seg_left;
       }
       if (!ok) break;
-      if (leader) mma_commit(&tfull[b]);
+      if (leader && rank == 0) commit(&tfull[b]);
       __syncwarp();
       mma_done += un.i1 - un.i0;
       ++u;
     }
     if (leader) DPTQ_TRACE_POINT(tr, 124);   // last MMA issued
     // Every MMA the leader issued must be complete before TMEM is released.
-    if (leader) mma_commit(drain);
+    if (leader && rank == 0) commit(drain);
     __syncwarp();
     volatile int no_abort = 0;
     mbar_wait_warp(drain, 0, &no_abort, a.err, kDevTimeoutDrain);
@@ -575,6 +619,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     }
     // rl trails rg by CS stages: the MMA of stage gc - CS was the last to read widened
     // slot c, and its commit completes that stage's `empty` barrier.
+    if constexpr (PAIR) {
+      cluster_wait();   // the other CTA's barriers are initialized
+      cluster_waited = true;
+    }
+    const uint32_t peer_full = PAIR ? cluster_map(smem_u32(pfull), 0) : 0;
     Ring rg(S), rc(CS), rl(S);
     const int grp = (warp - kConvWarp0) >> 2;   // converter group (alternate stages)
     const int tid_grp = (warp - kConvWarp0 - 4 * grp) * 32 + lane;
@@ -696,7 +745,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
           if (ctid == 0 && gc == 8) DPTQ_TRACE_CLOCK(tr, 233);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&cfull[c]);
+        if (lane == 0) {
+          if (PAIR && rank != 0)
+            mbar_arrive_remote(peer_full + 8u * (uint32_t)s);
+          else
+            mbar_arrive(&cfull[c]);
+        }
         if (tgc) DPTQ_TRACE_CLOCK(tr, 185 + 6 * (gc - 8));
         if ((kAltConv ? tid_grp == 0 : ctid == 0) && gc < kTraceStages) DPTQ_TRACE_POINT(tr, 56 + gc);
       }
@@ -748,8 +802,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
     while (epi_ok && iter.next(un)) {
       const int b = a.nbuf == 2 ? (u & 1) : 0;
       const uint32_t tpar = (a.nbuf == 2 ? (u >> 1) : u) & 1;
-      const int nt = un.tile / a.m_tiles;
-      const int mt = un.tile - nt * a.m_tiles;
+      const int np = un.tile / a.m_tiles;
+      const int mt = un.tile - np * a.m_tiles;
+      const int nt = PAIR ? 2 * np + rank : np;
+      if (un.slot >= 0) un.slot = PAIR ? 2 * un.slot + rank : un.slot;   // (a slot for each weight tile)
       const int n = nt * 128 + q * 32 + lane;
       const int m0 = mt * NT;
       // Scales are fetched while the MMAs of this unit still run.  Tiles of more than 64
@@ -768,7 +824,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       // Split tile: whether every other contributor is already in is asked while the MMAs
       // still run, and once more after them if not.
       volatile int* const flag = flags + 2 * (u & 1);   // [0]: all others in, [1]: last
-      const bool split = un.slot >= 0 && !clustered;
+      const bool split = un.slot >= 0 && !ksplit;
       if (split) {
         if (etid == 0) *flag = ld_acquire_gpu(a.counters + un.slot) == (uint32_t)(un.contributors - 1);
         if (!epi_sync()) break;
@@ -777,7 +833,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       if (etid == 0 && u < 4) DPTQ_TRACE_POINT(tr, 104 + u);
       tc_fence_after();
       if constexpr (kClusterTiles) {
-        if (clustered) {
+        if (ksplit) {
           const uint32_t acc = tmem_base + lane_base + (uint32_t)(b * NT);
           epi_ok = a.cl == 2 ? cluster_finish<NT, KPS, 2>(a, sm, bars, xbar, xpose, sa_sh, acc, n, nt, q, lane, abort_flag)
                              : cluster_finish<NT, KPS, 4>(a, sm, bars, xbar, xpose, sa_sh, acc, n, nt, q, lane, abort_flag);
@@ -1039,7 +1095,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, a.tmem_cols);
+    tmem_dealloc<PAIR>(tmem_base, a.tmem_cols);
   }
   if (threadIdx.x == 0) DPTQ_TRACE_POINT(tr, 120);
 }
@@ -1061,8 +1117,8 @@ int gemm_pick_nt(int M, int bits, int KB) {
 // wide tiles keep one k-block per stage for a deeper ring.
 static int kps_for(int nt) { return nt <= 64 || nt == 192 ? 2 : 1; }
 
-static int smem_for(int nt, int kps, int stages, int planes, int conv_slots) {
-  return 1024 + conv_slots * kps * kConvBytes + stages * kps * (planes * nt * 128 + kWTileBytes) + kBarrierBytes;
+static int smem_for(int act_rows, int kps, int stages, int planes, int conv_slots) {
+  return 1024 + conv_slots * kps * kConvBytes + stages * kps * (planes * act_rows * 128 + kWTileBytes) + kBarrierBytes;
 }
 
 // Launch time of a GEMM of more than 64 tokens in microseconds, by token tile: fixed +
@@ -1075,10 +1131,23 @@ static int smem_for(int nt, int kps, int stages, int planes, int conv_slots) {
 //   M = 333, N = 1024 / 4096, K = 4096: 16.1 -> 8.8 / 21.6 -> 14.8 us
 //   M = 512, N = K = 4096: 23.9 -> 15.0 us; M = 2048: 38.1 -> 33.0 us (192, whole)
 //   M = 2048, N = 28672, K = 4096: 163 -> 157 us (192, 17 whole waves)
+// Pairs of CTAs (an even number of weight tiles): stages of 0.484 us (one CTA: 0.515), but a
+// fixed cost higher by the tensor memory and barriers of two CTAs, so that one wave of them loses
+// (M = 700, N = K = 4096: 16.1 -> 16.6 us) and two win (M = 333, N = 12288: 25.2 -> 23.4 us).  The
+// partial sums of a split tile are hidden behind the other tile's stages as far as it has them
+// (M = 2048, N = 4096: split against whole 36.6 / 31.0 us at K = 4096, 73.1 / 82.7 at K = 14336).
+// Against one CTA, GEMM alone: M = 2048, K = 4096, N = 4096 / 12288 / 28672: 32.8 -> 31.0, 68.4 ->
+// 63.0, 157 -> 140 us; N = 4096, K = 14336: 82.4 -> 73.1 us; A8, M = 4096: N = 5120, K = 13824:
+// 369 -> 310 us, N = K = 8192: 312 -> 288 us.
 struct TileCost {
   double stage, fixed, split, apart;
 };
-static TileCost tile_cost(int nt, int planes) {
+static TileCost tile_cost(int nt, int planes, bool pair, int KI) {
+  if (pair) {
+    const double stage = planes == 1 ? 0.484 : 0.40;
+    const double split = 14.0 - 0.3 * stage * KI;
+    return TileCost{stage, planes == 1 ? 8.3 : 8.5, split > 4.0 ? split : 4.0, 11.0};
+  }
   if (nt == 64) return planes == 1 ? TileCost{0.336, 4.0, 4.5, 4.5} : TileCost{0.42, 4.5, 4.5, 4.5};
   if (nt == 192) return planes == 1 ? TileCost{0.515, 7.6, 8.0, 11.0} : TileCost{0.42, 7.3, 8.0, 11.0};
   return planes == 1 ? TileCost{0.41, 8.0, 5.0, 5.0} : TileCost{0.45, 8.0, 5.0, 5.0};
@@ -1088,7 +1157,7 @@ static TileCost tile_cost(int nt, int planes) {
 // planes (0: a multiple of the tile).  items > 0 (decode tiles): the grid needs only that many
 // CTAs for the rows' rotation (fused; 1 otherwise) and may be smaller than the general plan's.
 static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan, bool fused, int nt_forced,
-                       int M_pad_forced, int items = 0) {
+                       int M_pad_forced, int items = 0, bool pair = false) {
   GemmArgs& a = plan.args;
   const int KB = K_pad / kKBlock;
   const int planes = bits == 8 ? 2 : 1;
@@ -1134,7 +1203,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   if (fused && (kps != 2 || nt > 64)) return false;
   // Decode tiles may be finished by clusters, which receive partial sums in shared memory.
   const int xch = nt <= 64 && kps == 2 && segs == 1 ? (kCluster - 1) * (nt / kCluster) * 128 * 4 : 0;
-  auto smem_total = [&](int st) { return smem_for(nt, kps, st, planes, smem_conv) + xch; };
+  auto smem_total = [&](int st) { return smem_for(pair ? nt / 2 : nt, kps, st, planes, smem_conv) + xch; };
   int stages = kMaxStages;
   while (stages > 2 && smem_total(stages) > kSmemLimit) --stages;
   if (smem_total(stages) > kSmemLimit) return false;
@@ -1154,7 +1223,9 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   const int M_pad = M_pad_forced > 0 ? M_pad_forced : round_up(M, nt);
   const int n_wtiles = ceil_div(N, 128);
   const int m_tiles = ceil_div(M, nt);
-  const long long tiles = (long long)n_wtiles * m_tiles;
+  if (pair && (nt != 192 || n_wtiles % 2 != 0 || num_sms < 2)) return false;
+  if (pair) num_sms /= 2;   // below, a tile is a pair of tiles and an SM a pair of SMs
+  const long long tiles = (long long)n_wtiles * m_tiles / (pair ? 2 : 1);
   const long long iters = tiles * KI;
   int G = (int)(iters < num_sms ? iters : num_sms);
   if (G < 1) G = 1;
@@ -1185,7 +1256,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   if (M > 64) {
     // Whole tiles in waves, the last one on as many CTAs as it has tiles; or all but the last
     // waves whole and the rest split evenly over the SMs.
-    const TileCost c = tile_cost(nt, planes);
+    const TileCost c = tile_cost(nt, planes, pair, KI);
     const int P = (int)(tiles < num_sms ? tiles : num_sms);
     const double whole = c.fixed + c.stage * KI * ceil_div(tiles, P);
     const double even = c.fixed + (tiles < num_sms ? c.apart : c.split) + c.stage * ((double)tiles * KI / G);
@@ -1205,7 +1276,8 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   plan.nt = nt;
   plan.kps = kps;
   plan.M_pad = M_pad;
-  plan.grid = G;
+  plan.grid = pair ? 2 * G : G;
+  a.pair = pair ? 2 : 1;
   plan.smem_bytes = smem_total(stages);
   a.M = M;
   a.N = N;
@@ -1279,6 +1351,9 @@ bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan,
     if (plan_tiles(M, N, K_pad, bits, num_sms, p, false, 0, 0, 1)) plan = p;
     return true;
   }
+  GemmPlan pairs;
+  if (plan.nt == 192 && plan_tiles(M, N, K_pad, bits, num_sms, pairs, false, 0, 0, 0, true) && pairs.cost < plan.cost)
+    plan = pairs;
   if (K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;
   // The operand planes keep the rows of the wide tiles (192 and 128 are multiples of 64), so
   // that one quantized matrix serves layers of any N.
@@ -1297,9 +1372,9 @@ bool fused_rotation_split(int K, int B, int tail, int& cpr, int& wpc) {
   return cpr <= 2 && wpc <= kNumConvWarps;
 }
 
-template <int NT, int KPS, int RG = 0>
+template <int NT, int KPS, int RG = 0, bool PAIR = false>
 static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
-  cudaError_t e = ensure_max_dyn_smem(qgemm_kernel<NT, KPS, RG>);
+  cudaError_t e = ensure_max_dyn_smem(qgemm_kernel<NT, KPS, RG, PAIR>);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)plan.grid);
@@ -1314,12 +1389,17 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
   }
   cfg.attrs = attr;
   GemmArgs args = plan.args;
-  if (args.cl > 1) {
+  if (PAIR || args.cl > 1) {
     cudaLaunchAttribute* c = &attr[n];
     c->id = cudaLaunchAttributeClusterDimension;
-    c->val.clusterDim.x = (unsigned)args.cl;
+    c->val.clusterDim.x = PAIR ? 2u : (unsigned)args.cl;
     c->val.clusterDim.y = 1;
     c->val.clusterDim.z = 1;
+  }
+  if (PAIR) {
+    ++n;   // (pairs wait for no CTA of another pair)
+  } else if (args.cl > 1) {
+    cudaLaunchAttribute* c = &attr[n];
     // All CTAs have to be resident at once (a fused launch's wait for one another's rows).
     // Asked once per kernel and device, for the largest shared memory.
     static std::atomic<int> most[64];   // resident clusters + 1 (0: not asked yet)
@@ -1333,7 +1413,7 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
       cudaLaunchAttribute only = *c;
       probe.attrs = &only;
       probe.numAttrs = 1;
-      e = cudaOccupancyMaxActiveClusters(&m, qgemm_kernel<NT, KPS, RG>, &probe);
+      e = cudaOccupancyMaxActiveClusters(&m, qgemm_kernel<NT, KPS, RG, PAIR>, &probe);
       if (e != cudaSuccess) return e;
       most[dev].store(++m);
     }
@@ -1343,7 +1423,7 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
       args.cl = 1;   // the tiles' parts meet in global memory instead
   }
   cfg.numAttrs = (unsigned)n;
-  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RG>, args);
+  return cudaLaunchKernelEx(&cfg, qgemm_kernel<NT, KPS, RG, PAIR>, args);
 }
 
 cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
@@ -1369,7 +1449,7 @@ cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
       case 16: return launch_nt<16, 2>(plan, s, pdl);
       case 32: return launch_nt<32, 2>(plan, s, pdl);
       case 64: return launch_nt<64, 2>(plan, s, pdl);
-      case 192: return launch_nt<192, 2>(plan, s, pdl);
+      case 192: return plan.args.pair == 2 ? launch_nt<192, 2, 0, true>(plan, s, pdl) : launch_nt<192, 2>(plan, s, pdl);
       default: return cudaErrorInvalidValue;
     }
   }
@@ -1378,7 +1458,7 @@ cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
     case 32: return launch_nt<32, 1>(plan, s, pdl);
     case 64: return launch_nt<64, 1>(plan, s, pdl);
     case 128: return launch_nt<128, 1>(plan, s, pdl);
-    case 192: return launch_nt<192, 1>(plan, s, pdl);
+    case 192: return plan.args.pair == 2 ? launch_nt<192, 1, 0, true>(plan, s, pdl) : launch_nt<192, 1>(plan, s, pdl);
     case 256: return launch_nt<256, 1>(plan, s, pdl);
     default: return cudaErrorInvalidValue;
   }

@@ -296,9 +296,9 @@ def dptq_plan_info(M: int, N: int, K: int, bits: int, num_sms: int, fused: bool 
 
 
 def dptq_launch_plan(M: int, N: int, K: int, bits: int, num_sms: int, row_ctas: int = 0) -> dict:
-    """The plan that a launch takes (host only): PLAN_INFO_FIELDS, "sk_ctas", "cluster"; row_ctas
+    """The plan that a launch takes (host only): PLAN_INFO_FIELDS, "sk_ctas", "cluster", "pair"; row_ctas
     CTAs of a one-launch call rotate token rows (0: a GEMM launch)."""
-    fields = PLAN_INFO_FIELDS + ("sk_ctas", "cluster")
+    fields = PLAN_INFO_FIELDS + ("sk_ctas", "cluster", "pair")
     buf = (ctypes.c_int * len(fields))()
     _check(load().dptq_launch_plan(M, N, K, bits, num_sms, row_ctas, buf, len(fields)))
     return dict(zip(fields, list(buf)))

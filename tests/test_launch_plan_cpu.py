@@ -13,8 +13,9 @@ MS = [1, 16, 33, 64, 65, 100, 128, 129, 200, 333, 512, 1000, 2048, 8192]
 
 
 def units(p):
-    """(tile, i0, i1, slot, contributors) of every CTA, as the kernel walks them."""
-    G, KI, dp, sk, skG = p["grid"], p["KI"], p["dp_tiles"], p["sk_iters"], p["sk_ctas"]
+    """(tile, i0, i1, slot, contributors) of every CTA (a pair of CTAs: once, for its pair of
+    tiles), as the kernel walks them."""
+    G, KI, dp, sk, skG = p["grid"] // p["pair"], p["KI"], p["dp_tiles"], p["sk_iters"], p["sk_ctas"]
     begin = lambda c: c * sk // skG
     cta_of = lambda i: ((i + 1) * skG - 1) // sk
     for c in range(G):
@@ -55,7 +56,8 @@ def test_every_stage_once(N, K, bits, fused):
                 continue
         p = dptq.dptq_launch_plan(M, N, K, bits, 152, rows)
         assert p["fused"] == int(fused) and p["grid"] >= rows   # a CTA for every row's rotation
-        tiles = p["n_wtiles"] * p["m_tiles"]
+        tiles = p["n_wtiles"] * p["m_tiles"] // p["pair"]
+        assert p["grid"] % p["pair"] == 0 and p["n_wtiles"] % p["pair"] == 0 and (p["pair"] == 1 or p["nt"] == 192)
         assert p["m_tiles"] * p["nt"] >= M and p["m_tiles"] * p["nt"] <= p["M_pad"]
         assert p["smem_bytes"] <= 232448 and p["grid"] <= 152 and p["kps"] * p["KI"] == -(-K // 128)
         parts = {}
