@@ -261,7 +261,7 @@ __device__ __forceinline__ bool cluster_finish(const GemmArgs& a, const Smem<NT,
 // In a pair it is 80 KB, and what remains above the MMAs is the way round a widened slot (two fit
 // beside the accumulators): commit, widen, tell the first CTA.  That one issues every MMA and its
 // commits arrive in both; the second CTA's converters arrive on its `pfull` themselves (through
-// that CTA's MMA warp: 140.6 instead of 139.3 us at M = 2048, N = 28672, K = 4096), and the MMA
+// that CTA's MMA warp: 140.6 instead of 139.3 us for M = 2048, N = 28672, K = 4096), and the MMA
 // warp tells of landed codes and, with a unit's first stage, of a free accumulator.
 template <int NT, int KPS, int RG, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a) {
@@ -276,6 +276,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   // (wide tiles: all eight on the same stage, a k-block per group).
   constexpr bool kPairConv = kATmem && KPS == 2;
   constexpr bool kAltConv = kPairConv && NT <= 64;
+  // Wide tiles have two widened slots only: the next stage's weights are widened in registers
+  // before their slot is waited for (M = 2048, pairs: N = 28672, K = 4096 139.3 -> 136.9 us, N =
+  // 4096, K = 14336 72.4 -> 69.9 us).
+  constexpr bool kEarlyLoad = kPairConv && !kAltConv;
   // Clusters of two or four CTAs, each with its part of a weight tile's k range (small N).
   constexpr bool kClusterTiles = NT <= 64 && KPS == 2;
   constexpr int kActRows = PAIR ? NT / 2 : NT;   // tokens of a tile in this CTA
@@ -645,8 +649,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         // S >= CS, that copy has landed and been consumed once the MMA of stage gc - CS
         // is done.
         const bool fresh = gc < CS;   // the slot's first use: only the copy is waited for
-        if (!mbar_wait2(fresh ? &full[s] : &empty[rl.s], fresh ? rg.ph : rl.ph, &full[s], rg.ph, abort_flag, a.err,
-                        kDevTimeoutConv, a.wait_cycles)) {
+        if (!mbar_wait2(fresh || kEarlyLoad ? &full[s] : &empty[rl.s], fresh || kEarlyLoad ? rg.ph : rl.ph, &full[s],
+                        rg.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -679,10 +683,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
               v[8 * j + 6] = widen_lo(w[j].w);
               v[8 * j + 7] = widen_hi(w[j].w);
             }
+            if (kEarlyLoad && !fresh) {
+              ok = mbar_wait(&empty[rl.s], rl.ph, abort_flag, a.err, kDevTimeoutConv, a.wait_cycles);
+              __syncwarp();
+              tc_fence_after();
+            }
             tmem_st32(tmem_base + ((uint32_t)(q * 32) << 16) + a.a_col0 + (uint32_t)((c * KPS + h) * 32), v);
           }
           tmem_st_wait();
           tc_fence_before();
+          if (kEarlyLoad && !__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            break;
+          }
           if (tgc) DPTQ_TRACE_CLOCK(tr, 184 + 6 * (gc - 8));
         } else if constexpr (kATmem && KPS == 1) {
           // Warp (lane quarter q, half hs) widens k columns 64 hs .. 64 hs + 63 of rows
@@ -1131,20 +1144,20 @@ static int smem_for(int act_rows, int kps, int stages, int planes, int conv_slot
 //   M = 333, N = 1024 / 4096, K = 4096: 16.1 -> 8.8 / 21.6 -> 14.8 us
 //   M = 512, N = K = 4096: 23.9 -> 15.0 us; M = 2048: 38.1 -> 33.0 us (192, whole)
 //   M = 2048, N = 28672, K = 4096: 163 -> 157 us (192, 17 whole waves)
-// Pairs of CTAs (an even number of weight tiles): stages of 0.484 us (one CTA: 0.515), but a
+// Pairs of CTAs (an even number of weight tiles): stages of 0.475 us (one CTA: 0.515), but a
 // fixed cost higher by the tensor memory and barriers of two CTAs, so that one wave of them loses
 // (M = 700, N = K = 4096: 16.1 -> 16.6 us) and two win (M = 333, N = 12288: 25.2 -> 23.4 us).  The
 // partial sums of a split tile are hidden behind the other tile's stages as far as it has them
 // (M = 2048, N = 4096: split against whole 36.6 / 31.0 us at K = 4096, 73.1 / 82.7 at K = 14336).
 // Against one CTA, GEMM alone: M = 2048, K = 4096, N = 4096 / 12288 / 28672: 32.8 -> 31.0, 68.4 ->
 // 63.0, 157 -> 140 us; N = 4096, K = 14336: 82.4 -> 73.1 us; A8, M = 4096: N = 5120, K = 13824:
-// 369 -> 310 us, N = K = 8192: 312 -> 288 us.
+// 369 -> 310 us, N = K = 8192: 312 -> 288 us (and before the weights were widened early, kEarlyLoad).
 struct TileCost {
   double stage, fixed, split, apart;
 };
 static TileCost tile_cost(int nt, int planes, bool pair, int KI) {
   if (pair) {
-    const double stage = planes == 1 ? 0.484 : 0.40;
+    const double stage = planes == 1 ? 0.475 : 0.40;
     const double split = 14.0 - 0.3 * stage * KI;
     return TileCost{stage, planes == 1 ? 8.3 : 8.5, split > 4.0 ? split : 4.0, 11.0};
   }
