@@ -72,3 +72,26 @@ def test_policy_ties_tiny_and_infinite_values(dp, orc, d, bits):
     assert np.isinf(jr[3].item()) and np.isnan(snr[3].item())
     assert np.allclose(snr[:3].cpu().numpy(), before[:3].cpu().numpy(), rtol=1e-12, equal_nan=True)
     dp.dptq_last_device_error()
+
+
+# tokens of more than 4096 values: batches of 32 tokens that span layers, ragged last batches and
+# widths, one token
+@pytest.mark.parametrize("L,T,d", [(1, 1, 4100), (7, 5, 5120), (3, 700, 5120), (40, 33, 8192), (5, 9, 12292)])
+def test_policy_of_wide_tokens(dp, L, T, d):
+    g = torch.Generator(device="cuda").manual_seed(d + T)
+    x = torch.randn((L, T, d), generator=g, device="cuda")
+    dx = torch.randn((L, T, d), generator=g, device="cuda") * 0.3
+    jr, snr = torch.empty(L, dtype=torch.float64, device="cuda"), torch.empty(L, dtype=torch.float64, device="cuda")
+    bits = torch.empty(L, dtype=torch.uint8, device="cuda")
+    dp.dptq_sensitivity_policy(x, dx, 4, 1e-6, 0.1, 20.0, jr, snr, bits)
+    dp.dptq_last_device_error()
+    xs, ds = x.double(), dx.double()
+    u = x + dx
+    s = u.abs().amax(-1, keepdim=True) / 7
+    err = (s.double() * torch.clamp(torch.round(u / s), -8, 7).double() - ds - xs).pow(2).sum(-1)
+    nx = xs.pow(2).sum(-1)
+    # A thread sums up to d / 256 + 4 squares in fp32 (each step and the error's own roundings
+    # within 2^-24), the rest is fp64: relative 2 (d / 256 + 8) 2^-24, twice over in a ratio.
+    rel = 4 * (d / 256 + 8) * 2.0 ** -24
+    torch.testing.assert_close(jr, (ds.pow(2).sum(-1).sqrt() / (nx.sqrt() + 1e-6)).mean(1), rtol=rel, atol=0)
+    torch.testing.assert_close(snr, (10 * torch.log10(nx / (err + 1e-6))).mean(1), rtol=0, atol=10 * rel)
