@@ -226,7 +226,7 @@ def kernel_source_sha():
     """sha256/16 of the sources the timed kernel is compiled from."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("qgemm.cu", "rotate_row.cuh", "dptq_device.cuh"):
+    for f in ("qgemm.cu", "rotate_mma.cuh", "rotate_row.cuh", "dptq_device.cuh"):
         try:
             h.update(open(os.path.join(ROOT, "paper_2606_12487_gb300", "csrc", f), "rb").read())
         except OSError:

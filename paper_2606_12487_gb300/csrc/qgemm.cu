@@ -20,7 +20,7 @@
 // Operand roles (swap-AB): A (MMA M = 128) = weight rows, B (MMA N = NT) = tokens.
 // D[n][m] lives in TMEM with lane = output channel and column = token.
 //
-// Warp roles of the persistent CTA (one per SM):
+// Warp roles of the persistent CTA (one per SM; wide tiles: pairs of them, PAIR below):
 //   warp 0      weight producer: bulk copies (TMA engine) of packed weight tiles into a
 //               `stages`-deep ring (a stage holds KPS k-blocks of 128), from the start
 //   warp 1      TMEM allocator + single-thread tcgen05.mma issuer

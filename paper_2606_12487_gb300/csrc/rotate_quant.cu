@@ -32,12 +32,12 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // blockIdx.x / csize, + gridDim.x / csize, ...  A warp holds its unit's pairs in registers from
 // the exchange to the codes; the next row's loads are issued before the exchange.
 //
-// Bound by the issue of its own arithmetic (36 warp instructions per 32 elements, half of
-// the slots used: 14 to 16 warps of 128 registers an SM wait for one another once per row),
-// not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
-// 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 60.1 us; K = 4096,
-// B = 2048: 33.0 -> 20.1 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 628 us; M = 64,
-// same row: 33.8 -> 7.3 us.
+// Bound by the latency of its own chain of steps (34 warp instructions per 32 elements, just
+// under half of the issue slots used: 14 to 16 warps of 128 registers an SM wait for one another
+// once per row), not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
+// 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 60.5 us; K = 4096,
+// B = 2048: 33.0 -> 18.1 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 583 us; M = 64,
+// same row: 33.8 -> 7.2 us.
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
   extern __shared__ __align__(128) uint8_t rm_smem[];
