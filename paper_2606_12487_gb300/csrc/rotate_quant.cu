@@ -47,6 +47,9 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
   __shared__ uint32_t l1s[16];
   __shared__ uint32_t lead[2];       // [row parity]: largest |y| so far, nearly (odd log2 blocks)
   __shared__ uint32_t slow_rows[kBatch / 32];
+  // A store into another CTA of the cluster needs that CTA to have started: every thread
+  // arrives here, and waits while the first row's copies are on their way.
+  if (csize > 1) cluster_arrive();
   pdl_launch_dependents();
   pdl_wait();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -103,6 +106,8 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
   for (int row0 = (int)blockIdx.x / csize; row0 < a.rows_out; row0 += kBatch * ncl) {
     bool any_slow = false;
     if (row0 < a.rows_in) unit_prefetch(a.x + (size_t)row0 * K, u.e0, u.load_end, lane, stg);
+    // (the first batch: a cluster has at least one row, and its CTAs the same rows)
+    if (csize > 1 && row0 == (int)blockIdx.x / csize) cluster_wait();
 #pragma unroll 1
     for (int it = 0; it < kBatch; ++it, par ^= 1) {
       const int row = row0 + it * ncl;

@@ -23,9 +23,9 @@ def dp():
 
 # one short unit; exactly one unit; a tail after it; a unit that holds whole blocks and
 # part of the next; two- and four-warp blocks with and without tails; 17, 20 and 28 units
-# (two CTAs a row)
+# (two CTAs a row), 33 with a tail, 40 and 48 (three: their first maxima meet right after the launch)
 FORMS = [(32, 32), (160, 32), (1024, 1024), (1056, 1024), (2080, 64), (3072, 2048), (4096, 4096), (6144, 4096),
-         (5888, 512), (17408, 1024), (20480, 2048), (28672, 4096)]
+         (5888, 512), (17408, 1024), (20480, 2048), (28672, 4096), (33280, 1024), (40960, 4096), (49152, 256)]
 
 
 def rows_of_every_kind(K):
