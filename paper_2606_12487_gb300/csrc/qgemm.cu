@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
   uint64_t* pfull = xbar + 1;    // pairs, in the first CTA: the second is ready for the MMAs of slot s
   uint32_t* tmem_base_sh = reinterpret_cast<uint32_t*>(pfull + kMaxStages);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_sh + 1);
-  volatile int* flags = reinterpret_cast<volatile int*>(tmem_base_sh + 2);   // epilogue: 2 units x 2
+  volatile int* flags = reinterpret_cast<volatile int*>(tmem_base_sh + 2);   // epilogue: 2 split units x 2
   float* sa_sh = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);   // token scales (NT <= 64)
   __half* xpose = reinterpret_cast<__half*>(reinterpret_cast<uint8_t*>(bars) + 1024);  // 4 x [4 tokens][32 ch]
   uint32_t* rot_sh = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + 768);   // fused: 32 words
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
       return ok;
     };
     int sa_mt = -1;   // token tile whose activation scales sit in sa_sh
-    int u = 0;
+    int u = 0, nsplit = 0;   // units, split units
     while (epi_ok && iter.next(un)) {
       const int b = a.nbuf == 2 ? (u & 1) : 0;
       const uint32_t tpar = (a.nbuf == 2 ? (u >> 1) : u) & 1;
@@ -835,10 +835,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_kernel(const GemmArgs a
         sa_mt = mt;
       }
       // Split tile: whether every other contributor is already in is asked while the MMAs
-      // still run, and once more after them if not.
-      volatile int* const flag = flags + 2 * (u & 1);   // [0]: all others in, [1]: last
+      // still run, and once more after them if not.  The two answer slots alternate over the
+      // split units (not all units: a whole tile has no epilogue barrier when NT > 64), so a
+      // slot is written again only after the barrier of the split unit in between, by which
+      // every warp has read it.
+      volatile int* const flag = flags + 2 * (nsplit & 1);   // [0]: all others in, [1]: last
       const bool split = un.slot >= 0 && !ksplit;
       if (split) {
+        ++nsplit;
         if (etid == 0) *flag = ld_acquire_gpu(a.counters + un.slot) == (uint32_t)(un.contributors - 1);
         if (!epi_sync()) break;
       }

@@ -3,6 +3,8 @@ dimensions: accumulators equal the integer product, outputs its scaled rounding.
 import numpy as np
 import pytest
 
+from test_launch_plan_cpu import units
+
 from paper_2606_12487_gb300 import inputs
 
 torch = pytest.importorskip("torch")
@@ -25,6 +27,25 @@ def dp():
                                    (700, 1024, 384)])
 @pytest.mark.parametrize("bits", [4, 8])
 def test_accumulators_on_every_plan(dp, M, N, K, bits):
+    check_accumulators(dp, M, N, K, bits, 2)
+
+
+# a split tile, a whole one and a split one in one CTA's share (single CTAs and pairs): the
+# epilogue warps meet only in the split ones
+@pytest.mark.parametrize("M,N,K,bits", [(193, 11904, 11008, 4), (129, 22016, 4096, 8), (200, 20480, 8192, 4),
+                                        (333, 12176, 8192, 8)])
+def test_split_tiles_with_whole_ones_between(dp, M, N, K, bits):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    p = dp.dptq_launch_plan(M, N, K, bits, sms)
+    share = {}
+    for c, _, _, _, slot, _ in units(p):
+        share.setdefault(c, []).append(slot >= 0)
+    if sms == 152:
+        assert p["nt"] > 64 and any(s[i:i + 3] == [True, False, True] for s in share.values() for i in range(len(s)))
+    check_accumulators(dp, M, N, K, bits, 20)
+
+
+def check_accumulators(dp, M, N, K, bits, passes):
     layer = dp.dptq_pack_weights(torch.from_numpy(inputs.weights(N, K, layer=5)).cuda(), 128)
     wq, sw = dp.dptq_get_packed(layer)
     w = np.empty((N, K), dtype=np.int8)
@@ -40,7 +61,7 @@ def test_accumulators_on_every_plan(dp, M, N, K, bits):
     ref = (c.double() @ torch.from_numpy(w).cuda().double().t())   # whole numbers below 2^53: exact
     sad, swd = torch.from_numpy(sa).cuda(), torch.from_numpy(sw).cuda()
     want = ((ref.float() * sad[:, None]) * swd[None, :]).half()
-    for _ in range(2):   # split-tile sums are left clean
+    for _ in range(passes):   # split-tile sums are left clean
         out = torch.empty((M, N), dtype=torch.float16, device="cuda")
         acc = torch.empty((M, N), dtype=torch.int32, device="cuda")
         dp.dptq_qgemm_codes(layer, packed.contiguous(), sad, bits, out, acc)
