@@ -131,10 +131,10 @@ dptq_status dptq_rotate_act_rh(const void* x_fp16, int M, int K, int had_block, 
  * fp32 (IEEE division), c = clamp(round-half-even(x / s), -8, 7) (never -8), an
  * all-zero group has s = 0 and codes 0.
  * codes (device, written): uint8 [rows][cols/2] in the A4 format of
- * dptq_rotate_quant_act (low nibble = even column); scales (device, written): float
- * [rows][cols / group].  group: a multiple of 128 up to 1024 that divides cols (the
+ * dptq_rotate_quant_act (low nibble = even column), at any even address; scales (device,
+ * written): float [rows][cols / group].  group: a multiple of 128 up to 1024 that divides cols (the
  * paper's 128).  Asynchronous.  INVALID_ARG for null pointers, negative sizes or a
- * misaligned kv_fp16; UNSUPPORTED for other group sizes.  rows == 0 is a no-op. */
+ * misaligned kv_fp16 or codes; UNSUPPORTED for other group sizes.  rows == 0 is a no-op. */
 dptq_status dptq_kv4_quantize(const void* kv_fp16, int rows, int cols, int group, void* codes, float* scales,
                               void* stream);
 

@@ -706,6 +706,8 @@ dptq_status dptq_kv4_quantize(const void* kv_fp16, int rows, int cols, int group
   if (rows == 0) return DPTQ_OK;
   if (!kv_fp16 || !codes || !scales) return fail(DPTQ_ERR_INVALID_ARG, "null pointer");
   if (!aligned16(kv_fp16)) return fail(DPTQ_ERR_INVALID_ARG, "kv must be 16-byte aligned");
+  if ((reinterpret_cast<uintptr_t>(codes) & 1u) != 0)   // (the narrowest stores are 16 bits wide)
+    return fail(DPTQ_ERR_INVALID_ARG, "codes must be 2-byte aligned");
   if (group % 128 != 0 || group > 1024 || cols % group != 0)
     return fail(DPTQ_ERR_UNSUPPORTED, "group must be a multiple of 128 up to 1024 that divides cols");
   int dev;

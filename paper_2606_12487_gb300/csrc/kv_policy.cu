@@ -69,6 +69,9 @@ __device__ __forceinline__ float kv4_sum4(const float* q) {   // four codes in t
   return __fadd_rn(t, kRoundMagic + 34952.f);   // 34952 = 8 * 0x1111
 }
 
+// ALIGNED4: codes start 4-byte aligned and a lane stores its word at once; otherwise (2-byte
+// aligned) as two halves.
+template <bool ALIGNED4>
 __global__ void __launch_bounds__(kKvWarps * 32) kv4_quantize_g128_kernel(const KvArgs a) {
   const int lane = threadIdx.x & 31;
   const int sub = lane & 7, quad = lane >> 3;   // lane within the group, group of the four
@@ -127,7 +130,15 @@ __global__ void __launch_bounds__(kKvWarps * 32) kv4_quantize_g128_kernel(const 
           t1 = kv4_sum4(q + 4);
         }
         const uint32_t word = __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x5410) ^ 0x88888888u;
-        if (g < ngroups) reinterpret_cast<uint32_t*>(a.codes + (size_t)g * 64)[8 * j + sub] = word;
+        if (g < ngroups) {
+          uint8_t* dst = a.codes + (size_t)g * 64 + 4 * (8 * j + sub);
+          if constexpr (ALIGNED4) {
+            *reinterpret_cast<uint32_t*>(dst) = word;
+          } else {
+            reinterpret_cast<uint16_t*>(dst)[0] = (uint16_t)word;
+            reinterpret_cast<uint16_t*>(dst)[1] = (uint16_t)(word >> 16);
+          }
+        }
       }
     }
   }
@@ -185,9 +196,10 @@ cudaError_t launch_kv4(const KvArgs& a, int num_sms, cudaStream_t s) {
   const long long work = a.group == 128 ? (ngroups + 4 * kKvSets - 1) / (4 * kKvSets) : ngroups;   // warps' items
   long long blocks = (work + kKvWarps - 1) / kKvWarps;
   int per_sm = 8;
+  const auto g128 = (reinterpret_cast<uintptr_t>(a.codes) & 3u) == 0 ? kv4_quantize_g128_kernel<true>
+                                                                      : kv4_quantize_g128_kernel<false>;
   if (a.group == 128) {   // one wave of resident CTAs
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kv4_quantize_g128_kernel,
-                                                                        kKvWarps * 32, 0);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g128, kKvWarps * 32, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
   }
@@ -195,7 +207,7 @@ cudaError_t launch_kv4(const KvArgs& a, int num_sms, cudaStream_t s) {
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   if (a.group == 128)
-    kv4_quantize_g128_kernel<<<(unsigned)blocks, kKvWarps * 32, 0, s>>>(a);
+    g128<<<(unsigned)blocks, kKvWarps * 32, 0, s>>>(a);
   else
     kv4_quantize_kernel<<<(unsigned)blocks, kKvWarps * 32, 0, s>>>(a);
   return cudaGetLastError();

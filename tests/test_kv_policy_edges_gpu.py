@@ -45,6 +45,29 @@ def test_kv4_ties_and_non_finite_values(dp, orc, rows, cols):
     assert np.array_equal(c[-1, 128:], c_ref[-1, 128:]) and np.array_equal(c[:-1], c_ref[:-1])
 
 
+@pytest.mark.parametrize("offset", [2, 4, 6, 8])
+@pytest.mark.parametrize("cols,group", [(640, 128), (512, 256)])
+def test_kv4_codes_at_any_even_address(dp, offset, cols, group):
+    rows = 9
+    x = np.random.default_rng(offset).standard_normal((rows, cols)).astype(np.float16)
+    x[2, 3] = np.nan
+    want = torch.empty((rows, cols // 2), dtype=torch.uint8, device="cuda")
+    buf = torch.full((rows * cols // 2 + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    codes = buf[offset:offset + want.numel()].view(rows, cols // 2)
+    sc = torch.empty((rows, cols // group), dtype=torch.float32, device="cuda")
+    kv = torch.from_numpy(x).cuda()
+    dp.dptq_kv4_quantize(kv, group, want, sc)
+    dp.dptq_kv4_quantize(kv, group, codes, sc)
+    assert torch.equal(codes, want) and torch.all(buf[:offset] == 0xA5) and torch.all(buf[offset + want.numel():] == 0xA5)
+
+
+def test_kv4_codes_at_an_odd_address_are_refused(dp):
+    buf = torch.empty((128,), dtype=torch.uint8, device="cuda")
+    kv, sc = torch.zeros((1, 128), dtype=torch.float16, device="cuda"), torch.empty((1, 1), device="cuda")
+    with pytest.raises(dp.DptqError):
+        dp.dptq_kv4_quantize(kv, 128, buf[1:65].view(1, 64), sc)
+
+
 @pytest.mark.parametrize("d", [4, 1028, 4096])
 @pytest.mark.parametrize("bits", [4, 8])
 def test_policy_ties_tiny_and_infinite_values(dp, orc, d, bits):
