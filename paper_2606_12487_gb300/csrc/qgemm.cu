@@ -1418,12 +1418,13 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
   } else if (args.cl > 1) {
     cudaLaunchAttribute* c = &attr[n];
     // All CTAs have to be resident at once (a fused launch's wait for one another's rows).
-    // Asked once per kernel and device, for the largest shared memory.
-    static std::atomic<int> most[64];   // resident clusters + 1 (0: not asked yet)
+    // Asked once per kernel, cluster size and device, for the largest shared memory.
+    static std::atomic<int> most[2][64];   // [four or two][device]: resident clusters + 1 (0: not asked yet)
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int m = dev < 64 ? most[dev].load() : 1;
+    std::atomic<int>* const known = dev < 64 ? &most[args.cl == 4 ? 1 : 0][dev] : nullptr;
+    int m = known != nullptr ? known->load() : 1;
     if (m == 0) {
       cudaLaunchConfig_t probe = cfg;
       probe.dynamicSmemBytes = kSmemLimit;
@@ -1432,7 +1433,7 @@ static cudaError_t launch_nt(const GemmPlan& plan, cudaStream_t s, bool pdl) {
       probe.numAttrs = 1;
       e = cudaOccupancyMaxActiveClusters(&m, qgemm_kernel<NT, KPS, RG, PAIR>, &probe);
       if (e != cudaSuccess) return e;
-      most[dev].store(++m);
+      known->store(++m);
     }
     if ((m - 1) * args.cl >= plan.grid)
       ++n;
