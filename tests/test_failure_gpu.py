@@ -114,6 +114,34 @@ def test_injected_allocation_failure_reports_oom(fail_at, expect):
     assert out == expect, out
 
 
+RESERVE_CHILD = """
+    import torch
+    from paper_2606_12487_gb300 import dptq
+    M, N, K = 256, 256, 384
+    dptq.dptq_reserve(M, K, 0)
+    have = dptq.dptq_scratch_buffers()
+    layer = dptq.dptq_pack_weights(torch.randn((N, K), device="cuda").half(), 128)
+    x, out = torch.randn((M, K), device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        dptq.dptq_qlinear(layer, x, 8, out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert dptq.dptq_scratch_buffers() == have, "the call grew the reserved scratch"
+    again = torch.empty_like(out)
+    dptq.dptq_qlinear(layer, x, 8, again)
+    assert torch.equal(out, again)
+    dptq.dptq_last_device_error()
+"""
+
+
+def test_reserve_covers_a_captured_call_of_its_size():
+    """K = 384: an odd number of 128-element blocks, which layers pad to an even one."""
+    r = subprocess.run([sys.executable, "-c", textwrap.dedent(RESERVE_CHILD)], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
 TIMEOUT_CHILD = """
 import torch
 from paper_2606_12487_gb300 import dptq, inputs
