@@ -764,7 +764,7 @@ dptq_status dptq_plan_info(int M, int N, int K, int bits, int num_sms, int fused
   const dptq_status st = check_plan_args(M, N, K, bits, num_sms, info, info_len, DPTQ_PLAN_INFO_LEN);
   if (st != DPTQ_OK) return st;
   GemmPlan plan{};
-  if (!plan_gemm(M, N, round_up(K, kKBlock), bits, num_sms, plan, fused != 0))
+  if (!plan_gemm(M, N, round_up(K, kKPad), bits, num_sms, plan, fused != 0))
     return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
   write_plan(plan, info, DPTQ_PLAN_INFO_LEN);
   return DPTQ_OK;
@@ -775,7 +775,7 @@ dptq_status dptq_launch_plan(int M, int N, int K, int bits, int num_sms, int row
   if (st != DPTQ_OK) return st;
   if (row_ctas < 0) return fail(DPTQ_ERR_INVALID_ARG, "row_ctas must be >= 0");
   GemmPlan plan{};
-  if (!plan_launch(M, N, round_up(K, kKBlock), bits, num_sms, plan, row_ctas))
+  if (!plan_launch(M, N, round_up(K, kKPad), bits, num_sms, plan, row_ctas))
     return fail(DPTQ_ERR_UNSUPPORTED, "no GEMM plan for this shape");
   write_plan(plan, info, DPTQ_LAUNCH_PLAN_LEN);
   return DPTQ_OK;

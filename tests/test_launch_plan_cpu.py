@@ -59,7 +59,7 @@ def test_every_stage_once(N, K, bits, fused):
         tiles = p["n_wtiles"] * p["m_tiles"] // p["pair"]
         assert p["grid"] % p["pair"] == 0 and p["n_wtiles"] % p["pair"] == 0 and (p["pair"] == 1 or p["nt"] == 192)
         assert p["m_tiles"] * p["nt"] >= M and p["m_tiles"] * p["nt"] <= p["M_pad"]
-        assert p["smem_bytes"] <= 232448 and p["grid"] <= 152 and p["kps"] * p["KI"] == -(-K // 128)
+        assert p["smem_bytes"] <= 232448 and p["grid"] <= 152 and p["kps"] * p["KI"] == -(-K // 256) * 2
         parts = {}
         for c, t, i0, i1, slot, n in units(p):
             parts.setdefault(t, []).append((i0, i1, slot, n))

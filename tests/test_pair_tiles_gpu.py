@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 
 
 # whole waves and split tiles, one tile of tokens and many, a ragged last weight tile and token
-# tile, an odd number of weight tiles (no pairs) and of k-blocks (one-block stages)
+# tile, an odd number of weight tiles (no pairs), K padded from 1152 to 1280
 @pytest.mark.parametrize("M,N,K,pair", [(192, 38912, 4096, 2), (1000, 38912, 512, 2), (577, 12176, 4096, 2),
                                         (577, 12272, 2048, 2), (2048, 4096, 14336, 2), (1025, 12176, 1152, 2),
                                         (2048, 11904, 1024, 1)])

@@ -34,7 +34,7 @@ def _check_plan(p, M, N, K, bits, sms):
     # token padding and tiling
     assert p["M_pad"] % nt == 0 and M <= p["M_pad"] < M + nt
     assert p["m_tiles"] == p["M_pad"] // nt and p["n_wtiles"] == -(-N // 128)
-    kb = -(-K // 128)
+    kb = -(-K // 256) * 2   # layers pad K to 256, so that a stage may hold two blocks of 128
     assert kb % kps == 0 and p["KI"] == kb // kps
     # tensor memory: accumulators (and the weight slots when they live there) fit
     acc = p["nbuf"] * nt * p["segs"]
@@ -58,15 +58,11 @@ def test_split_plans_fit_and_cover(N, K, M, bits, sms):
     _check_plan(p, M, N, K, bits, sms)
     assert p["fused"] == 0
     # tile shapes the kernels are built for
-    even_kb = (-(-K // 128)) % 2 == 0
     if M <= 64:
-        # two-block stages with the weights in tensor memory, unless K has an odd number
-        # of k-blocks
-        assert nt_expected_decode(M) == p["nt"]
-        assert p["kps"] == (2 if even_kb else 1) and p["a_tmem"] == (1 if even_kb else 0)
+        # two-block stages with the weights in tensor memory
+        assert nt_expected_decode(M) == p["nt"] and p["kps"] == 2 and p["a_tmem"] == 1
     elif bits == 4 and M > 128:
-        assert p["nt"] == 192 and p["a_tmem"] == 1
-        assert p["kps"] == (2 if even_kb else 1)
+        assert p["nt"] == 192 and p["a_tmem"] == 1 and p["kps"] == 2
     elif bits == 8 and M > 128:
         # two 24 KB activation planes per k-block: one k-block per stage, at least 4 stages
         assert p["nt"] == 192 and p["a_tmem"] == 1 and p["kps"] == 1 and p["stages"] >= 4
@@ -82,11 +78,6 @@ def nt_expected_decode(M):
 @pytest.mark.parametrize("M", [1, 8, 16, 32, 33, 64])
 @pytest.mark.parametrize("bits", [4, 8])
 def test_fused_decode_plans(N, K, M, bits):
-    if (-(-K // 128)) % 2:
-        # the fused kernel needs two-block stages; dptq_qlinear then takes two launches
-        with pytest.raises(dptq.DptqError):
-            dptq.dptq_plan_info(M, N, K, bits, 152, fused=True)
-        return
     split = dptq.dptq_plan_info(M, N, K, bits, 152)
     M_pad = split["M_pad"]
     tiles = split["n_wtiles"] * split["m_tiles"]

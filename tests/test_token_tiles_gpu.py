@@ -21,7 +21,7 @@ def dp():
 
 
 # 64-token tiles whole, split, and with one k-block more than a stage; 192-token tiles whole in
-# waves and split; an odd number of k-blocks (no 64-token plan)
+# waves and split; K padded from 384 to 512
 @pytest.mark.parametrize("M,N,K", [(65, 48, 512), (100, 1024, 4096), (129, 272, 768), (200, 4096, 1024),
                                    (333, 12288, 512), (449, 2064, 2048), (1000, 4096, 2048), (2048, 4096, 512),
                                    (700, 1024, 384)])
