@@ -1224,7 +1224,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   int stages = kMaxStages;
   while (stages > 2 && smem_total(stages) > kSmemLimit) --stages;
   if (smem_total(stages) > kSmemLimit) return false;
-  if (fused && stages * kps * (planes * nt * 128 + kWTileBytes) < 8 * kUnitBytes) return false;
+  if (fused && stages * kps * (planes * nt * 128 + kWTileBytes) < 8 * (kUnitBytes + kOffBytes)) return false;
   // The converters learn that a widened slot is free from the `empty` barrier of the
   // stage that last read it, CS stages back; with CS <= stages that barrier cannot
   // complete a further phase before they look.

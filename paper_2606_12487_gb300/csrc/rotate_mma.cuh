@@ -6,12 +6,15 @@
 // A sum of such halves with signs is exact in fp32 while it stays below 2^24 of its unit:
 //   hi: the block's sum of |x| is below 2^(24 + u) = 2^(25 - l + k)      (k is chosen so);
 //   lo: 2^l 2^(u - 1) = 2^k is at most 2^24 units of 2^(k - 24), and every x is a multiple
-//       of 2^(k - 24): always true for k = 0 (binary16 is a multiple of 2^-24), tested
-//       for k > 0.
+//       of 2^(k - 24): always true for k = 0 (binary16 is a multiple of 2^-24).
 // So each Hadamard sum is an exact fp32 pair, and fl(hi + lo), one addition, is the
-// correctly rounded fp32 of the sum.  Rows that fail the test (a sum of |x| of 2^(25 - l) or
-// more next to values below 2^(k - 14), infinities, NaN) are rotated in 64-bit integers
-// (rotate_slow_row).
+// correctly rounded fp32 of the sum.
+// For k > 0 (a block's sum of |x| of 2^(25 - l) or more) the few values below 2^(k - 14) that
+// are finer than 2^(k - 24) are rounded to it first, and what that takes off (at most
+// 2^(k - 25), a multiple of 2^-24) goes into a list of the unit: every sum of the block is then
+// corrected by plus or minus each entry (unit_to_grid, unit_add_off; N(0, 3^2) in blocks of
+// 4096 has one entry in 14 blocks).  Rows with a longer list, a sum of 2^22 or more,
+// infinities or NaN are rotated in 64-bit integers (rotate_slow_row).
 //
 // Work split.  A warp takes a unit of 1024 consecutive elements, 32 a thread; 1, 2 or 4 warps
 // share a block (G).  Element i of a unit, bits i9..i0:
@@ -40,7 +43,9 @@ namespace dptq {
 
 constexpr int kUnit = 1024;            // elements of one warp
 constexpr int kUnitBytes = kUnit * 8;  // its (hi, lo) pairs in the exchange
-constexpr int kStageBytes = kUnit * 2;  // its halves, waiting for their turn
+constexpr int kOffMax = 63;             // entries of its list (unit_to_grid)
+constexpr int kOffBytes = 4 * (1 + kOffMax);
+constexpr int kStageBytes = kUnit * 2 + kOffBytes;  // its halves, waiting for their turn, and its list
 constexpr uint32_t kRowSlow = 0x7FFFFFFFu;   // in place of a maximum: the row leaves the pair form
 
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
@@ -182,10 +187,10 @@ __device__ __forceinline__ void unit_prefetch(const __half* row, int e0, int end
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// An upper bound of the unit's sum of |x| in units of 1/4, at least 2^22 when the sum is
-// not known to be below 2^20 (also for infinities and NaN).  Eight binary16 additions in a
+// An upper bound of the unit's sum of |x| in units of 1/4, at least 2^24 when the sum is
+// not known to be below 2^22 (also for infinities and NaN).  Eight binary16 additions in a
 // row lose at most 7 2^-11 of their sum; the factor 1 + 2^-7 covers that and the fp32 steps.
-constexpr uint32_t kL1Slow = 1u << 22;
+constexpr uint32_t kL1Slow = 1u << 24;   // (in all 128 lanes of a group: 2^31)
 template <class Run>
 __device__ __forceinline__ uint32_t unit_l1(Run run) {
   __half2 s[2];
@@ -209,22 +214,50 @@ __device__ __forceinline__ int split_k(uint32_t l1q, int l) {
   const int k = lg - (27 - l);
   return k > 0 ? k : 0;
 }
-// Whether every value is a multiple of 2^(k - 24) (k >= 1).
-template <class Run>
-__device__ __forceinline__ bool unit_on_grid(Run run, int k) {
+// The unit's halves (in shared memory, [run][lane], each lane its own) rounded to multiples of
+// 2^(k - 24) (k >= 1), what that took off, with the signs, into the unit's list: the count, then
+// n 2^12 + i for n 2^-24 off element i of the group (|n| <= 2^(k - 1)).  A count above kOffMax: the
+// list is too short.  A function of its own, in a small loop: few rows come here, and inlined it
+// slowed the others down (2048 rows of K = 4096: 17.5 instead of 16.4 us).  Against a second
+// pass over such rows in 64-bit integers, B = 4096, 4 bits: a fused launch of 32 tokens of
+// N(0, 2.5^2), N = 4096, 25.8 -> 11.7 us (N(0, 1): 9.3 us); 2048 rows of K = 4096, N(0, 3^2),
+// 95 -> 21 us, N(0, 1) with one value of 30000 in each, 166 -> 27 us (N(0, 1): 16 us).
+static __device__ __noinline__ void unit_to_grid(uint8_t* halves, uint32_t* list, const int8_t* signs, int e0, int load_end,
+                                                 int k, int wg, int lane) {
   const __half2 c = __half2half2(__ushort_as_half((unsigned short)((k - 14 + 15) << 10)));   // 2^(k - 14)
-  bool ok = true;
-#pragma unroll
+  int count = 0;
+#pragma unroll 1
   for (int j = 0; j < 4; ++j) {
-    const uint4 v = run(j);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint4* const run = reinterpret_cast<uint4*>(halves + 512 * j + 16 * lane);
+    const uint4 v = *run;
+    uint32_t w[4] = {v.x, v.y, v.z, v.w}, d[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const __half2 m = __hmin2(__habs2(as_half2(w[i])), c);
-      ok = ok && as_u32(__hsub2_rn(__hadd2_rn(m, c), c)) == as_u32(m);
+      d[i] = as_u32(__hsub2_rn(m, __hsub2_rn(__hadd2_rn(m, c), c)));   // exact; 0 for |x| >= c
     }
+    if (!__any_sync(0xffffffffu, ((d[0] | d[1] | d[2] | d[3]) & 0x7FFF7FFFu) != 0u)) continue;
+    uint4 sv = v;
+    const int o = e0 + unit_lane_offset(lane) + 64 * j;
+    if (signs != nullptr && o < load_end) run_signs(signs, o, sv);
+    const uint32_t sw[4] = {sv.x, sv.y, sv.z, sv.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      w[i] = as_u32(__hsub2_rn(as_half2(w[i]), as_half2(d[i] ^ (w[i] & 0x80008000u))));   // exact
+      const float2 t = __half22float2(as_half2(d[i] ^ (sw[i] & 0x80008000u)));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float e = h ? t.y : t.x;
+        const uint32_t has = __ballot_sync(0xffffffffu, e != 0.f);
+        const int at = count + __popc(has & ((1u << lane) - 1u));
+        if (e != 0.f && at < kOffMax)
+          list[1 + at] = (uint32_t)((int)(e * 16777216.f) * 4096 + wg * kUnit + o - e0 + 2 * i + h);
+        count += __popc(has);
+      }
+    }
+    *run = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  return ok;
+  if (lane == 0) list[0] = (uint32_t)count;
 }
 
 // Split, MMAs and the butterflies of bits 0 .. 7, then the unit's pairs into the exchange
@@ -329,6 +362,71 @@ __device__ __forceinline__ void unit_phase2(const uint8_t* xg, int t, int l, uin
         if (!(x & (RL::R << bit))) f2_bfly(v[x], v[x + (RL::R << bit)]);
     }
   }
+}
+
+// The lists of the group's units (`stride` bytes apart) added to the thread's sums: an entry t at
+// element i is +-t in the sums j of its block, minus for an odd number of common bits of i and j.
+// |S| < 2^22, so with the pair first made (f, S - f), f = fl(S), |S - f| <= 1/8, the second part
+// takes all corrections (multiples of 2^-24, below 1/2 together) exactly.
+template <int G>
+__device__ __forceinline__ void unit_add_off(const uint8_t* lists, int stride, int t, int l, uint64_t (&v)[32]) {
+  using RL = RunLayout<G>;
+#pragma unroll
+  for (int x = 0; x < 32; ++x) {
+    float h, o;
+    f2_unpack(v[x], h, o);
+    const float f = __fadd_rn(h, o), bv = __fsub_rn(f, h);   // two-sum: the remainder is exact
+    v[x] = f2_pack(f, __fadd_rn(__fsub_rn(h, __fsub_rn(f, bv)), __fsub_rn(o, bv)));
+  }
+  // Value x is element j = low | 256 (x / R) + x % R (bits apart): its five bits of j one by one.
+  const uint32_t low = (uint32_t)RL::low(t);
+  constexpr uint32_t kBits[5] = {0xAAAAAAAAu, 0xCCCCCCCCu, 0xF0F0F0F0u, 0xFF00FF00u, 0xFFFF0000u};   // bit x: bit b of x
+#pragma unroll 1
+  for (int g = 0; g < G; ++g) {
+    const uint32_t* const list = reinterpret_cast<const uint32_t*>(lists + g * stride);
+    const int n = (int)list[0];
+#pragma unroll 1
+    for (int e = 1; e <= n; ++e) {
+      const uint32_t i = list[e] & 4095u;
+      const float d = (float)((int)list[e] >> 12) * 0x1p-24f;
+      uint32_t odd = 0u - (__popc(i & low & ((1u << l) - 1u)) & 1u);   // bit x: minus
+      uint32_t in = (((i ^ low) & RL::low(32 * G - 1)) >> l) == 0u ? ~0u : 0u;   // bit x: i and j in one block
+#pragma unroll
+      for (int b = 0; b < 5; ++b) {
+        const int jb = (1 << b) < RL::R ? b : 8 + b - (RL::R == 8 ? 3 : RL::R == 4 ? 2 : 1);
+        const uint32_t set = (i >> jb) & 1u ? kBits[b] : 0u;
+        if (jb < l)
+          odd ^= set;
+        else
+          in &= (i >> jb) & 1u ? kBits[b] : ~kBits[b];
+      }
+      if (in == 0u) continue;
+      const uint32_t db = __float_as_uint(d);
+#pragma unroll
+      for (int x = 0; x < 32; ++x) {
+        float f, rem;
+        f2_unpack(v[x], f, rem);
+        if (in & (1u << x)) rem = __fadd_rn(rem, __uint_as_float(db ^ ((odd << (31 - x)) & 0x80000000u)));
+        v[x] = f2_pack(f, rem);
+      }
+    }
+  }
+}
+
+// The same out of line, on sums that wait in the thread's own places of the exchange (`buf`: its
+// first 16 bytes; 512 bytes from pair to pair).
+template <int G>
+__device__ __noinline__ void unit_add_off_at(const uint8_t* lists, int stride, int t, int l, ulonglong2* buf) {
+  uint64_t v[32];
+#pragma unroll
+  for (int x = 0; x < 32; x += 2) {
+    const ulonglong2 w = buf[16 * x];
+    v[x] = w.x;
+    v[x + 1] = w.y;
+  }
+  unit_add_off<G>(lists, stride, t, l, v);
+#pragma unroll
+  for (int x = 0; x < 32; x += 2) buf[16 * x] = make_ulonglong2(v[x], v[x + 1]);
 }
 
 // Largest |fl(S)| of the warp's values, as fp32 bits; part[g]: the lane's over values 8 g .. 8 g + 7.
@@ -637,14 +735,16 @@ struct UnitGeom {
   }
 };
 
-// From the lane's halves (raw(j): run j, signs(j, v): the signs applied to it) to the
-// thread's exact sums; false when the unit's block leaves the pair form (v is then
-// meaningless).  l1s: a word per warp of the group; group_sync: its barrier; after_split():
-// called when the halves are no longer needed (the next row's loads).
-template <int G, class Raw, class Signs, class GroupSync, class After>
-__device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, Signs signs, const uint32_t (&am)[4], int lane,
-                                          uint8_t* xu, uint32_t* l1s, GroupSync group_sync, After after_split,
-                                          uint64_t (&v)[32]) {
+// From the lane's halves (raw(j): run j, signs(j, v): the signs applied to it, to_grid(k):
+// unit_to_grid for them) to the thread's exact sums; false when the unit's block leaves the pair
+// form (v is then meaningless).  l1s: a word per warp of the group; off: the unit's list, the
+// group's OFF bytes apart; group_sync: the group's barrier; after_split(): called when the
+// halves are no longer needed (the next row's loads).  ONCE: the code runs once a launch, and what
+// few rows need stays out of its way (the fused launch, M = 16, N = 512, K = 256: 7.57 -> 7.29 us).
+template <int G, int OFF, bool ONCE, class Raw, class ToGrid, class Signs, class GroupSync, class After>
+__device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, ToGrid to_grid, Signs signs, const uint32_t (&am)[4],
+                                          int lane, uint8_t* xu, uint32_t* l1s, uint8_t* off, GroupSync group_sync,
+                                          After after_split, uint64_t (&v)[32]) {
   constexpr int full_l = G == 1 ? 10 : G == 2 ? 11 : 12;
   uint32_t l1 = unit_l1(raw);
   if constexpr (G > 1) {
@@ -655,8 +755,8 @@ __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, Signs s
     for (int i = 0; i < G; ++i) l1 += l1s[i];
   }
   bool ok = l1 < kL1Slow;
-  const int k = ok ? split_k(l1, u.l) : 0;
-  if (k > 0) ok = __all_sync(0xffffffffu, unit_on_grid(raw, k));
+  const int k = ok ? split_k(l1, u.l) : 0;   // (the same in the whole group)
+  if (__builtin_expect(k > 0, 0)) to_grid(k);
   auto run = [&](int j) {
     uint4 x = raw(j);
     signs(j, x);
@@ -673,6 +773,31 @@ __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, Signs s
     unit_phase2<G, true>(xg, u.tg, u.l, v);
   else
     unit_phase2<G, false>(xg, u.tg, u.l, v);
+  if (__builtin_expect(k > 0, 0)) {
+    const uint8_t* const lists = off - u.wg * OFF;
+    uint32_t most = 0;   // entries of the group's longest list: every warp of it goes the same way
+#pragma unroll
+    for (int g = 0; g < G; ++g) most = max(most, *reinterpret_cast<const uint32_t*>(lists + g * OFF));
+    if (most > (uint32_t)kOffMax) {
+      ok = false;
+    } else if (most > 0u) {
+      if constexpr (ONCE) {
+        group_sync();   // the group has read the exchange
+        ulonglong2* const buf = reinterpret_cast<ulonglong2*>(xu) + lane;
+#pragma unroll
+        for (int x = 0; x < 32; x += 2) buf[16 * x] = make_ulonglong2(v[x], v[x + 1]);
+        unit_add_off_at<G>(lists, OFF, u.tg, u.l, buf);
+#pragma unroll
+        for (int x = 0; x < 32; x += 2) {
+          const ulonglong2 w = buf[16 * x];
+          v[x] = w.x;
+          v[x + 1] = w.y;
+        }
+      } else {
+        unit_add_off<G>(lists, OFF, u.tg, u.l, v);
+      }
+    }
+  }
   return ok;
 }
 
@@ -783,11 +908,24 @@ __device__ __forceinline__ void fused_rotate_rows(const RQArgs& a, int item, int
     unit_load(a.x + (size_t)row * a.K, u.e0, u.load_end, lane, w);
     mma_hadamard_a(u.l, lane, am);
     const int o = u.e0 + unit_lane_offset(lane);
-    const bool ok = unit_sums<G>(u, [&](int j) { return w[j]; },
+    const bool ok = unit_sums<G, kOffBytes, true>(
+                                 u, [&](int j) { return w[j]; },
+                                 [&](int k) {   // by way of the exchange, not yet in use
+                                   uint8_t* const xu = smem + wc * kUnitBytes;
+                                   uint4* const at = reinterpret_cast<uint4*>(xu) + lane;
+#pragma unroll
+                                   for (int j = 0; j < 4; ++j) at[32 * j] = w[j];
+                                   unit_to_grid(xu, reinterpret_cast<uint32_t*>(smem + 8 * kUnitBytes + wc * kOffBytes),
+                                                a.signs, u.e0, u.load_end, k, u.wg, lane);
+#pragma unroll
+                                   for (int j = 0; j < 4; ++j) w[j] = at[32 * j];
+                                   __syncwarp();
+                                 },
                                  [&](int j, uint4& x) {
                                    if (a.signs != nullptr && o + 64 * j < u.load_end) run_signs(a.signs, o + 64 * j, x);
                                  },
                                  am, lane, smem + wc * kUnitBytes, l1s + wc - u.wg,
+                                 smem + 8 * kUnitBytes + wc * kOffBytes,
                                  [&] {
                                    if constexpr (G == 1)
                                      __syncwarp();

@@ -35,9 +35,9 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // Bound by the latency of its own chain of steps (34 warp instructions per 32 elements, just
 // under half of the issue slots used: 14 to 16 warps of 128 registers an SM wait for one another
 // once per row), not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
-// 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 60.5 us; K = 4096,
-// B = 2048: 33.0 -> 18.1 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 583 us; M = 64,
-// same row: 33.8 -> 7.2 us.
+// 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 57.0 us; K = 4096,
+// B = 2048: 33.0 -> 17.2 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 570 us; M = 64,
+// same row, 4 bits: 33.8 -> 7.6 us.
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
   extern __shared__ __align__(128) uint8_t rm_smem[];
@@ -123,13 +123,16 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");   // the lane's own copies
       uint64_t v[32];
-      const bool ok = unit_sums<G>(
+      const bool ok = unit_sums<G, kStageBytes, false>(
           u, [&](int j) { return *reinterpret_cast<const uint4*>(stg + 512 * j + 16 * lane); },
+          [&](int k) {
+            unit_to_grid(stg, reinterpret_cast<uint32_t*>(stg + kUnit * 2), a.signs, u.e0, u.load_end, k, u.wg, lane);
+          },
           [&](int j, uint4& x) {
             const int o = u.e0 + unit_lane_offset(lane) + 64 * j;
             if (a.signs != nullptr && o < u.load_end) run_signs(a.signs, o, x);
           },
-          am, lane, xu, l1s + warp - u.wg, group_sync,
+          am, lane, xu, l1s + warp - u.wg, stg + kUnit * 2, group_sync,
           [&] {
             if (it + 1 < kBatch && row + ncl < a.rows_in)
               unit_prefetch(a.x + (size_t)(row + ncl) * K, u.e0, u.load_end, lane, stg);
@@ -197,7 +200,7 @@ cudaError_t launch_rotate_mma_g(const RQArgs& a, cudaStream_t s, bool pdl) {
   const int units = unit_map(a.K, a.tail, G).units;
   const int csize = ceil_div(units, 16);
   const int W = round_up(ceil_div(units, csize), G);
-  // The exchange, or (64-bit integers) a block of 1024 G values; the coming row.
+  // The exchange, or (64-bit integers) a block of 1024 G values; the coming row and the lists.
   const int smem = W * (kUnitBytes + kStageBytes);
   int sms = 0;
   cudaError_t e = device_sms(&sms);

@@ -1,6 +1,6 @@
 """The tensor-core rotation at the edges of its forms: units of 1024 elements, blocks over
 1, 2 and 4 warps, tails in units of their own, rows over a cluster of CTAs, and rows whose
-values leave the fp32-pair form and are rotated in 64-bit integers."""
+values leave the plain fp32-pair form."""
 import numpy as np
 import pytest
 
@@ -33,8 +33,8 @@ def rows_of_every_kind(K):
     n = rng.standard_normal((7, K)).astype(np.float32)
     n[1] *= 1e-4                                   # near binary16's smallest values
     n[2] = 40.0 * rng.integers(-100, 101, K)       # large sums on a coarse grid: pairs with k > 0
-    n[3, :3] = 60000.0                             # large sums and fine values: 64-bit integers
-    n[4] = 65504.0                                 # the largest sum
+    n[3, :3] = 60000.0                             # large sums and fine values: pairs with a list
+    n[4] = 65504.0                                 # the largest sum: 64-bit integers
     n[5] = 0.0
     n[6, K // 2:] = 0.0                            # zero units
     return inputs.to_f16(n)

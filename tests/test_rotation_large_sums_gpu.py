@@ -1,0 +1,138 @@
+"""Rows whose sums of |x| go beyond what one pair of grids holds: the few finer values are listed
+and corrected for, longer lists and larger sums go through 64-bit integers.  Same values either
+way, and no kind of row makes a call much slower than another."""
+import numpy as np
+import pytest
+
+import parity
+from paper_2606_12487_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_12487_gb300 import dptq
+    dptq.load()
+    return dptq
+
+
+def rows_of_large_sums(K):
+    rng = np.random.default_rng(K + 1)
+    n = rng.standard_normal((12, K))
+    n[0] *= 3.0
+    n[1] *= 40.0
+    n[2] *= 500.0
+    n[3, K // 3] = 30000.0
+    n[4, [0, K // 5, K // 2, K - 1]] = (30000.0, -60000.0, 65504.0, 9000.0)
+    n[5] *= 0.01
+    n[5, K // 7] = 40000.0                              # many values below the grid
+    n[6] *= 0.01
+    n[6, rng.choice(K, K // 8, replace=False)] = 900.0   # lists too long: 64-bit integers
+    n[7] *= 9000.0                                      # sums above 2^22 in every full block
+    n[8] = np.where(rng.random(K) < 0.5, 60000.0, 2.0 ** -24)
+    n[9] *= np.exp2(rng.integers(-20, 12, K))
+    n[10] *= 10.0
+    n[10, ::3] = 0.0
+    return inputs.to_f16(n.astype(np.float32))
+
+
+# one, two and four warps a block, several blocks in a unit, tails (in groups of their own), rows over two
+# and three CTAs
+@pytest.mark.parametrize("K,B", [(256, 256), (1024, 1024), (1056, 1024), (2048, 64), (3072, 2048), (4096, 4096), (6144, 4096),
+                                 (14336, 2048), (20480, 4096), (34816, 2048)])
+def test_values_match_the_oracle(dp, orc, K, B):
+    x = rows_of_large_sums(K)
+    M = x.shape[0]
+    signs = np.where(np.random.default_rng(9).random(K) < 0.5, -1, 1).astype(np.int8)
+    xd, sd = torch.from_numpy(x).cuda(), torch.from_numpy(signs).cuda()
+    exact = (B.bit_length() - 1) % 2 == 0 and K % B == 0   # even log2: no irrational factor
+    for sg in (None, signs):
+        y_ref = orc.rotate(x, B, sg)
+        y = torch.empty((M, K), dtype=torch.float32, device="cuda")
+        dp.dptq_rotate_act(xd, B, y) if sg is None else dp.dptq_rotate_act_rh(xd, B, sd, y)
+        parity.check_rotation(y.cpu().numpy(), y_ref)
+        if exact:
+            assert np.array_equal(y.cpu().numpy(), y_ref)
+        c_ref, s_ref = orc.rotate_quant_act(x, B, 8, sg)
+        codes = torch.empty((M, K), dtype=torch.int8, device="cuda")
+        sc = torch.empty((M,), dtype=torch.float32, device="cuda")
+        if sg is None:
+            dp.dptq_rotate_quant_act(xd, B, 8, codes, sc)
+        else:
+            dp.dptq_rotate_quant_act_rh(xd, B, 8, sd, codes, sc)
+        parity.check_scales(sc.cpu().numpy(), s_ref)
+        n = parity.check_codes(codes.cpu().numpy(), c_ref, y_ref, s_ref, 8)
+        if exact:
+            assert n == 0 and np.array_equal(sc.cpu().numpy(), s_ref)
+    dp.dptq_last_device_error()
+
+
+# a row a CTA, half a row, rows side by side; lists and 64-bit rows in one call
+@pytest.mark.parametrize("M,N,K,B", [(31, 4096, 4096, 4096), (16, 4096, 2048, 2048), (12, 8192, 11008, 256),
+                                     (12, 4096, 16384, 4096), (64, 640, 1024, 1024)])
+@pytest.mark.parametrize("bits", [4, 8])
+def test_one_launch_equals_two(dp, M, N, K, B, bits):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    units = K // 1024
+    row_ctas = 2 * M if units > 8 else M
+    if (M, N) == (64, 640):
+        row_ctas = -(-M // (8 // units))
+    assert dp.dptq_launch_plan(M, N, K, bits, sms, row_ctas)["fused"] == 1
+    base = rows_of_large_sums(K)
+    x = torch.from_numpy(np.concatenate([base] * (-(-M // 12)))[:M]).cuda()
+    signs = np.where(np.random.default_rng(2).random(K) < 0.5, -1, 1).astype(np.int8)
+    layer = dp.dptq_pack_weights_rh(torch.from_numpy(inputs.weights(N, K, layer=4)).cuda(), B, signs)
+    one = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    two = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    for _ in range(2):
+        dp.dptq_qlinear(layer, x, bits, one)
+    dp.dptq_qlinear_quantize(layer, x, bits)
+    dp.dptq_qlinear_gemm(layer, M, bits, two)
+    assert torch.equal(one.view(torch.int16), two.view(torch.int16))
+    dp.dptq_last_device_error()
+    layer.close()
+
+
+def seconds(call, passes=100):
+    graph = torch.cuda.CUDAGraph()
+    call()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        for _ in range(passes):
+            call()
+    times = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        graph.replay()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) / passes)
+    return sorted(times)[3]
+
+
+@pytest.mark.parametrize("M,N", [(32, 4096), (2048, 0)])
+def test_time_does_not_depend_on_the_values(dp, M, N):
+    """K = 4096 in one block, values of N(0, 3^2) and one outlier of 30000 against N(0, 1)."""
+    K = 4096
+    g = torch.Generator(device="cuda").manual_seed(3)
+    base = torch.randn((M, K), generator=g, device="cuda")
+    layer = dp.dptq_pack_weights(torch.randn((N, K), generator=g, device="cuda").half(), K) if N else None
+    out = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    codes = torch.empty((M, K // 2), dtype=torch.uint8, device="cuda")
+    sc = torch.empty((M,), dtype=torch.float32, device="cuda")
+
+    def timed(x):
+        x = x.half()
+        return seconds(lambda: dp.dptq_qlinear(layer, x, 4, out) if N else dp.dptq_rotate_quant_act(x, K, 4, codes, sc))
+
+    wide, outlier = 3.0 * base, base.clone()
+    outlier[:, 77] = 30000.0
+    plain = timed(base)
+    limit = 2.0 * plain   # (measured 1.1 to 1.65; in 64-bit integers 2.7 to 9.7)
+    assert timed(wide) < limit and timed(outlier) < limit
+    layer is None or layer.close()

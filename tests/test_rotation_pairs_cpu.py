@@ -1,7 +1,7 @@
 """The split behind the tensor-core rotation, restated in numpy: x = hi + lo with hi a
 multiple of 2^u, u = 1 - l + k, both halves binary16, and every signed sum of the 2^l
 halves of a block exact in fp32 when the block's sum of |x| is below 2^(25 - l + k) and x
-is a multiple of 2^(k - 24)."""
+is a multiple of 2^(k - 24); and for k > 0 the list of what rounding to that grid takes off."""
 import numpy as np
 import pytest
 
@@ -25,15 +25,15 @@ def fwht(v):
     return v
 
 
-# The kernel takes rows whose sum of |x| is below 2^20 this way, so k is at most l - 5.
-@pytest.mark.parametrize("l,k", [(l, k) for l in (0, 1, 4, 5, 6, 7, 8, 10, 11, 12) for k in (0, 1, 4, 7)
-                                 if k <= max(0, l - 5)])
+# The kernel takes rows whose sum of |x| is below 2^22 this way, so k is at most l - 3.
+@pytest.mark.parametrize("l,k", [(l, k) for l in (0, 1, 4, 5, 6, 7, 8, 10, 11, 12) for k in (0, 1, 4, 7, 9)
+                                 if k <= max(0, l - 3)])
 def test_split_sums_are_exact(l, k):
     n = 1 << l
     rng = np.random.default_rng(100 * l + k)
     rows = [rng.standard_normal(n), rng.standard_normal(n) * 1e-4, np.full(n, 1.0), rng.standard_normal(n) * 20]
     rows[1][0] = 300.0
-    top = min(2.0 ** (25 - l + k), 2.0 ** 20)
+    top = min(2.0 ** (25 - l + k), 2.0 ** 22)
     tried = 0
     for row in rows:
         for scale in (1.0, 0.5 * top / max(np.abs(row).sum(), 1e-9), 0.99 * top / max(np.abs(row).sum(), 1e-9)):
@@ -65,6 +65,53 @@ def test_grid_test_of_large_sums():
         m = np.minimum(np.abs(x), c)
         ok = ((m + c).astype(F16) - c).astype(F16) == m
         assert np.array_equal(ok, (x.astype(np.float64) * 2.0 ** (24 - k)) % 1.0 == 0)
+
+
+def to_grid(x, k):
+    """x rounded to multiples of 2^(k - 24) (binary16), and what that took off."""
+    c = F16(2.0 ** (k - 14))
+    m = np.minimum(np.abs(x), c)
+    d = (m - ((m + c).astype(F16) - c).astype(F16)).astype(F16)
+    d = np.where(np.signbit(x), -d, d).astype(F16)
+    return (x - d).astype(F16), d
+
+
+def test_rounding_to_the_grid():
+    """For every finite binary16: on the grid, at most half a step off, and exactly undone by
+    an integer number n of 2^-24, |n| <= 2^(k - 1)."""
+    x = np.arange(0, 0x7C00, dtype=np.uint16).view(F16)
+    x = np.concatenate([x, -x])
+    for k in range(1, 10):
+        g, d = to_grid(x, k)
+        g64, n = g.astype(np.float64), d.astype(np.float64) * 2.0 ** 24
+        assert np.array_equal(g64 + n * 2.0 ** -24, x.astype(np.float64))
+        assert np.all(g64 * 2.0 ** (24 - k) % 1.0 == 0) and np.all(n % 1.0 == 0) and np.all(np.abs(n) <= 2 ** (k - 1))
+
+
+@pytest.mark.parametrize("l,k", [(12, 1), (12, 4), (12, 9), (11, 8), (10, 7), (8, 3)])
+def test_listed_remainders_correct_the_sums_exactly(l, k):
+    n = 1 << l
+    rng = np.random.default_rng(7 * l + k)
+    top = 2.0 ** (25 - l + k)
+    parity = np.array([bin(v).count("1") & 1 for v in range(n)])
+    for share in (0.51, 0.99):
+        x = (rng.standard_normal(n) * (share * top / n / 0.8)).astype(F16)
+        x[rng.choice(n, 40, replace=False)] = (rng.standard_normal(40) * 2.0 ** (k - 16)).astype(F16)   # fine values
+        x[0] = F16(min(65504.0, max(0.0, share * top - np.abs(x[1:].astype(np.float64)).sum())))
+        assert np.abs(x.astype(np.float64)).sum() < top
+        on, d = to_grid(x, k)
+        entries = np.flatnonzero(d)
+        assert 0 < entries.size <= 63
+        hi, lo = split(on, l, k)
+        h, o = fwht(hi.astype(F32)[None])[0], fwht(lo.astype(F32)[None])[0]
+        f = h + o
+        bv = f - h
+        rem = (h - (f - bv)) + (o - bv)
+        for i in entries:
+            rem = rem + np.where(parity[np.arange(n) & i], -d[i], d[i]).astype(F32)
+        assert f.dtype == rem.dtype == F32
+        S = fwht(x.astype(np.float64)[None])[0]
+        assert np.array_equal(f.astype(np.float64) + rem, S) and np.array_equal(f + rem, S.astype(F32))
 
 
 def test_exchange_has_no_bank_conflicts():
