@@ -75,3 +75,24 @@ def unpack_public_a4(packed, K):
     out[:, 0::2] = lo
     out[:, 1::2] = hi
     return out
+
+
+def one_launch_row_ctas(dp, M, N, K, B, bits, sms):
+    """CTAs that rotate the token rows when dptq_qlinear runs as one launch (its own steps: a
+    CTA for up to 8 units of 1024 elements, two CTAs for a longer row, or rows side by side), and
+    the plan of that launch.  Raises if the call takes two launches."""
+    tail = K % B
+    b = B if K > tail else tail
+    G = 1 if b <= 1024 else b // 1024
+    units = -(-(K - tail) // (1024 * G)) * G + (G if tail else 0)
+    cpr = -(-units // 8)
+    wpc = -(-(-(-units // cpr)) // G) * G
+    assert cpr <= 2 and wpc <= 8
+    for items in (M * cpr, -(-M // (8 // wpc)) if cpr == 1 else M * cpr):
+        try:
+            plan = dp.dptq_launch_plan(M, N, K, bits, sms, items)
+        except dp.DptqError:
+            continue
+        assert plan["fused"] == 1
+        return items, plan
+    raise AssertionError(f"M = {M}, N = {N}, K = {K}: two launches")

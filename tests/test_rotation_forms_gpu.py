@@ -99,11 +99,15 @@ def test_operand_planes_hold_the_public_codes(dp, K, B, bits):
 
 # one row a CTA, two CTAs a row, several rows side by side in a CTA (1, 2 and 4 warps each, a
 # last CTA that is not full), whole tiles and clusters of two and four CTAs
-@pytest.mark.parametrize("M,N,K,B", [(16, 512, 256, 256), (13, 128, 1024, 1024), (64, 256, 2048, 2048),
-                                     (33, 128, 4096, 4096), (64, 1024, 4096, 2048), (7, 4096, 11008, 256),
-                                     (32, 6144, 4096, 4096), (21, 8192, 1536, 512)])
+# (`rows` a CTA: 0 for half a row)
+@pytest.mark.parametrize("M,N,K,B,rows", [(16, 512, 256, 256, 8), (13, 128, 1024, 1024, 8), (64, 512, 2048, 2048, 4),
+                                          (33, 640, 4096, 4096, 2), (64, 1024, 4096, 2048, 2), (7, 4096, 11008, 256, 0),
+                                          (32, 6144, 4096, 4096, 1), (21, 8192, 1536, 512, 1), (31, 512, 3072, 1024, 2)])
 @pytest.mark.parametrize("bits", [4, 8])
-def test_one_launch_equals_two(dp, M, N, K, B, bits):
+def test_one_launch_equals_two(dp, M, N, K, B, rows, bits):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    items, _ = parity.one_launch_row_ctas(dp, M, N, K, B, bits, sms)
+    assert items == (-(-M // rows) if rows else 2 * M)
     base = rows_of_every_kind(K)
     x = torch.from_numpy(np.concatenate([base] * (-(-M // 7)))[:M]).to(DEV)
     x[7:] *= torch.linspace(0.2, 1.0, max(1, M - 7), device=DEV)[:max(0, M - 7), None].half()

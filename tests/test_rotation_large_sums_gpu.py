@@ -77,11 +77,7 @@ def test_values_match_the_oracle(dp, orc, K, B):
 @pytest.mark.parametrize("bits", [4, 8])
 def test_one_launch_equals_two(dp, M, N, K, B, bits):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    units = K // 1024
-    row_ctas = 2 * M if units > 8 else M
-    if (M, N) == (64, 640):
-        row_ctas = -(-M // (8 // units))
-    assert dp.dptq_launch_plan(M, N, K, bits, sms, row_ctas)["fused"] == 1
+    parity.one_launch_row_ctas(dp, M, N, K, B, bits, sms)   # (it is one)
     base = rows_of_large_sums(K)
     x = torch.from_numpy(np.concatenate([base] * (-(-M // 12)))[:M]).cuda()
     signs = np.where(np.random.default_rng(2).random(K) < 0.5, -1, 1).astype(np.int8)
