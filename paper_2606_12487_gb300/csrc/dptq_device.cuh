@@ -211,9 +211,11 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
   return r;
 }
 // Arrive on another CTA's mbarrier (an address of cluster_map).  For tensor-memory stores and
-// bulk copies that this thread has already seen complete: a release at cluster scope would wait
-// for more and takes longer than a whole stage (266 instead of 140 us for M = 2048, N = 28672, K
-// = 4096).
+// bulk copies that this thread has already seen complete.  Neither this nor the other CTA's wait
+// is at cluster scope, so the PTX memory model does not by itself promise that they order these
+// for that CTA's MMAs; the completed copies and stores, the tcgen05 fences on both sides and
+// bit-exact results are what it rests on.  A release at cluster scope would wait for more and
+// takes longer than a whole stage (266 instead of 140 us for M = 2048, N = 28672, K = 4096).
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -394,16 +396,6 @@ __device__ __forceinline__ void tmem_st_wait() {
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-// The same wait, tied to the registers of one load, so that no use of them can be
-// scheduled before it (used when another load is issued before these are consumed).
-__device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15])
-               :
-               : "memory");
-}
 
 // ------------------------------------------------------------------ PDL
 // GPU-scope acquire load and acquire-release add (split-tile arrival counters).
@@ -433,10 +425,6 @@ __device__ __forceinline__ void release_add_gpu(uint32_t* p, uint32_t v) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-__device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 }  // namespace dptq

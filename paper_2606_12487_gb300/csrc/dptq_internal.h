@@ -136,7 +136,7 @@ struct GemmArgs {
   // (written to `act` / `sa` by the converter warps of CTAs 0 .. rq_items - 1) and the two grid counters [rows ready, CTAs done] that order it before the GEMM
   // (zero between launches).
   RQArgs rq;
-  int rq_np;           // CTAs the grid holds per token row (2 or 4)
+  int rq_np;           // general one-launch plan: CTAs of the grid per token row (2 or 4; reported only, a row takes rq_cpr)
   int rq_cpr;          // CTAs that share a row's rotation (1 or 2)
   int rq_wpc;          // units of 1024 elements (warps) of a row in each of them, at most 8
   int rq_rpc;          // rows a CTA rotates side by side (rq_cpr = 1; at most 8 / rq_wpc)

@@ -18,32 +18,11 @@
 namespace dptq {
 
 // ------------------------------------------------------------------ KV4
-// One warp per (row, group) at a time.  Lane l holds columns 4l .. 4l + 3 of each
+// Any group size: one warp per (row, group) at a time.  Lane l holds columns 4l .. 4l + 3 of each
 // 128-column block of the group (J = group / 128 blocks, at most 8): one 8-byte load per
 // block, the group's absmax by shuffles, then four codes per block packed into 2 bytes
 // (the warp stores 64 contiguous bytes per block).
 constexpr int kKvWarps = 8;
-
-// Quantize the 4 values of one lane (raw fp16 bits), given the group's absmax, into 4
-// nibbles (low nibble first).
-__device__ __forceinline__ uint32_t kv4_codes(uint2 raw, float s, float r, bool nz) {
-  const __half2 h0 = *reinterpret_cast<const __half2*>(&raw.x);
-  const __half2 h1 = *reinterpret_cast<const __half2*>(&raw.y);
-  const float y[4] = {__low2float(h0), __high2float(h0), __low2float(h1), __high2float(h1)};
-  float c[4] = {0.f, 0.f, 0.f, 0.f};
-  if (nz) quant_code4(y, s, r, -8.f, 7.f, c);
-  uint32_t packed = 0;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) packed |= ((uint32_t)(int)c[e] & 0xFu) << (4 * e);
-  return packed;
-}
-
-__device__ __forceinline__ float absmax4(uint2 raw) {
-  const __half2 h0 = *reinterpret_cast<const __half2*>(&raw.x);
-  const __half2 h1 = *reinterpret_cast<const __half2*>(&raw.y);
-  return fmaxf(fmaxf(fabsf(__low2float(h0)), fabsf(__high2float(h0))),
-               fmaxf(fabsf(__low2float(h1)), fabsf(__high2float(h1))));
-}
 
 // Groups of 128 (the paper's size): eight lanes a group, 16 values a lane in two runs of
 // eight (16-byte loads, 128 contiguous bytes per eight lanes), four groups a warp at a time,

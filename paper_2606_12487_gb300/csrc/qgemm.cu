@@ -1183,7 +1183,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   // A8 192-token tiles take one k-block per stage: a stage holds two 24 KB activation
   // planes, so two-block stages would leave room for only two of them.
   if (nt == 192 && planes == 2) kps = 1;
-  if (KB % kps != 0) kps = 1;
+  // (Layers pad K to two k-blocks: KB is even.)
   // Largest |code| * |weight| sum per stage, and the stages one fp32 accumulator can
   // take before the exact-integer bound 2^24 could be crossed.
   auto seg_plan = [&](int kps_, int& seg_iters, int& segs) {
@@ -1198,7 +1198,7 @@ static bool plan_tiles(int M, int N, int K_pad, int bits, int num_sms, GemmPlan&
   while (nt > 16 && nt * segs > 512) {
     nt = nt == 192 ? 128 : nt >> 1;
     const int k2 = (nt == 192 && planes == 2) ? 1 : kps_for(nt);
-    if (k2 != kps && KB % k2 == 0) {
+    if (k2 != kps) {
       kps = k2;
       seg_plan(kps, seg_iters, segs);
     }
@@ -1371,7 +1371,7 @@ bool plan_launch(int M, int N, int K_pad, int bits, int num_sms, GemmPlan& plan,
   GemmPlan pairs;
   if (plan.nt == 192 && plan_tiles(M, N, K_pad, bits, num_sms, pairs, false, 0, 0, 0, true) && pairs.cost < plan.cost)
     plan = pairs;
-  if (K_pad % (2 * kKBlock) != 0 || plan.M_pad % 64 != 0) return true;
+  if (plan.M_pad % 64 != 0) return true;
   // The operand planes keep the rows of the wide tiles (192 and 128 are multiples of 64), so
   // that one quantized matrix serves layers of any N.
   GemmPlan narrow;
@@ -1472,12 +1472,8 @@ cudaError_t launch_gemm(const GemmPlan& plan, cudaStream_t s, bool pdl) {
     }
   }
   switch (plan.nt) {
-    case 16: return launch_nt<16, 1>(plan, s, pdl);
-    case 32: return launch_nt<32, 1>(plan, s, pdl);
-    case 64: return launch_nt<64, 1>(plan, s, pdl);
     case 128: return launch_nt<128, 1>(plan, s, pdl);
     case 192: return plan.args.pair == 2 ? launch_nt<192, 1, 0, true>(plan, s, pdl) : launch_nt<192, 1>(plan, s, pdl);
-    case 256: return launch_nt<256, 1>(plan, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

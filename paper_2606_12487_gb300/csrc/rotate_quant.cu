@@ -15,7 +15,7 @@
 
 namespace dptq {
 
-// Three CTAs per SM (at most 85 registers a thread; the body needs 72 without spilling):
+// Three CTAs per SM (at most 85 registers a thread; the body takes 79 or 80, without spilling):
 // many-row launches (prefill) are bound by the latency of each row's chain of steps, so
 // rows in flight per SM set their throughput.
 template <int MODE>
@@ -37,7 +37,8 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // once per row), not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
 // 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 57.0 us; K = 4096,
 // B = 2048: 33.0 -> 17.2 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 570 us; M = 64,
-// same row, 4 bits: 33.8 -> 7.6 us.
+// same row, 4 bits: 33.8 -> 7.6 us.  At 128 registers nothing spills where it counts (codes, planes with
+// blocks over 2 or 4 warps); planes of shorter blocks spill 24 bytes a thread, the rotated fp32 rows 44 to 64.
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
   extern __shared__ __align__(128) uint8_t rm_smem[];
