@@ -540,7 +540,7 @@ struct RowOut {
   uint8_t* p;          // row base (kRQPublic, kRQY) or the operand planes (kRQAct)
   size_t plane;        // kRQAct, 8 bits: bytes to the second plane
   size_t kb_stride;    // kRQAct: rows_out * 128
-  int row, bits;
+  int row, bits;       // (kRQY: `bits` is 1 if the rows start 16-byte aligned)
   // Address of element k, and from it to element k + 256.
   template <int MODE>
   __device__ __forceinline__ uint8_t* at(int k) const {
@@ -615,9 +615,18 @@ __device__ __forceinline__ void store_codes_at(const RowOut& d, uint8_t* p, cons
         reinterpret_cast<uint32_t*>(p)[1] = word(4);
       }
     }
-  } else {   // kRQY: q holds the rotated values
+  } else {   // kRQY: q holds the rotated values; rows start 16-byte aligned if `bits` says so
+    if (d.bits) {
+      if constexpr (R == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(q[0], q[1]);
+      } else {
 #pragma unroll
-    for (int e = 0; e < R; ++e) reinterpret_cast<float*>(p)[e] = q[e];
+        for (int e = 0; e < R; e += 4) *reinterpret_cast<float4*>(p + 4 * e) = make_float4(q[e], q[e + 1], q[e + 2], q[e + 3]);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < R; ++e) reinterpret_cast<float*>(p)[e] = q[e];
+    }
   }
 }
 
@@ -739,9 +748,10 @@ struct UnitGeom {
 // unit_to_grid for them) to the thread's exact sums; false when the unit's block leaves the pair
 // form (v is then meaningless).  l1s: a word per warp of the group; off: the unit's list, the
 // group's OFF bytes apart; group_sync: the group's barrier; after_split(): called when the
-// halves are no longer needed (the next row's loads).  ONCE: the code runs once a launch, and what
-// few rows need stays out of its way (the fused launch, M = 16, N = 512, K = 256: 7.57 -> 7.29 us).
-template <int G, int OFF, bool ONCE, class Raw, class ToGrid, class Signs, class GroupSync, class After>
+// halves are no longer needed (the next row's loads).  APART: what few rows need is a call, for
+// code that runs once a launch (the fused launch, M = 16, N = 512, K = 256: 7.57 -> 7.29 us) or
+// spills more without (rotated fp32 rows, M = 4000, K = 28672: 271 -> 260 us).
+template <int G, int OFF, bool APART, class Raw, class ToGrid, class Signs, class GroupSync, class After>
 __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, ToGrid to_grid, Signs signs, const uint32_t (&am)[4],
                                           int lane, uint8_t* xu, uint32_t* l1s, uint8_t* off, GroupSync group_sync,
                                           After after_split, uint64_t (&v)[32]) {
@@ -781,7 +791,7 @@ __device__ __forceinline__ bool unit_sums(const UnitGeom<G>& u, Raw raw, ToGrid 
     if (most > (uint32_t)kOffMax) {
       ok = false;
     } else if (most > 0u) {
-      if constexpr (ONCE) {
+      if constexpr (APART) {
         group_sync();   // the group has read the exchange
         ulonglong2* const buf = reinterpret_cast<ulonglong2*>(xu) + lane;
 #pragma unroll

@@ -37,8 +37,8 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // once per row), not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
 // 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 57.0 us; K = 4096,
 // B = 2048: 33.0 -> 17.2 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 570 us; M = 64,
-// same row, 4 bits: 33.8 -> 7.6 us.  At 128 registers nothing spills where it counts (codes, planes with
-// blocks over 2 or 4 warps); planes of shorter blocks spill 24 bytes a thread, the rotated fp32 rows 44 to 64.
+// same row, 4 bits: 33.8 -> 7.6 us.  At 128 registers the codes, and the planes of blocks over 2 or 4
+// warps, spill nothing; planes of shorter blocks spill 16 bytes a thread, rotated fp32 rows 28 to 40.
 template <int MODE, int G>
 __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, const int csize) {
   extern __shared__ __align__(128) uint8_t rm_smem[];
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
   RowOut dst;
   dst.plane = (size_t)a.KB * a.rows_out * 128;
   dst.kb_stride = (size_t)a.rows_out * 128;
-  dst.bits = a.bits;
+  dst.bits = MODE == kRQY ? (int)((reinterpret_cast<uintptr_t>(a.out) & 15u) == 0) : a.bits;
   auto row_out = [&](int r) {
     dst.row = r;
     dst.p = static_cast<uint8_t*>(a.out);
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(512, 1) rotate_mma_kernel(const RQArgs a, cons
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");   // the lane's own copies
       uint64_t v[32];
-      const bool ok = unit_sums<G, kStageBytes, false>(
+      const bool ok = unit_sums<G, kStageBytes, MODE == kRQY || (MODE == kRQAct && G == 1)>(
           u, [&](int j) { return *reinterpret_cast<const uint4*>(stg + 512 * j + 16 * lane); },
           [&](int k) {
             unit_to_grid(stg, reinterpret_cast<uint32_t*>(stg + kUnit * 2), a.signs, u.e0, u.load_end, k, u.wg, lane);

@@ -57,6 +57,9 @@ def test_values_match_the_oracle(dp, orc, K, B):
         parity.check_rotation(y.cpu().numpy(), y_ref)
         if exact:
             assert np.array_equal(y.cpu().numpy(), y_ref)
+        off = torch.empty((M * K + 1,), dtype=torch.float32, device="cuda")[1:].view(M, K)   # 4-byte aligned only
+        dp.dptq_rotate_act(xd, B, off) if sg is None else dp.dptq_rotate_act_rh(xd, B, sd, off)
+        assert torch.equal(off, y)
         c_ref, s_ref = orc.rotate_quant_act(x, B, 8, sg)
         codes = torch.empty((M, K), dtype=torch.int8, device="cuda")
         sc = torch.empty((M,), dtype=torch.float32, device="cuda")
