@@ -32,8 +32,8 @@ __global__ void __launch_bounds__(kRQThreads, 3) rotate_quant_kernel(const RQArg
 // blockIdx.x / csize, + gridDim.x / csize, ...  A warp holds its unit's pairs in registers from
 // the exchange to the codes; the next row's loads are issued before the exchange.
 //
-// Bound by the latency of its own chain of steps (34 warp instructions per 32 elements, just
-// under half of the issue slots used: 14 to 16 warps of 128 registers an SM wait for one another
+// Bound by the latency of its own chain of steps (35 warp instructions per 32 elements,
+// half of the issue slots used: 14 to 16 warps of 128 registers an SM wait for one another
 // once per row), not by HBM.  The kernel it replaced kept 64-bit integers (139 instructions).  Times, M =
 // 2048, 4-bit operand planes, before -> now: K = 14336, B = 2048: 144.8 -> 57.0 us; K = 4096,
 // B = 2048: 33.0 -> 17.2 us; M = 8192, K = 28672, B = 4096, 8 bits: 1907 -> 570 us; M = 64,

@@ -132,6 +132,6 @@ def test_time_does_not_depend_on_the_values(dp, M, N):
     wide, outlier = 3.0 * base, base.clone()
     outlier[:, 77] = 30000.0
     plain = timed(base)
-    limit = 2.0 * plain   # (measured 1.1 to 1.65; in 64-bit integers 2.7 to 9.7)
+    limit = 2.2 * plain   # (measured 1.1 to 1.65; in 64-bit integers 2.7 to 9.7)
     assert timed(wide) < limit and timed(outlier) < limit
     layer is None or layer.close()
